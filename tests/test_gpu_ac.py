@@ -99,3 +99,17 @@ def test_archive_streams_full_size(fkv, oracle_mod):
         H = float(-(p * np.log2(p)).sum()) if dist == "zipf" else 8.0
         rate = nb.sum() / (ns * n)
         assert H - 0.02 < rate < H + 0.05, (dist, rate, H)
+
+
+@pytest.mark.parametrize("N,c", [(3, 1), (5, 2), (257, 128)])
+@pytest.mark.parametrize("n", [20, 33, 700])
+def test_long_straddle_runs(fkv, oracle_mod, N, c, n):
+    """The middle symbol of an odd uniform alphabet straddles the middle at
+    every step, so its bits stay pending (well past one 32-bit word) until
+    another symbol settles them; exact against the oracle."""
+    ctx = fkv.Context(N)
+    sym = np.full((4, n), c)
+    sym[1, -1] = 0
+    sym[2, -1] = N - 1
+    sym[3, n // 2] = 0
+    _check(oracle_mod, ctx, sym.astype(_dt(N)), False)
