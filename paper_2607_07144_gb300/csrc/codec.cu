@@ -183,25 +183,6 @@ struct FastDiv {
     }
 };
 
-// Decode span s of `stream` (one per thread): the walk's symbols go through
-// `put(j, c)`, j = 0 .. m-1 from the span's last symbol back to its first,
-// straight from registers to their place; a point whose walk does not end at
-// the anchor sets the corrupt status.
-template <class Put>
-__device__ __forceinline__ void decode_span(const fkvdec::Tables &t, const double2 *__restrict__ pts, int64_t n,
-                                            int64_t pt_stride, int64_t stream, int64_t s,
-                                            const fkv_decconst *__restrict__ dc, int L, unsigned *status, Put put,
-                                            int &m)
-{
-    m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
-    const double2 p = pts[stream * pt_stride + s];
-    long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-    fkvdec::walk(t, X, Y, m, put);
-    const long long lim = __ldg(&dc->alim[m]);
-    if (X > lim || X < -lim || Y > lim || Y < -lim)
-        atomicOr(status, FKV_ST_CORRUPT);
-}
-
 // Persistent: a block loads the decoder tables once and walks chunks of
 // dec_threads spans (chunk = stream * bps + span block), blockIdx.x,
 // + gridDim.x, ...; each thread stores its span's symbols directly, so the
@@ -217,14 +198,25 @@ k_span_decode(const double2 *__restrict__ pts, int64_t n, int64_t pt_stride, int
     __syncthreads();
     constexpr int TPB = dec_threads<Sym>();
     ChunkWalk w(bps);
-    for (int64_t ck = blockIdx.x; ck < n_chunks; ck += gridDim.x, w.next()) {
+    auto point = [&](const ChunkWalk &c, bool more) {     // this thread's point of a chunk, loaded a chunk ahead
+        const int64_t s = c.sb * TPB + threadIdx.x;
+        return more && s < spans ? __ldg(&pts[c.stream * pt_stride + s]) : make_double2(0.0, 0.0);
+    };
+    double2 p = point(w, blockIdx.x < n_chunks);
+    for (int64_t ck = blockIdx.x; ck < n_chunks; ck += gridDim.x) {
         const int64_t s = w.sb * TPB + threadIdx.x;
-        if (s >= spans)
-            continue;
         Sym *dst = sym + w.stream * sym_stride + s * L;
-        int m = 0;
-        decode_span(t, pts, n, pt_stride, w.stream, s, dc, L, status,
-                    [&](int j, int c) { dst[m - 1 - j] = static_cast<Sym>(c); }, m);
+        w.next();
+        const double2 pn = point(w, ck + gridDim.x < n_chunks);
+        if (s < spans) {
+            const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
+            dst += m - 1;
+            if (!fkvdec::decode_point(t, p, m, __ldg(&dc->alim[m]), [&] {
+                    return [=](int j, int c) { dst[-j] = static_cast<Sym>(c); };
+                }))
+                atomicOr(status, FKV_ST_CORRUPT);
+        }
+        p = pn;
     }
 }
 
@@ -239,12 +231,10 @@ __device__ __forceinline__ void decode_chunk(const fkvdec::Tables &t, const doub
     const int64_t s = s0 + threadIdx.x;
     if (s < spans) {
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
-        const double2 p = pts[stream * pt_stride + s];
-        long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-        Sym *my = sbuf + threadIdx.x * L;
-        fkvdec::walk(t, X, Y, m, [&](int j, int c) { my[m - 1 - j] = static_cast<Sym>(c); });
-        const long long lim = __ldg(&dc->alim[m]);
-        if (X > lim || X < -lim || Y > lim || Y < -lim)
+        Sym *my = sbuf + threadIdx.x * L + m - 1;
+        if (!fkvdec::decode_point(t, pts[stream * pt_stride + s], m, __ldg(&dc->alim[m]), [&] {
+                return [=](int j, int c) { my[-j] = static_cast<Sym>(c); };
+            }))
             atomicOr(status, FKV_ST_CORRUPT);
     }
 }
@@ -314,30 +304,36 @@ k_span_decode_planar(const double2 *__restrict__ pts, unsigned n_rec, int64_t pt
     __syncthreads();
     const long long lim_full = __ldg(&dc->alim[L]);
     ChunkWalk w(bps);
-    for (unsigned ck = blockIdx.x; ck < n_chunks; ck += gridDim.x, w.next()) {
+    auto point = [&](const ChunkWalk &c, bool more) {     // this thread's point of a chunk, loaded a chunk ahead
+        const unsigned s = static_cast<unsigned>(c.sb) * TPB + threadIdx.x;
+        return more && s < spans ? __ldg(&pts[c.stream * pt_stride + s]) : make_double2(0.0, 0.0);
+    };
+    double2 p = point(w, blockIdx.x < n_chunks);
+    for (unsigned ck = blockIdx.x; ck < n_chunks; ck += gridDim.x) {
         const unsigned s = static_cast<unsigned>(w.sb) * TPB + threadIdx.x;
-        if (s >= spans)
-            continue;
-        const unsigned first = s * static_cast<unsigned>(L);
-        const int m = n - first < static_cast<unsigned>(L) ? static_cast<int>(n - first) : L;
-        const unsigned q = first + m - 1;             // the span's last symbol
-        unsigned rec = div_r.div(q);
-        int o = static_cast<int>(q - rec * static_cast<unsigned>(R));
         Sym *base = out + w.stream * static_cast<int64_t>(n);
-        const double2 p = pts[w.stream * pt_stride + s];
-        long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-        fkvdec::walk(t, X, Y, m, [&](int, int c) {
-            const unsigned S = o < nk ? SK : SV;
-            base[poff[o] + rec * S] = static_cast<Sym>(c);
-            if (o == 0) {
-                o = R;
-                --rec;
-            }
-            --o;
-        });
-        const long long lim = m == L ? lim_full : __ldg(&dc->alim[m]);
-        if (X > lim || X < -lim || Y > lim || Y < -lim)
-            atomicOr(status, FKV_ST_CORRUPT);
+        w.next();
+        const double2 pn = point(w, ck + gridDim.x < n_chunks);
+        if (s < spans) {
+            const unsigned first = s * static_cast<unsigned>(L);
+            const int m = n - first < static_cast<unsigned>(L) ? static_cast<int>(n - first) : L;
+            const unsigned q = first + m - 1;             // the span's last symbol
+            const unsigned rec = div_r.div(q);
+            const int o = static_cast<int>(q - rec * static_cast<unsigned>(R));
+            if (!fkvdec::decode_point(t, p, m, m == L ? lim_full : __ldg(&dc->alim[m]), [&] {
+                    return [=, o = o, rec = rec](int, int c) mutable {
+                        const unsigned S = o < nk ? SK : SV;
+                        base[poff[o] + rec * S] = static_cast<Sym>(c);
+                        if (o == 0) {
+                            o = R;
+                            --rec;
+                        }
+                        --o;
+                    };
+                }))
+                atomicOr(status, FKV_ST_CORRUPT);
+        }
+        p = pn;
     }
 }
 
@@ -605,12 +601,10 @@ k_span_decode_ragged(const double2 *__restrict__ pts, const int64_t *__restrict_
         if (s < 0 || s * L >= n)
             continue;
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
-        const double2 p = pts[g];
-        long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-        Sym *dst = sym + __ldg(&so[i]) + s * L;
-        fkvdec::walk(t, X, Y, m, [&](int j, int c) { dst[m - 1 - j] = static_cast<Sym>(c); });
-        const long long lim = __ldg(&dc->alim[m]);
-        if (X > lim || X < -lim || Y > lim || Y < -lim)
+        Sym *dst = sym + __ldg(&so[i]) + s * L + m - 1;
+        if (!fkvdec::decode_point(t, pts[g], m, __ldg(&dc->alim[m]), [&] {
+                return [=](int j, int c) { dst[-j] = static_cast<Sym>(c); };
+            }))
             atomicOr(status, FKV_ST_CORRUPT);
     }
 }

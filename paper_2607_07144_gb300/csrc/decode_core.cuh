@@ -32,11 +32,10 @@
 //   * N > 8: Voronoi regions of the vertices are angular sectors, so the fp32
 //     angle picks the sector; within twice the angle's error bound of a
 //     boundary (the bound: 1.2e-5 rad for the arctangent polynomial plus
-//     1.5e-6 rad for the fp32 direction, division and reflections, plus
-//     N 2^-24 sector widths for the scaling) the two neighbouring sectors are
-//     decided by the sign of Q . (V(a) - V(b)); the record reads take the
-//     angle from atan2f instead (a shorter dependency chain) with a band of
-//     1e-3 sector widths.
+//     1.5e-6 rad for the fp32 direction, division and reflections, plus 5e-7
+//     rad for the coefficients rounded in sector widths, plus N 2^-24 sector
+//     widths for the scaling) the two neighbouring sectors are decided by the
+//     sign of Q . (V(a) - V(b)).
 #pragma once
 
 #include <climits>
@@ -47,8 +46,8 @@ namespace fkvdec {
 
 // atan u ~ u (a1 + a3 u^2 + a5 u^4 + a7 u^6 + a9 u^8) on [0, 1], from
 // fit_atan.py: float32 Horner evaluation within 1.18e-5 rad of atan
-__device__ constexpr float kAtan[5] = {9.998637438e-01f, -3.302824795e-01f, 1.800999194e-01f, -8.509350568e-02f,
-                                       2.082198113e-02f};
+constexpr float kAtan[5] = {9.998637438e-01f, -3.302824795e-01f, 1.800999194e-01f, -8.509350568e-02f,
+                            2.082198113e-02f};
 
 struct Tables {
     const longlong2 *T;   // [L][N] (x, y), shared memory
@@ -57,6 +56,8 @@ struct Tables {
     const float2 *vf;     // [N] V(c) as float, shared memory
     int N;
     float sect_thr;       // sector test: |fraction| below this is decided in fp32
+    float sect_a[5];      // kAtan in sector widths (times N / 2 pi)
+    int sect_sh;          // floor(2^16 log2(1/r)): the scale of a walk's step
 };
 
 // Shared-memory footprint of the tables for (N, L).
@@ -80,7 +81,11 @@ __device__ inline Tables load(const fkv_decconst *__restrict__ g, const longlong
         vy[i] = g->vy[i];
         vf[i] = make_float2(g->vfx[i], g->vfy[i]);
     }
-    return Tables{T, vx, vy, vf, N, g->sect_thr};
+    Tables t{T, vx, vy, vf, N, g->sect_thr, {}, g->sect_sh};
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+        t.sect_a[i] = g->sect_a[i];
+    return t;
 }
 
 // Q . V(c) in units of 2^-60: the high words of the two 128-bit products
@@ -121,11 +126,43 @@ __device__ __forceinline__ void direction(long long X, long long Y, float &qx, f
     qy = __int2float_rn(static_cast<int>(static_cast<unsigned>(ys >> 32)));
 }
 
-// kShortChain: the sector angle from the library's atan2f, whose dependency
-// chain is shorter than the polynomial's (record reads, where one walk per
-// lane is the whole latency); otherwise from the polynomial, which issues
-// fewer instructions (bulk decoders, many walks in flight).
-template <bool kShortChain = false>
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The sector of direction (qx, qy), integers that image (X, Y): octant
+// reduction to u in [0, 1], atan u in sector widths from the odd polynomial of
+// fit_atan.py, the octant's reflections, and rounding by adding 1.5 2^23.
+__device__ __forceinline__ int classify_sector(const Tables &t, long long X, long long Y, float qx, float qy)
+{
+    const int N = t.N;
+    const float ax = fabsf(qx), ay = fabsf(qy);
+    // integers: no range or subnormal cases, and 0 / 1 at the origin
+    const float u = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), 1.0f));
+    const float u2 = u * u;
+    float a = u * fmaf(fmaf(fmaf(fmaf(t.sect_a[4], u2, t.sect_a[3]), u2, t.sect_a[2]), u2, t.sect_a[1]), u2,
+                       t.sect_a[0]);
+    if (ay > ax)
+        a = 0.25f * static_cast<float>(N) - a;
+    if (qx < 0.0f)
+        a = 0.5f * static_cast<float>(N) - a;
+    a = copysignf(a, qy);                      // in [-N/2, N/2]
+    const float big = a + 12582912.0f;
+    const float f = a - (big - 12582912.0f);   // in [-0.5, 0.5]
+    int c = __float_as_int(big) - 0x4B400000;
+    c += c < 0 ? N : 0;
+    // away from a sector boundary by more than the angle's error allows
+    if (fabsf(f) < t.sect_thr)
+        return c;
+    // else the nearer of the two sectors by exact products
+    const int c1 = f > 0.0f ? (c + 1 < N ? c + 1 : 0) : (c > 0 ? c - 1 : N - 1);
+    const long long d = exact_dot(t, X, Y, c) - exact_dot(t, X, Y, c1);
+    return d > 0 ? c : (d < 0 ? c1 : min(c, c1));
+}
+
 __device__ __forceinline__ int classify(const Tables &t, long long X, long long Y)
 {
     const int N = t.N;
@@ -154,97 +191,107 @@ __device__ __forceinline__ int classify(const Tables &t, long long X, long long 
             return bi;
         return classify_exact_all(t, X, Y);
     }
-    float ph, thr;
-    if constexpr (kShortChain) {
-        // atan2f is within a few ulp: 1e-3 sector widths covers it at any N
-        ph = atan2f(qy, qx);
-        thr = 0.499f;
-    } else {
-        // the angle of (qx, qy): octant reduction to u in [0, 1], atan u
-        // from the odd polynomial of fit_atan.py (error below 1.2e-5 rad),
-        // then the octant's reflections, giving an angle in [-pi, pi]
-        const float ax = fabsf(qx), ay = fabsf(qy);
-        const float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
-        const float u = mx > 0.0f ? __fdividef(mn, mx) : 0.0f;
-        const float u2 = u * u;
-        ph = u * fmaf(fmaf(fmaf(fmaf(kAtan[4], u2, kAtan[3]), u2, kAtan[2]), u2, kAtan[1]), u2, kAtan[0]);
-        if (ay > ax)
-            ph = 1.57079637f - ph;
-        if (qx < 0.0f)
-            ph = 3.14159274f - ph;
-        if (qy < 0.0f)
-            ph = -ph;
-        thr = t.sect_thr;
-    }
-    const float a = ph * (static_cast<float>(N) * 0.159154937f);
-    const float ar = rintf(a);
-    const float f = a - ar;                        // in [-0.5, 0.5]
-    int c0 = static_cast<int>(ar);
-    if (c0 < 0)
-        c0 += N;
-    if (c0 >= N)
-        c0 -= N;
-    // away from a sector boundary by more than the angle's error allows
-    if (fabsf(f) < thr)
-        return c0;
-    int c1 = f > 0.0f ? c0 + 1 : c0 - 1;           // the neighbour across the near boundary
-    if (c1 < 0)
-        c1 += N;
-    if (c1 >= N)
-        c1 -= N;
-    const long long d = exact_dot(t, X, Y, c0) - exact_dot(t, X, Y, c1);
-    if (d > 0)
-        return c0;
-    if (d < 0)
-        return c1;
-    return c0 < c1 ? c0 : c1;
+    return classify_sector(t, X, Y, qx, qy);
 }
 
-// round(v * 2^62) to nearest, ties to even, saturated to int64 (NaN gives
-// INT64_MIN), from the binary64 fields with integer ops: v = m 2^(e - 1075),
-// so v 2^62 = m 2^(e - 1013), a left shift or a rounded right shift of m.
+// round(v * 2^62) to nearest, saturated to int64 (NaN gives INT64_MIN), from
+// the binary64 fields with integer ops: v = m 2^(e - 1075), so v 2^62 =
+// m 2^10 / 2^(1023 - e), and m 2^10 < 2^63 leaves room for half a unit.
 __device__ __forceinline__ long long to_q62(double v)
 {
-    const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
-    const int e = static_cast<int>((b >> 52) & 0x7FF);
-    const unsigned long long frac = b & 0xFFFFFFFFFFFFFull;
-    const bool neg = (b >> 63) != 0;
-    if (e >= 1024) {                           // |v| >= 2, infinity or NaN
-        if (e == 2047 && frac)
+    const long long b = __double_as_longlong(v);
+    const unsigned long long frac = static_cast<unsigned long long>(b) & 0xFFFFFFFFFFFFFull;
+    const int k = 1023 - static_cast<int>((b >> 52) & 0x7FF);
+    if (k < 0) {                               // |v| >= 2, infinity or NaN
+        if (k == -1024 && frac)
             return LLONG_MIN;
-        return neg ? LLONG_MIN : LLONG_MAX;
+        return b < 0 ? LLONG_MIN : LLONG_MAX;
     }
-    if (e == 0)                                // zero or subnormal: |v 2^62| < 2^-960
-        return 0;
-    const unsigned long long m = frac | (1ull << 52);
-    const int s = e - 1013;
+    // (m 2^10 + 2^k / 2) >> k; PTX shifts by 64 and more give zero, as does
+    // the zero and subnormal exponent (k = 1023)
     unsigned long long mag;
-    if (s >= 0) {
-        mag = m << s;                          // s <= 10: below 2^63
-    } else if (s > -54) {
-        const int k = -s;
-        const unsigned long long q = m >> k, rem = m & ((1ull << k) - 1), half = 1ull << (k - 1);
-        mag = q + ((rem > half || (rem == half && (q & 1))) ? 1 : 0);
-    } else {
-        mag = 0;                               // below half a unit
-    }
-    return neg ? -static_cast<long long>(mag) : static_cast<long long>(mag);
+    asm("{\n\t.reg .b64 h;\n\t"
+        "shl.b64 h, %2, %3;\n\t"
+        "shr.u64 h, h, 1;\n\t"
+        "add.u64 h, h, %1;\n\t"
+        "shr.u64 %0, h, %3;\n\t}"
+        : "=l"(mag)
+        : "l"((frac | (1ull << 52)) << 10), "l"(1ull), "r"(k));
+    return b < 0 ? -static_cast<long long>(mag) : static_cast<long long>(mag);
 }
 
 // Decode `steps` symbols backward from Q (the span's stored point in Q1.62):
 // step j = 0 .. steps-1 emits the symbol at offset m-1-j of the span.
-// `emit(j, c)` receives each symbol.
-template <bool kShortChain = false, class Emit>
+// `emit(j, c)` receives each symbol.  Any Q, of any size: random reads,
+// retrieval, and spans that are no code point.
+template <class Emit>
 __device__ __forceinline__ void walk(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
 {
     const int N = t.N;
     for (int j = 0; j < steps; ++j) {
-        const int c = classify<kShortChain>(t, X, Y);
+        const int c = classify(t, X, Y);
         emit(j, c);
         const longlong2 w = t.T[j * N + c];
         X = static_cast<long long>(static_cast<unsigned long long>(X) - static_cast<unsigned long long>(w.x));
         Y = static_cast<long long>(static_cast<unsigned long long>(Y) - static_cast<unsigned long long>(w.y));
     }
+}
+
+template <class Emit>
+static __device__ __noinline__ void walk_any(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
+{
+    walk(t, X, Y, steps, emit);
+}
+
+// The walk of a code point for N > 8, where Voronoi regions are sectors.  A
+// code point's scale is known: |p_k| is in [1 - 2r, 1] (each p_k = V(c) +
+// r (p_{k-1} - V(c))), so step j's Q is within r^j [1 - 2r, 1] and a shift by
+// floor(j log2(1/r)) puts its magnitude in (0.24, 1] of the full scale (1 - 2r
+// >= 0.48 for N >= 9).  The direction is then one shift of each coordinate's
+// words and a 32-bit conversion, off by less than 2^-28 of its length.
+// Bound: instruction issue (62 % issue active; 88 instructions a symbol with
+// the span's set-up and stores).  50.3 M symbols of 6-symbol spans decode in
+// 0.170 ms; 0.216 ms with the magnitude found by leading-zero counts, two
+// 64-bit shifts, a division with its range cases and conversions for the
+// rounding (the planar decoder 0.089 against 0.119 ms for 25.1 M).
+// A Q that is no code point gets symbols of some kind (always in [0, N)) and
+// fails the anchor check: no other point is within 2^-4 r^m of the sum of the
+// steps taken.
+template <class Emit>
+__device__ __forceinline__ void walk_sectors(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
+{
+    const longlong2 *T = t.T;
+    int sh16 = 0;
+    for (int j = 0; j < steps; ++j, T += t.N, sh16 += t.sect_sh) {
+        const int sh = sh16 >> 16;
+        const float qx = __int2float_rn(static_cast<int>((static_cast<unsigned long long>(X) << sh) >> 32));
+        const float qy = __int2float_rn(static_cast<int>((static_cast<unsigned long long>(Y) << sh) >> 32));
+        const int c = classify_sector(t, X, Y, qx, qy);
+        emit(j, c);
+        const longlong2 w = T[c];
+        X = static_cast<long long>(static_cast<unsigned long long>(X) - static_cast<unsigned long long>(w.x));
+        Y = static_cast<long long>(static_cast<unsigned long long>(Y) - static_cast<unsigned long long>(w.y));
+    }
+}
+
+// Decode the m symbols of the span stored as p.  start() gives the receiver
+// emit(j, c) of a walk from its beginning; false when the walk does not end at
+// the anchor (|Q_0| <= lim), the symbols then being those of the general walk.
+template <class Start>
+__device__ __forceinline__ bool decode_point(const Tables &t, double2 p, int m, long long lim, Start start)
+{
+    long long X = to_q62(p.x), Y = to_q62(p.y);
+    auto off = [&] { return X > lim || X < -lim || Y > lim || Y < -lim; };
+    if (t.N <= 8) {
+        walk(t, X, Y, m, start());
+        return !off();
+    }
+    walk_sectors(t, X, Y, m, start());
+    if (!off())
+        return true;
+    long long X2 = to_q62(p.x), Y2 = to_q62(p.y);
+    walk_any(t, X2, Y2, m, start());
+    return false;
 }
 
 }  // namespace fkvdec

@@ -9,7 +9,7 @@
 #include <mutex>
 #include <vector>
 
-#include "fkv_internal.h"
+#include "decode_core.cuh"
 
 namespace {
 
@@ -360,11 +360,16 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
         rj *= static_cast<long double>(r);
     }
     // the fp32 sector angle's error, in sector widths: 1.2e-5 rad (arctangent
-    // polynomial) + 1.5e-6 rad (direction, division, reflections), times
+    // polynomial) + 1.5e-6 rad (direction, division, reflections) + 5e-7 rad
+    // (the polynomial's coefficients rounded again in sector widths), times
     // N / (2 pi), + N 2^-24 (scaling); fractions within twice that of a
     // boundary take the exact test
-    const double sect_err = N * (1.2e-5 + 1.5e-6) / (2.0 * 3.14159265358979) + N * 0x1p-24;
+    const double two_pi = 2.0 * 3.14159265358979;
+    const double sect_err = N * (1.2e-5 + 1.5e-6 + 5e-7) / two_pi + N * 0x1p-24;
     dec.sect_thr = static_cast<float>(0.5 - 2.0 * sect_err);
+    for (int i = 0; i < 5; ++i)
+        dec.sect_a[i] = static_cast<float>(static_cast<double>(fkvdec::kAtan[i]) * N / two_pi);
+    dec.sect_sh = static_cast<int>(floor(65536.0 * log2(1.0 / r)));
     CK(cudaMalloc(&ctx->d_V, N * sizeof(double2)), "vertex alloc");
     CK(cudaMemcpy(ctx->d_V, V.data(), N * sizeof(double2), cudaMemcpyHostToDevice), "vertex copy");
     CK(cudaMalloc(&ctx->d_dec, sizeof(fkv_decconst)), "decoder alloc");

@@ -39,6 +39,8 @@ struct fkv_decconst {
     float vfx[FKV_MAX_N], vfy[FKV_MAX_N];      // V(c) rounded to float
     long long alim[48];            // anchor limit 2^-4 r^m in Q1.62, per span length m
     float sect_thr;                // sector test threshold, N > 8 (decode_core.cuh classify)
+    float sect_a[5];               // arctangent polynomial in sector widths
+    int sect_sh;                   // floor(2^16 log2(1/r))
 };
 
 struct fkv_ctx {

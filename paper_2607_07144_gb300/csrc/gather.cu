@@ -389,16 +389,14 @@ __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a
         bool bad = false;
         for (int64_t u = u0 + lane; u <= u1; u += 32) {
             const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
-            const double2 p = a.pts[st * a.pt_stride + u];
-            long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-            const int64_t base = u * L - sym0;
-            fkvdec::walk<true>(t, X, Y, m, [&](int j, int c) {
-                const int64_t pos = base + m - 1 - j;
-                if (pos >= 0 && pos < R)
-                    my[pos] = static_cast<Sym>(c);
+            const int last = static_cast<int>(u * L - sym0) + m - 1;
+            bad |= !fkvdec::decode_point(t, a.pts[st * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
+                return [=](int j, int c) {
+                    const int pos = last - j;
+                    if (pos >= 0 && pos < R)
+                        my[pos] = static_cast<Sym>(c);
+                };
             });
-            const long long lim = __ldg(&a.dec->alim[m]);
-            bad |= X > lim || X < -lim || Y > lim || Y < -lim;
         }
         if (bad)
             atomicOr(a.status, FKV_ST_CORRUPT);
@@ -481,17 +479,15 @@ __global__ void __launch_bounds__(256) k_read_syms(const ReadArgs a, int spr)
         if (u > (sym0 + R - 1) / L)
             continue;
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
-        const double2 p = a.pts[e.y * a.pt_stride + u];
-        long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-        const int64_t base = u * L - sym0;
+        const int last = static_cast<int>(u * L - sym0) + m - 1;
         Sym *dst = scr + i * R;
-        fkvdec::walk<true>(t, X, Y, m, [&](int j, int c) {
-            const int64_t pos = base + m - 1 - j;
-            if (pos >= 0 && pos < R)
-                dst[pos] = static_cast<Sym>(c);
-        });
-        const long long lim = __ldg(&a.dec->alim[m]);
-        if (X > lim || X < -lim || Y > lim || Y < -lim)
+        if (!fkvdec::decode_point(t, a.pts[e.y * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
+                return [=](int j, int c) {
+                    const int pos = last - j;
+                    if (pos >= 0 && pos < R)
+                        dst[pos] = static_cast<Sym>(c);
+                };
+            }))
             atomicOr(a.status, FKV_ST_CORRUPT);
     }
 }

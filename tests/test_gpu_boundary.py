@@ -60,3 +60,23 @@ def test_boundary_spans_round_trip_bit_exact(fkv, oracle_mod, N):
     got = ctx.read_ragged(pts, po, so, torch.from_numpy(req).cuda()).cpu().numpy().astype(np.int64) & 0xFFFF
     assert ctx.sync_status() == 0
     assert np.array_equal(got, flat)
+
+
+@pytest.mark.parametrize("N", [9, 16, 255, 256, 1024])
+def test_points_that_code_nothing_decode_as_random_reads_do(fkv, N):
+    """Points outside every cell (the origin, far out, on an axis, not finite,
+    random) are reported, and the bulk decoders, whose fast walk assumes a code
+    point's scale, give the symbols the general walk of a random read gives."""
+    ctx = fkv.Context(N)
+    rng = np.random.default_rng(N)
+    p = np.concatenate([[(0, 0), (1e-300, 0), (0.9, 1e-17), (1.9, -1.9), (-5.0, 3.0), (np.inf, 0), (np.nan, 1)],
+                        rng.uniform(-1, 1, (505, 2)), rng.uniform(-1e-3, 1e-3, (512, 2))])
+    pts = torch.from_numpy(p[None].copy()).cuda()
+    n = p.shape[0] * ctx.L
+    dec = ctx.span_decode(pts, n)
+    assert ctx.sync_status() == -5
+    req = torch.stack([torch.zeros(n, dtype=torch.int64), torch.arange(n)], dim=1).cuda()
+    assert torch.equal(ctx.read(pts, n, req), dec[0])
+    so, po = ctx.ragged_offsets([n])
+    assert torch.equal(ctx.span_decode_ragged(pts[0], po, so), dec[0])
+    assert ctx.sync_status() == -5
