@@ -133,27 +133,33 @@ __device__ __forceinline__ float rcp_approx(float x)
     return y;
 }
 
-// The sector of direction (qx, qy), integers that image (X, Y): octant
-// reduction to u in [0, 1], atan u in sector widths from the odd polynomial of
-// fit_atan.py, the octant's reflections, and rounding by adding 1.5 2^23.
-__device__ __forceinline__ int classify_sector(const Tables &t, long long X, long long Y, float qx, float qy)
+// The sector of direction (qx, qy): octant reduction to u in [0, 1], atan u
+// in sector widths (coefficients k) from the odd polynomial of fit_atan.py,
+// the octant's reflections, and rounding by adding 1.5 2^23; f receives the
+// distance to the sector's centre.  No subnormal or huge coordinates; the
+// larger one is at least `least`, or both are zero.
+__device__ __forceinline__ int sector_of(int N, const float *k, float qx, float qy, float least, float &f)
 {
-    const int N = t.N;
     const float ax = fabsf(qx), ay = fabsf(qy);
-    // integers: no range or subnormal cases, and 0 / 1 at the origin
-    const float u = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), 1.0f));
+    const float u = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), least));
     const float u2 = u * u;
-    float a = u * fmaf(fmaf(fmaf(fmaf(t.sect_a[4], u2, t.sect_a[3]), u2, t.sect_a[2]), u2, t.sect_a[1]), u2,
-                       t.sect_a[0]);
+    float a = u * fmaf(fmaf(fmaf(fmaf(k[4], u2, k[3]), u2, k[2]), u2, k[1]), u2, k[0]);
     if (ay > ax)
         a = 0.25f * static_cast<float>(N) - a;
     if (qx < 0.0f)
         a = 0.5f * static_cast<float>(N) - a;
     a = copysignf(a, qy);                      // in [-N/2, N/2]
     const float big = a + 12582912.0f;
-    const float f = a - (big - 12582912.0f);   // in [-0.5, 0.5]
-    int c = __float_as_int(big) - 0x4B400000;
-    c += c < 0 ? N : 0;
+    f = a - (big - 12582912.0f);               // in [-0.5, 0.5]
+    const int c = __float_as_int(big) - 0x4B400000;
+    return c < 0 ? c + N : c;
+}
+
+// The sector of (X, Y), imaged by the integers (qx, qy).
+__device__ __forceinline__ int classify_sector(const Tables &t, long long X, long long Y, float qx, float qy)
+{
+    float f;
+    const int N = t.N, c = sector_of(N, t.sect_a, qx, qy, 1.0f, f);
     // away from a sector boundary by more than the angle's error allows
     if (fabsf(f) < t.sect_thr)
         return c;

@@ -369,15 +369,30 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
     dec.sect_thr = static_cast<float>(0.5 - 2.0 * sect_err);
     for (int i = 0; i < 5; ++i)
         dec.sect_a[i] = static_cast<float>(static_cast<double>(fkvdec::kAtan[i]) * N / two_pi);
+    memcpy(ctx->sect_a, dec.sect_a, sizeof(dec.sect_a));
+    ctx->sect_thr = dec.sect_thr;
     dec.sect_sh = static_cast<int>(floor(65536.0 * log2(1.0 / r)));
-    CK(cudaMalloc(&ctx->d_V, N * sizeof(double2)), "vertex alloc");
-    CK(cudaMemcpy(ctx->d_V, V.data(), N * sizeof(double2), cudaMemcpyHostToDevice), "vertex copy");
-    CK(cudaMalloc(&ctx->d_dec, sizeof(fkv_decconst)), "decoder alloc");
-    CK(cudaMemcpy(ctx->d_dec, &dec, sizeof(dec), cudaMemcpyHostToDevice), "decoder copy");
-    CK(cudaMalloc(&ctx->d_T, T.size() * sizeof(longlong2)), "decoder alloc");
-    CK(cudaMemcpy(ctx->d_T, T.data(), T.size() * sizeof(longlong2), cudaMemcpyHostToDevice), "decoder copy");
-    CK(cudaMalloc(&ctx->d_status, sizeof(unsigned)), "status alloc");
-    CK(cudaMemset(ctx->d_status, 0, sizeof(unsigned)), "status init");
+    // one allocation: the host-made tables in one copy, then the status word
+    // and the encoders' point table, filled on the device
+    int pre_count = 0;
+    ctx->pre_k = pre_table_symbols(N, span_len, &pre_count);
+    auto up16 = [](size_t n) { return (n + 15) & ~size_t(15); };
+    const size_t o_T = up16(N * sizeof(double2)), o_dec = o_T + up16(T.size() * sizeof(longlong2)),
+                 o_status = o_dec + up16(sizeof(dec)), o_pre = o_status + 16;
+    std::vector<uint8_t> tab(o_pre, 0);
+    memcpy(tab.data(), V.data(), N * sizeof(double2));
+    memcpy(tab.data() + o_T, T.data(), T.size() * sizeof(longlong2));
+    memcpy(tab.data() + o_dec, &dec, sizeof(dec));
+    uint8_t *base = nullptr;
+    CK(cudaMalloc(&base, o_pre + pre_count * sizeof(double2)), "context alloc");
+    ctx->d_V = reinterpret_cast<double2 *>(base);
+    ctx->d_T = reinterpret_cast<longlong2 *>(base + o_T);
+    ctx->d_dec = reinterpret_cast<fkv_decconst *>(base + o_dec);
+    ctx->d_status = reinterpret_cast<unsigned *>(base + o_status);
+    ctx->d_pre = reinterpret_cast<double2 *>(base + o_pre);
+    CK(cudaMemcpy(base, tab.data(), tab.size(), cudaMemcpyHostToDevice), "context copy");
+    CK(launch_pre_table(ctx, nullptr), "point table launch");
+    CK(cudaStreamSynchronize(nullptr), "context init");   // before any other stream uses the tables
 
     if (cb) {
         // the allocation-free archive read's fixed scratch: its address is
@@ -415,10 +430,7 @@ int fkv_destroy(fkv_ctx *ctx)
     if (!ctx)
         return FKV_OK;
     cudaDeviceSynchronize();
-    cudaFree(ctx->d_V);
-    cudaFree(ctx->d_dec);
-    cudaFree(ctx->d_T);
-    cudaFree(ctx->d_status);
+    cudaFree(ctx->d_V);            // and every table of fkv_create behind it
     cudaFree(ctx->d_scratch);
     cudaFree(ctx->d_read_order);
     destroy_cbset(ctx->cb[0]);

@@ -48,9 +48,13 @@ struct fkv_ctx {
     double r = 0.0;
     int L = 0;
     int device = 0;
-    double2 *d_V = nullptr;        // [N] vertices
+    double2 *d_V = nullptr;        // [N] vertices; first of one allocation with d_T, d_dec, d_status and d_pre
     fkv_decconst *d_dec = nullptr; // decoder constants (device copy)
     longlong2 *d_T = nullptr;      // [L][N] (1-r) r^j V(c) in Q1.62
+    double2 *d_pre = nullptr;      // [N^pre_k] points after pre_k symbols from the anchor (codec.cu)
+    int pre_k = 0;
+    float sect_a[5] = {};          // host copies of the decoder's sector constants
+    float sect_thr = 0.0f;
     unsigned *d_status = nullptr;
     // archive geometry and codebooks
     bool has_cb = false;
@@ -85,6 +89,11 @@ struct fkv_streams {
 // decoder tables plus one chunk of staged symbols.
 int codec_smem_bytes(int N, int L);
 constexpr int kMaxDynSmem = 232448;   // 227 KB per block on sm_103a
+
+// The bulk encoders' table of points after the first symbols of a span: how
+// many symbols it covers (and its entries), and the kernel that fills d_pre.
+int pre_table_symbols(int N, int L, int *count);
+cudaError_t launch_pre_table(const fkv_ctx *c, cudaStream_t st);
 
 // Symbols are uint8 when c->N <= 256, else uint16; strides count symbols.
 cudaError_t launch_span_encode(const fkv_ctx *c, const void *sym, int64_t n_streams, int64_t n,

@@ -155,3 +155,39 @@ def test_gpt2_archive_full_size(fkv, oracle_mod):
     assert not wrong[:, T * L:].any()                      # the recent spans are exact
     rate = wrong[:, :T * L].reshape(ns, T, L).mean(axis=(0, 1))
     assert rate[-1] < 0.01 and rate[0] > 0.9              # each span keeps its end, loses its start
+
+
+@pytest.mark.parametrize("N,r", [(3, 0.5), (3, 0.3), (4, 0.25), (7, 0.3), (16, 0.125), (16, 0.1), (256, 0.012),
+                                 (256, 0.0078125), (1000, 0.003)])
+def test_any_ratio_encodes_and_decodes_as_the_oracle(fkv, oracle_mod, N, r):
+    """Ratios below r_N, powers of two among them, where the encoders' product
+    and the lossy walk's division leave the FP64 pipe: points, codes and
+    (damaged) symbols bit for bit, span tails of every length included, and a
+    symbol >= N anywhere in a span is reported."""
+    ctx = fkv.Context(N, r=r)
+    L = ctx.L
+    dt = np.uint8 if N <= 256 else np.int16
+    for m in range(1, L + 1):
+        n = 65 * L + m
+        sym = _streams(N, 2, n, N + m)
+        pts = ctx.span_encode(torch.from_numpy(sym).cuda())
+        so, po = ctx.ragged_offsets([n, n])
+        rag = ctx.span_encode_ragged(torch.from_numpy(sym.reshape(-1)).cuda(), so, po)
+        bits = 2 + (11 * m) % 52
+        codes, tail = ctx.truncate(pts, n, bits, 3)
+        dec = ctx.lossy_decode(codes, tail, n, bits, 3).cpu().numpy()
+        assert ctx.sync_status() == 0
+        ph = pts.cpu().numpy()
+        assert np.array_equal(rag.cpu().numpy().reshape(ph.shape).view(np.uint64), ph.view(np.uint64))
+        for i in range(2):
+            want = oracle_mod.span_encode(sym[i].astype(np.int32), N, r, L)
+            assert np.array_equal(ph[i].view(np.uint64), want.view(np.uint64))
+            assert np.array_equal(dec[i], oracle_mod.lossy_decode(ph[i], n, N, r, L, bits, 3))
+    if N == 256:
+        return                                    # every byte is a symbol
+    for at in range(L):
+        sym = np.zeros((1, 2 * L), dt)
+        sym[0, at] = N
+        pts = ctx.span_encode(torch.from_numpy(sym).cuda())
+        assert ctx.sync_status() == -5
+        assert torch.isnan(pts[0, 0]).all() and not torch.isnan(pts[0, 1]).any()
