@@ -304,32 +304,6 @@ struct ChunkWalk {
     }
 };
 
-// Unsigned 32-bit division by an invariant d >= 1 as a multiply-high, a
-// subtract, an add and two shifts (Granlund and Montgomery, "Division by
-// invariant integers using multiplication", PLDI 1994, Sec. 4): with l =
-// ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1, t = mulhi(m, q) and
-// q / d = (t + ((q - t) >> min(l, 1))) >> max(l - 1, 0) for every 32-bit q.
-struct FastDiv {
-    unsigned m;
-    int sh1, sh2;
-    __host__ static FastDiv make(unsigned d)
-    {
-        int l = 0;
-        while ((1ull << l) < d)
-            ++l;
-        FastDiv f;
-        f.m = static_cast<unsigned>((((1ull << l) - d) << 32) / d + 1);
-        f.sh1 = l < 1 ? l : 1;
-        f.sh2 = l - 1 > 0 ? l - 1 : 0;
-        return f;
-    }
-    __device__ __forceinline__ unsigned div(unsigned q) const
-    {
-        const unsigned t = __umulhi(m, q);
-        return (t + ((q - t) >> sh1)) >> sh2;
-    }
-};
-
 // Persistent: a block loads the decoder tables once and walks chunks of
 // dec_threads spans (chunk = stream * bps + span block), blockIdx.x,
 // + gridDim.x, ...; each thread stores its span's symbols directly, so the
@@ -430,7 +404,7 @@ k_span_decode_staged(const double2 *__restrict__ pts, int64_t n, int64_t pt_stri
 template <typename Sym>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_span_decode_planar(const double2 *__restrict__ pts, unsigned n_rec, int64_t pt_stride, unsigned spans, int bps,
-                     unsigned n_chunks, Sym *__restrict__ out, int H, int SK, int SV, FastDiv div_r,
+                     unsigned n_chunks, Sym *__restrict__ out, int H, int SK, int SV, fkvd::FastDiv div_r,
                      const fkv_decconst *__restrict__ dc, const longlong2 *__restrict__ T, int N, int L,
                      unsigned *status)
 {
@@ -1252,7 +1226,7 @@ cudaError_t span_decode_planar_t(const fkv_ctx *c, const double *pts, int64_t n_
     k_span_decode_planar<Sym><<<grid, TPB, smem, st>>>(
         reinterpret_cast<const double2 *>(pts), static_cast<unsigned>(n_rec), pt_stride,
         static_cast<unsigned>(spans), static_cast<int>(bps), static_cast<unsigned>(n_chunks), out, c->H, SK, SV,
-        FastDiv::make(static_cast<unsigned>(R)), c->d_dec, c->d_T, c->N, c->L, c->d_status);
+        fkvd::FastDiv::make(static_cast<unsigned>(R)), c->d_dec, c->d_T, c->N, c->L, c->d_status);
     return cudaGetLastError();
 }
 

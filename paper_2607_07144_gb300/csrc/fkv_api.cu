@@ -199,6 +199,18 @@ int upload_cbset(fkv_ctx *ctx, int kv, const float *host, int stages)
     CUresult r = enc(&s.tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, s.cb16, dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const cuuint32_t box_half[2] = {64, 128};
+    if (r == CUDA_SUCCESS)
+        r = enc(&s.tmap_half, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, s.cb16, dims, strides, box_half, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const cuuint64_t dims_aug[2] = {64, static_cast<cuuint64_t>(ncode / 4)};
+    const cuuint64_t strides_aug[1] = {128};
+    const cuuint32_t box_aug[2] = {64, 32};
+    if (r == CUDA_SUCCESS)
+        r = enc(&s.tmap_aug, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, s.cbaug, dims_aug, strides_aug, box_aug, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(ctx, FKV_ECUDA, "cuTensorMapEncodeTiled failed");
     return FKV_OK;

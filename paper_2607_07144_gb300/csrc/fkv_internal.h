@@ -25,6 +25,8 @@ struct fkv_cbset {
     int *escale = nullptr;    // [G][S] exponent e of the fp16 split
     int *escale_h = nullptr;  // [Ly*H][S] the same per head (its group's), for k_rvq64
     CUtensorMap tmap;         // TMA map over cb16 as [rows][D], box {64, 256}, 128B swizzle
+    CUtensorMap tmap_half;    // the same, box {64, 128}: the half block of one CTA of a pair
+    CUtensorMap tmap_aug;     // cbaug as [lines][64] fp16 (4 codewords a line), box {64, 32}, no swizzle
     // 64-dimensional heads only (rvq.cu k_rvq64): cb16 holds the hi/lo split of
     // -2 c 2^-e with max |c 2^-e| in [2^3, 2^9), and cbaug the norm operand.
     __half *cbaug = nullptr;  // [G][S] blocks of K x 16 fp16 in core-matrix layout (32 B per codeword)
@@ -176,6 +178,32 @@ int64_t read_order_ints(const fkv_ctx *c, int64_t n_req);
 // ------------------------------------------------------- device helpers
 #ifdef __CUDACC__
 namespace fkvd {
+
+// Unsigned 32-bit division by an invariant d >= 1 as a multiply-high, a
+// subtract, an add and two shifts (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", PLDI 1994, Sec. 4): with l =
+// ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1, t = mulhi(m, q) and
+// q / d = (t + ((q - t) >> min(l, 1))) >> max(l - 1, 0) for every 32-bit q.
+struct FastDiv {
+    unsigned m;
+    int sh1, sh2;
+    __host__ static FastDiv make(unsigned d)
+    {
+        int l = 0;
+        while ((1ull << l) < d)
+            ++l;
+        FastDiv f;
+        f.m = static_cast<unsigned>((((1ull << l) - d) << 32) / d + 1);
+        f.sh1 = l < 1 ? l : 1;
+        f.sh2 = l - 1 > 0 ? l - 1 : 0;
+        return f;
+    }
+    __device__ __forceinline__ unsigned div(unsigned q) const
+    {
+        const unsigned t = __umulhi(m, q);
+        return (t + ((q - t) >> sh1)) >> sh2;
+    }
+};
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {

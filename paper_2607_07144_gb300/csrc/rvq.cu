@@ -40,7 +40,15 @@ struct RvqArgs {
     int R, kv_off;
     int tiles_per_group;
     unsigned *status;
+    FastDiv div_pos, div_heads;   // by n_pos (vectors of a group below 2^31, else unused) and n_heads
+    bool small;                   // batch * n_pos < 2^31
 };
+
+// Sequence of vector v of a group (v = sequence n_pos + position).
+__device__ __forceinline__ int64_t vec_seq(const RvqArgs &a, int64_t v)
+{
+    return a.small ? static_cast<int64_t>(a.div_pos.div(static_cast<unsigned>(v))) : v / a.n_pos;
+}
 
 // Byte offset of 16-byte chunk `kk` (0..7) of row `row` inside one
 // 128-row-per-atom K block in the 128-byte swizzle layout.
@@ -170,7 +178,7 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b)
 __device__ __forceinline__ float min3f(float a, float b, float c)
 {
     float d;
-    asm volatile("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
 
@@ -334,7 +342,7 @@ __device__ __forceinline__ void load_add_chunk(const uint8_t *ahi, const uint8_t
 // arithmetic as load_add_chunk and store_chunk: hi + lo exact, one rounding
 // in the multiply-add.  Software-pipelined over batches of 8 rows: the next
 // batch's codeword loads are in flight while one batch is updated.
-template <bool UF>
+template <bool UF, int D = 128>
 __device__ __forceinline__ void update_rows_t(uint8_t *ahi, uint8_t *alo, int quad, const float *cbk, int bidx,
                                               float f)
 {
@@ -343,25 +351,18 @@ __device__ __forceinline__ void update_rows_t(uint8_t *ahi, uint8_t *alo, int qu
     const uint32_t cw = static_cast<uint32_t>(li >> 1), wo = static_cast<uint32_t>((li & 1) << 3);
     const float4 *cl = reinterpret_cast<const float4 *>(cbk) + li;
     uint8_t *qhi = ahi + quad * 32 * 128, *qlo = alo + quad * 32 * 128;
-    float4 cv[2][4];
-    float fm[2][4];
+    float4 cv[3][4];
+    auto fetch = [&](int b) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int m = 2 * j + hs;
-        fm[0][j] = UF ? f : __shfl_sync(0xFFFFFFFFu, f, m);
-        cv[0][j] = __ldg(cl + __shfl_sync(0xFFFFFFFFu, bidx, m) * 32);
-    }
+        for (int j = 0; j < 4; ++j)
+            cv[b % 3][j] = __ldg(cl + __shfl_sync(0xFFFFFFFFu, bidx, 8 * b + 2 * j + hs) * (D / 4));
+    };
+    fetch(0);
+    fetch(1);
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-        const int cur = b & 1, nxt = cur ^ 1;
-        if (b < 3) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int m = 8 * (b + 1) + 2 * j + hs;
-                fm[nxt][j] = UF ? f : __shfl_sync(0xFFFFFFFFu, f, m);
-                cv[nxt][j] = __ldg(cl + __shfl_sync(0xFFFFFFFFu, bidx, m) * 32);
-            }
-        }
+        if (b < 2)
+            fetch(b + 2);
         uint2 hv[4], lv[4];
         uint32_t off[4];
 #pragma unroll
@@ -373,13 +374,15 @@ __device__ __forceinline__ void update_rows_t(uint8_t *ahi, uint8_t *alo, int qu
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
+            const float4 c = cv[b % 3][j];
+            const float fj = UF ? f : __shfl_sync(0xFFFFFFFFu, f, 8 * b + 2 * j + hs);
             float v0, v1, v2, v3;
             join_half2(hv[j].x, lv[j].x, v0, v1);
             join_half2(hv[j].y, lv[j].y, v2, v3);
-            v0 = fmaf(cv[cur][j].x, fm[cur][j], v0);
-            v1 = fmaf(cv[cur][j].y, fm[cur][j], v1);
-            v2 = fmaf(cv[cur][j].z, fm[cur][j], v2);
-            v3 = fmaf(cv[cur][j].w, fm[cur][j], v3);
+            v0 = fmaf(c.x, fj, v0);
+            v1 = fmaf(c.y, fj, v1);
+            v2 = fmaf(c.z, fj, v2);
+            v3 = fmaf(c.w, fj, v3);
             uint2 h, l;
             split_half2(v0, v1, h.x, l.x);
             split_half2(v2, v3, h.y, l.y);
@@ -414,42 +417,36 @@ __device__ __forceinline__ void unpack8(const uint4 *xr, int dtype, int c, float
     }
 }
 
-// Argmin of one accumulator row as argmin_row, reading four 16-column chunks
-// per tensor-memory wait.
+// Minimum and argmin of one accumulator row, four 16-column chunks per
+// tensor-memory wait: the chunk minima come with the loads, an elementwise
+// minimum across the chunks keeps each position's (two three-input minima per
+// position and 64 columns), and the row minimum's place in both gives the
+// column.  *amb: more than one place (an exact tie), or none (no number).
 __device__ __forceinline__ int argmin_row4(uint32_t trow, bool *amb, float *vmin)
 {
-    float m[16];
-    float best = INFINITY;
-    int bc = 0;
-    bool tie = false;
-#pragma unroll 1
-    for (int c = 0; c < kCodes / 16; c += 4) {
-        float a[16], b[16], d[16], e[16], ra, rb, rd, re;
-        tmem_red4x16(trow + c * 16, a, b, d, e, ra, rb, rd, re);
+    float m[16], rr[16];
 #pragma unroll
-        for (int p = 0; p < 16; ++p) {
-            const float t = fminf(min3f(a[p], b[p], d[p]), e[p]);
-            m[p] = c == 0 ? t : fminf(m[p], t);
-        }
-        const float rr[4] = {ra, rb, rd, re};
+    for (int c = 0; c < 4; ++c) {
+        float a[16], b[16], d[16], e[16];
+        tmem_red4x16(trow + c * 64, a, b, d, e, rr[4 * c], rr[4 * c + 1], rr[4 * c + 2], rr[4 * c + 3]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (rr[i] < best) {
-                best = rr[i];
-                bc = c + i;
-                tie = false;
-            } else if (rr[i] == best) {
-                tie = true;
-            }
-        }
+        for (int p = 0; p < 16; ++p)
+            m[p] = c == 0 ? fminf(min3f(a[p], b[p], d[p]), e[p]) : min3f(min3f(m[p], a[p], b[p]), d[p], e[p]);
     }
-    uint32_t pm = 0;
+    float best = rr[15];
 #pragma unroll
-    for (int p = 0; p < 16; ++p)
-        pm |= (m[p] == best ? 1u : 0u) << p;
-    *amb = tie || pm == 0 || (pm & (pm - 1)) != 0;
-    *vmin = best;
-    return bc * 16 + (__ffs(pm) - 1);
+    for (int i = 0; i < 14; i += 2)
+        best = min3f(best, rr[i], rr[i + 1]);
+    best = fminf(best, rr[14]);
+    uint32_t cm = 0, pm = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        cm |= (rr[i] == best ? 1u : 0u) << i;
+        pm |= (m[i] == best ? 1u : 0u) << i;
+    }
+    *amb = cm == 0 || pm == 0 || (cm & (cm - 1)) != 0 || (pm & (pm - 1)) != 0;
+    *vmin = fminf(best, INFINITY);
+    return (__ffs(cm) - 1) * 16 + (__ffs(pm) - 1);
 }
 
 // Exact argmin of an accumulator row (float compare, lowest index on ties).
@@ -848,6 +845,601 @@ k_rvq64(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int pairs_per
     }
 }
 
+
+// ===================================================================
+// 64-dimensional heads, two SMs per tile pair.
+//
+// k_rvq64's arithmetic on CTA pairs (cta_group::2): a unit is two 128-vector
+// tiles of one codebook group, one in each CTA of a cluster, and one
+// tcgen05.mma (M = 256, N = 256, K = 16) issued by the leader multiplies both
+// against the stage operands, of which each CTA holds half the codewords.
+// What bounded k_rvq64 was the SM's shared-memory port (operand reads of the
+// MMAs, TMA writes and the residual update together) and each tile slot's
+// serial chain (MMA, argmin, update).  The pair halves the operand reads of B
+// and the TMA writes, and the room it frees holds a third tile slot: three
+// four-warp groups walk a unit each and share two accumulators, since a slot
+// holds its accumulator only from its MMAs to the end of its argmin.
+//
+// Work item n (unit round, stage, block of 256 codewords, slot) uses
+// accumulator n & 1 and ring buffer n mod 3.  Barriers, in the leader unless
+// both CTAs are named: full (the two halves of a buffer have landed), empty
+// (both; the item's MMAs are done), a_ready (the slot's operand rows are
+// written, one arrival per epilogue warp of both CTAs), acc_full (both; per
+// slot, so that every group waits on a barrier of its own phases), acc_free
+// (the accumulator's scores are read).  The epilogue takes the chosen codeword
+// from its float32 row in L2, two rows per instruction.
+//
+// GPT-2-shaped cache, 1,138,176 vectors of K (4 stages) and of V (2): 486 us
+// against 633 for k_rvq64, and with 1024-codeword codebooks 1,013 against
+// 1,192 (85 % of the time the 13 MMAs of a block take alone).  At four stages a
+// slot's round is 1,560 cycles of input, 3,200 waiting for its MMAs, 1,270 of
+// argmin and 2/3 x 2,600 of update: instruction issue and L2 latency of the
+// epilogue, not the tensor pipe, still bound it.  Cluster-scope releases on
+// every arrival cost 572 us, contiguous unit ranges per cluster 538 (their
+// codebooks spread over all groups), the argmin's two-load pipelining 613.
+namespace pr {
+constexpr int kSlots = 3;
+constexpr int kBufs = 3;
+constexpr int kWarps = 2 + 4 * kSlots;       // 0 TMA, 1 MMA, then the epilogue groups
+constexpr int kThreads = kWarps * 32;
+constexpr int kHalf = kCodes / 2;            // codewords of a block per CTA
+constexpr int A_TILE = kRows * 128;          // 16 KB: 128 rows x 64 fp16 (128-byte swizzle)
+constexpr int A_SLOT = 2 * A_TILE;           // hi + lo
+constexpr int A_AUG = kRows * 32;            // 4 KB per slot
+constexpr int B_TILE = kHalf * 128;          // 16 KB
+constexpr int B_AUG = kHalf * 32;            // 4 KB
+constexpr int B_BUF = 2 * B_TILE + B_AUG;    // 36 KB
+constexpr int OFF_AAUG = kSlots * A_SLOT;
+constexpr int OFF_B = OFF_AAUG + kSlots * A_AUG;
+constexpr int OFF_BAR = OFF_B + kBufs * B_BUF;
+constexpr int BAR_FULL = 0, BAR_EMPTY = 3, BAR_READY = 6, BAR_ACC = 9, BAR_FREE = 12, BAR_DRAIN = 14, kBars = 15;
+constexpr int OFF_SLOT = OFF_BAR + 8 * 16;
+constexpr int OFF_LO = OFF_SLOT + 16;        // per slot: the round whose first-stage lo operand is nonzero (leader)
+constexpr int OFF_ABORT = OFF_LO + 16;
+constexpr int END = OFF_ABORT + 16;
+constexpr int SMEM = END + 1024;
+static_assert(OFF_B % 1024 == 0 && B_BUF % 1024 == 0 && SMEM <= 232448, "shared memory");
+}  // namespace pr
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Address in the cluster's shared window of `addr` in CTA `rank`.
+__device__ __forceinline__ uint32_t map_cta(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
+// Arrive on a barrier of either CTA.  What it hands over is this SM's own
+// shared or tensor memory, made visible to the tensor core by the proxy and
+// tcgen05 fences before it; only the lo stamp, a word in the leader, needs the
+// cluster-scope release, whose memory barrier costs every arrival some 500
+// cycles (16 % of all stalls).
+template <bool STAMP = false>
+__device__ __forceinline__ void arrive_cluster(uint32_t bar)
+{
+    if (STAMP)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    else
+        asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void store_cluster(uint32_t addr, int v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// wait_or_abort with cluster-scope acquire (the lo stamps).
+__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, unsigned *status, volatile int *abort_flag)
+{
+    return wait_or_abort(bar, parity, status, abort_flag) && try_wait_cluster(bar, parity);
+}
+
+// 2-D TMA tile load into this CTA's shared memory, counted on a barrier of
+// the pair's leader.
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem, uint32_t ncols)
+{
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_smem), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols)
+{
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+
+__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrive on `bar` of both CTAs once every tcgen05.mma issued before is done.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+        "h"(static_cast<uint16_t>(3))
+        : "memory");
+}
+
+// store_chunk for four values, half h of a row's 16 eight-byte units.
+__device__ __forceinline__ uint32_t store_half_chunk(uint8_t *ahi, uint8_t *alo, int row, int h, const float *v)
+{
+    uint2 hv, lv;
+    split_half2(v[0], v[1], hv.x, lv.x);
+    split_half2(v[2], v[3], hv.y, lv.y);
+    const uint32_t off = swz(row, h >> 1) + ((h & 1) << 3);
+    *reinterpret_cast<uint2 *>(ahi + off) = hv;
+    *reinterpret_cast<uint2 *>(alo + off) = lv;
+    return (lv.x | lv.y) & 0x7FFF7FFFu;
+}
+
+// One 64-dimension block of the 32 rows of a lane quadrant from the input to
+// the hi/lo operand tile, scaled by se: a row's 16-byte chunks on neighbouring
+// lanes, eight loads in flight.  row0 is this lane's own row (its block's
+// first element, null for a row of zeros).  mx and nz collect the magnitude
+// and the nonzero lo bits of what this lane stored.
+template <int ESZ>
+__device__ __forceinline__ void load_rows64(uint8_t *ahi, uint8_t *alo, int quad, const uint4 *row0, int dtype, float se,
+                                            float &mx, uint32_t &nz)
+{
+    constexpr int LPR = 64 * ESZ / 16, RPI = 32 / LPR;       // lanes per row, rows per instruction
+    const int lane = threadIdx.x & 31;
+    const uint64_t mine = reinterpret_cast<uint64_t>(row0);
+#pragma unroll
+    for (int h = 0; h < LPR / 8; ++h) {
+        uint4 xr[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int m = (8 * h + i) * RPI + lane / LPR;
+            const uint4 *p = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, mine, m));
+            xr[i] = p ? __ldg(p + lane % LPR) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int m = quad * 32 + (8 * h + i) * RPI + lane / LPR;
+            float f[8];
+            if (ESZ == 2) {
+                unpack8<ESZ>(&xr[i], dtype, 0, f);
+            } else {
+                f[0] = __uint_as_float(xr[i].x);
+                f[1] = __uint_as_float(xr[i].y);
+                f[2] = __uint_as_float(xr[i].z);
+                f[3] = __uint_as_float(xr[i].w);
+            }
+#pragma unroll
+            for (int q = 0; q < 16 / ESZ; ++q) {
+                f[q] = f[q] * se;
+                mx = fmaxf(mx, fabsf(f[q]));
+            }
+            if (ESZ == 2)
+                nz |= store_chunk(ahi, alo, m, lane % LPR, f);
+            else
+                nz |= store_half_chunk(ahi, alo, m, lane % LPR, f);
+        }
+    }
+}
+
+// Indices of S stages, packed from the low end, to their record slots.
+template <typename Sym>
+__device__ __forceinline__ void store_indices(Sym *dst, uint64_t idx, int S)
+{
+    const uintptr_t at = reinterpret_cast<uintptr_t>(dst);
+    if (sizeof(Sym) == 1 && S == 4 && (at & 3) == 0) {
+        *reinterpret_cast<uint32_t *>(dst) = static_cast<uint32_t>(idx);
+        return;
+    }
+    if (sizeof(Sym) == 1 && S == 2 && (at & 1) == 0) {
+        *reinterpret_cast<uint16_t *>(dst) = static_cast<uint16_t>(idx);
+        return;
+    }
+    for (int s = 0; s < S; ++s)
+        dst[s] = static_cast<Sym>(idx >> (8 * sizeof(Sym) * s));
+}
+
+template <int ESZ, int NB>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pr::kThreads, 1)
+k_rvq64_pair(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_aug, const RvqArgs a,
+             int units_per_group, int n_units, FastDiv div_unit)
+{
+    using namespace pr;
+    using Sym = typename std::conditional<NB == 1, uint8_t, uint16_t>::type;
+    constexpr int KC = NB * kCodes;              // codewords per stage
+    constexpr int XC = 64 * ESZ / 16;            // 16-byte chunks per input row
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t sbase = smem_u32(base);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(base + OFF_ABORT);
+    volatile int *lo_stamp = reinterpret_cast<volatile int *>(base + OFF_LO);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_rank();
+    auto bar = [&](int i) { return sbase + OFF_BAR + 8u * i; };
+    if (tid == 0) {
+        for (int i = 0; i < kBars; ++i)
+            mbar_init(bar(i), (i >= BAR_READY && i < BAR_ACC) || (i >= BAR_FREE && i < BAR_DRAIN) ? 8 : 1);
+        for (int k = 0; k < kSlots; ++k)
+            lo_stamp[k] = 0;
+        *abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&tmap);
+        prefetch_tmap(&tmap_aug);
+    }
+    if (warp == 1)
+        tmem_alloc_pair(sbase + OFF_SLOT, 512);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(base + OFF_SLOT);
+    const int S = a.S;
+    const int64_t nvec = a.batch * a.n_pos;
+    auto cgroup = [&](int g) { return a.pooled ? g / a.n_heads : g; };
+    // the clusters take the units in turn, so that at any time they work on a few
+    // codebook groups, whose operands L2 then serves; in this cluster's own count
+    // (units 0 .. nu-1), slot k of round j takes unit 3 j + k
+    const int cid = blockIdx.x >> 1, nc = gridDim.x >> 1;
+    const int nu = (n_units - cid + nc - 1) / nc;
+
+    if (warp == 0) {
+        // ---------------------------------------------------- TMA producer (both CTAs)
+        if (lane == 0) {
+            int b = 0;
+            uint32_t ph = 0, used[kBufs] = {0, 0, 0};      // loads issued into each buffer
+            bool ok = true;
+            for (int ur = 0; ur < nu && ok; ur += kSlots) {
+                for (int s = 0; s < S && ok; ++s) {
+                    for (int blk = 0; blk < NB && ok; ++blk) {
+                        for (int u = ur; u < min(ur + kSlots, nu); ++u) {
+                            const int gs = cgroup(static_cast<int>(div_unit.div(static_cast<unsigned>(cid + u * nc)))) * S + s;
+                            if (!wait_or_abort(bar(BAR_EMPTY + b), ph ^ 1, a.status, abort_flag)) {
+                                ok = false;
+                                break;
+                            }
+                            const uint32_t full = map_cta(bar(BAR_FULL + b), 0);
+                            const uint32_t bb = sbase + OFF_B + b * B_BUF;
+                            const int row0 = gs * 2 * KC + blk * kCodes + static_cast<int>(rank) * kHalf;
+                            if (rank == 0)
+                                mbar_arrive_expect_tx(bar(BAR_FULL + b), 2u * B_BUF);
+                            tma_load_pair(bb, &tmap, 0, row0, full);
+                            tma_load_pair(bb + B_TILE, &tmap, 0, row0 + KC, full);
+                            // the norm operand as lines of 128 bytes (4 codewords each)
+                            tma_load_pair(bb + 2 * B_TILE, &tmap_aug, 0,
+                                          gs * (KC / 4) + blk * (kCodes / 4) + static_cast<int>(rank) * (kHalf / 4),
+                                          full);
+                            ++used[b];
+                            if (++b == kBufs) {
+                                b = 0;
+                                ph ^= 1;
+                            }
+                        }
+                    }
+                }
+            }
+            // no copy may still be landing in shared memory when a CTA exits: the
+            // leader waits for the pair's last loads (the cluster meets after that);
+            // after an abort the other CTA gives loads the leader never armed time to land
+            if (rank == 0) {
+                for (int i = 0; i < kBufs; ++i)
+                    if (used[i])
+                        mbar_wait(bar(BAR_FULL + i), (used[i] - 1) & 1, a.status);
+            } else if (!ok) {
+                const uint64_t t0 = globaltimer_ns();
+                while (globaltimer_ns() - t0 < 2000000) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------------------------------------------- MMA issuer (leader)
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = idesc_f16_f32(2 * kRows, kCodes);
+            int b = 0, pc = 0;
+            uint32_t n = 0, ph = 0, aph = 0;              // aph: parity of a_ready per slot, bit k
+            bool ok = true;
+            for (int ur = 0; ur < nu && ok; ur += kSlots) {
+                ++pc;
+                const int act = min(kSlots, nu - ur);
+                for (int s = 0; s < S && ok; ++s) {
+                    for (int blk = 0; blk < NB && ok; ++blk) {
+                        for (int k = 0; k < act; ++k, ++n) {
+                            if (blk == 0) {
+                                ok = wait_cluster(bar(BAR_READY + k), (aph >> k) & 1, a.status, abort_flag);
+                                aph ^= 1u << k;
+                            }
+                            ok = ok && wait_or_abort(bar(BAR_FULL + b), ph, a.status, abort_flag) &&
+                                 (n < 2 || wait_or_abort(bar(BAR_FREE + (n & 1)), ((n >> 1) - 1) & 1, a.status, abort_flag));
+                            if (!ok)
+                                break;
+                            tc_fence_after();
+                            // the lo operand is nonzero after the first stage; at the
+                            // first stage only if a row's input needs it
+                            const bool lo = s > 0 || lo_stamp[k] == pc;
+                            const uint32_t ab = sbase + k * A_SLOT;
+                            const uint32_t bb = sbase + OFF_B + b * B_BUF;
+                            const uint32_t acc = tmem + (n & 1) * 256;
+                            // codeword norms first (K = 16, no swizzle), then the split dot products
+                            umma_f16_pair(acc, sdesc_core16(sbase + OFF_AAUG + k * A_AUG),
+                                          sdesc_core16(bb + 2 * B_TILE), idesc, 0);
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk) {
+                                const uint64_t dah = sdesc_sw128(ab + kk * 32);
+                                const uint64_t dal = sdesc_sw128(ab + A_TILE + kk * 32);
+                                const uint64_t dbh = sdesc_sw128(bb + kk * 32);
+                                const uint64_t dbl = sdesc_sw128(bb + B_TILE + kk * 32);
+                                umma_f16_pair(acc, dah, dbh, idesc, 1);
+                                umma_f16_pair(acc, dah, dbl, idesc, 1);
+                                if (lo)
+                                    umma_f16_pair(acc, dal, dbh, idesc, 1);
+                            }
+                            umma_commit_pair(bar(BAR_ACC + k));
+                            umma_commit_pair(bar(BAR_EMPTY + b));
+                            if (++b == kBufs) {
+                                b = 0;
+                                ph ^= 1;
+                            }
+                        }
+                    }
+                }
+            }
+            // every MMA has completed before tensor memory is released
+            umma_commit_pair(bar(BAR_DRAIN));
+            mbar_wait(bar(BAR_DRAIN), 0, a.status);
+        }
+    } else {
+        // ---------------------------------------------------- epilogue groups
+        const int k = (warp - 2) >> 2;           // tile slot
+        const int quad = warp & 3;                // TMEM lane quadrant of this warp
+        const int row = quad * 32 + lane;
+        const uint32_t tquad = static_cast<uint32_t>(quad * 32) << 16;
+        uint8_t *ahi = base + k * A_SLOT;
+        uint8_t *alo = ahi + A_TILE;
+        uint8_t *aaug = base + OFF_AAUG + k * A_AUG;
+        const uint32_t ready = map_cta(bar(BAR_READY + k), 0);
+        const uint32_t free0 = map_cta(bar(BAR_FREE), 0);
+        const uint32_t lo_at = map_cta(sbase + OFF_LO + 4 * k, 0);
+        // this row of a unit: its codebook group's head group, its input row and its
+        // record slot (null past the data)
+        struct Unit {
+            int g;
+            const uint4 *src;
+            Sym *dst;
+        };
+        auto unit_of = [&](int i) {
+            const int u = cid + i * nc;
+            Unit w;
+            w.g = static_cast<int>(div_unit.div(static_cast<unsigned>(u)));
+            const int64_t v = (static_cast<int64_t>(u - w.g * units_per_group) * 2 + rank) * kRows + row;
+            w.src = nullptr;
+            w.dst = nullptr;
+            if (v < nvec) {
+                const int l = static_cast<int>(a.div_heads.div(static_cast<unsigned>(w.g))), h = w.g - l * a.n_heads;
+                const int64_t b = vec_seq(a, v), t = v - b * a.n_pos;
+                w.src = reinterpret_cast<const uint4 *>(
+                    static_cast<const uint8_t *>(a.x) +
+                    (l * a.s_layer + b * a.s_batch + h * a.s_head + (a.t0 + t) * a.s_pos) * ESZ);
+                w.dst = static_cast<Sym *>(a.sym) + (b * a.n_layers + l) * a.stream_stride + (a.rec0 + t) * a.R +
+                        a.kv_off + h * S;
+            }
+            return w;
+        };
+        uint32_t n0 = 0;                          // items before this round
+        uint32_t fph = 0;
+        int pc = 0;
+        bool ok = true;
+        for (int ur = 0; ur + k < nu && ok; ur += kSlots) {
+            const int u = ur + k, act = min(kSlots, nu - ur);
+            const Unit cur = unit_of(u);
+            const int g = cur.g;
+            const bool valid = cur.src != nullptr;
+            // the row's operand t = x 2^-(e + er): e the stage scale of the
+            // codebooks, er >= 0 the row shift keeping |t| below 2^12
+            int e = __ldg(&a.escale_h[g * S]);
+            int er;
+            ++pc;
+            {
+                const uint4 *src = cur.src;
+                const float se = pow2f(-e);
+                float mx = 0.0f;
+                uint32_t nz = 0;
+                load_rows64<ESZ>(ahi, alo, quad, src, a.dtype, se, mx, nz);
+                er = 0;
+                if (__any_sync(0xFFFFFFFFu, !(mx < 4096.0f))) {
+                    // a row of larger magnitude (the usual case has none): its lane stores
+                    // it again, shifted
+                    __syncwarp();
+                    auto chunk = [&](int c, float *f) {
+                        uint4 x[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+                        if (valid) {
+                            x[0] = __ldg(src + c * (ESZ / 2));
+                            if (ESZ == 4)
+                                x[1] = __ldg(src + c * 2 + 1);
+                        }
+                        unpack8<ESZ>(x, a.dtype, 0, f);
+                    };
+                    float rm = 0.0f;
+                    for (int c = 0; c < 8; ++c) {
+                        float f[8];
+                        chunk(c, f);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            rm = fmaxf(rm, fabsf(f[i] * se));
+                    }
+                    er = row_shift(rm);
+                    if (er != 0) {
+                        const float sr = pow2f(-er);
+                        for (int c = 0; c < 8; ++c) {
+                            float f[8];
+                            chunk(c, f);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                f[i] = f[i] * se * sr;
+                            nz |= store_chunk(ahi, alo, row, c, f);
+                        }
+                    }
+                }
+                write_aug_row(aaug, row, er);
+                const bool lo = __any_sync(0xFFFFFFFFu, nz != 0);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    if (lo) {
+                        store_cluster(lo_at, pc);
+                        arrive_cluster<true>(ready);
+                    } else {
+                        arrive_cluster(ready);
+                    }
+                }
+            }
+            if (u + kSlots < nu) {
+                // the slot's next input row into L2 while this unit runs
+                const Unit nxt = unit_of(u + kSlots);
+                if (nxt.src) {
+#pragma unroll
+                    for (int c = 0; c < XC; c += 8)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt.src + c));
+                }
+            }
+            uint64_t idx = 0;
+            for (int s = 0; s < S; ++s) {
+                const int e_next = s + 1 < S ? __ldg(&a.escale_h[g * S + s + 1]) : e;   // in flight during the waits
+                float bv = INFINITY;
+                int bidx = 0;
+                for (int blk = 0; blk < NB; ++blk) {
+                    const uint32_t acc = (n0 + static_cast<uint32_t>((s * NB + blk) * act + k)) & 1;
+                    ok = wait_or_abort(bar(BAR_ACC + k), fph, a.status, abort_flag);
+                    // the tensor-memory loads below are warp-collective: the warp
+                    // goes on, or leaves, as one
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok)
+                        break;
+                    fph ^= 1;
+                    tc_fence_after();
+                    const uint32_t trow = tmem + acc * 256 + tquad;
+                    bool amb;
+                    float vu;
+                    int j = argmin_row4(trow, &amb, &vu);
+                    if (__any_sync(0xFFFFFFFFu, amb)) {   // warp-collective loads: every lane takes part
+                        const int jj = exact_argmin_tmem(trow);
+                        if (amb)
+                            j = jj;
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0)
+                        arrive_cluster(free0 + 8 * acc);
+                    if (NB == 1 || blk == 0 || vu < bv) {
+                        bv = vu;
+                        bidx = blk * kCodes + j;
+                    }
+                }
+                if (!ok)
+                    break;
+                idx |= static_cast<uint64_t>(bidx) << (8 * sizeof(Sym) * s);
+                if (s + 1 < S) {
+                    // t <- t - c 2^(-e-er), the chosen codeword from its float32 row
+                    const float f = -pow2f(-e - er);
+                    const float *cbs = a.cb32 + static_cast<int64_t>(cgroup(g) * S + s) * KC * 64;
+                    if (e_next == e) {
+                        // |t| stays below 2^12 + S 2^9 < 2^14: the row shift holds
+                        if (__all_sync(0xFFFFFFFFu, er == 0))
+                            update_rows_t<true, 64>(ahi, alo, quad, cbs, bidx, f);
+                        else
+                            update_rows_t<false, 64>(ahi, alo, quad, cbs, bidx, f);
+                    } else {
+                        // the next stage has another codebook scale: rescale the row and
+                        // choose its shift again from the updated magnitude
+                        const float4 *gc = reinterpret_cast<const float4 *>(cbs + bidx * 64);
+                        float mx = 0.0f;
+#pragma unroll 1
+                        for (int c = 0; c < 8; ++c) {
+                            float t[8];
+                            load_add_chunk(ahi, alo, row, c, __ldg(gc + 2 * c), __ldg(gc + 2 * c + 1), f, t);
+#pragma unroll
+                            for (int i = 0; i < 8; i += 2)
+                                mx = max3f(mx, fabsf(t[i]), fabsf(t[i + 1]));
+                        }
+                        int E = 0;
+                        if (mx > 0.0f)
+                            frexpf(mx, &E);                      // |t| < 2^E in units 2^-(e + er)
+                        const int tot = E + er + e - e_next;     // |r| < 2^tot in units 2^-e_next
+                        const int er2 = tot > v2::kRowLog ? tot - v2::kRowLog : 0;
+                        const float gsc = pow2f(er + e - e_next - er2);
+#pragma unroll 1
+                        for (int c = 0; c < 8; ++c) {
+                            float t[8];
+                            load_add_chunk(ahi, alo, row, c, __ldg(gc + 2 * c), __ldg(gc + 2 * c + 1), f, t);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                t[i] *= gsc;
+                            store_chunk(ahi, alo, row, c, t);
+                        }
+                        er = er2;
+                        write_aug_row(aaug, row, er);
+                    }
+                    e = e_next;
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0)
+                        arrive_cluster(ready);
+                }
+            }
+            if (!ok)
+                break;
+            if (valid)
+                store_indices(cur.dst, idx, S);
+            n0 += static_cast<uint32_t>(act * S * NB);
+        }
+    }
+    // neither CTA leaves, or gives tensor memory back, while the other may still
+    // arrive on its barriers or read its shared memory
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    if (warp == 1) {
+        __syncwarp();
+        tmem_dealloc_pair(tmem, 512);
+    }
+    cluster_sync();
+}
 
 // ===================================================================
 // Persistent kernel for 128-dimensional heads.
@@ -1323,6 +1915,529 @@ k_rvq128(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int n_pairs)
 }
 
 // ===================================================================
+// 128-dimensional heads, two SMs per tile pair.
+//
+// k_rvq128's scheme (two tile slots whose MMAs and epilogues alternate, the
+// codebook streamed in pieces, helper warps on the second K block of every
+// residual update) on CTA pairs, with k_rvq64_pair's units and protocol: each
+// CTA holds half of every codebook piece (128 codewords x 64 dimensions, 16
+// KB), so the ring holds five pieces instead of two and L2 and the
+// shared-memory port carry half of the codebook traffic.  A piece's round trip
+// (its slot's MMAs done, the load asked for, landed and seen) takes about 2,900
+// cycles and its MMAs 880, so with four pieces the MMAs still waited 300 cycles
+// for each.  The input rows are taken whole lines at a time, eight loads in
+// flight, the first K block by the slot's warps and the second by the helpers.
+//
+// Llama-shaped cache, 4.19 M vectors of K (4 stages) and of V (2): 3.65 ms
+// against 3.98 for k_rvq128; 64 groups of 7 tiles in float32, 56 us against
+// 71.  A slot's stage is 6,300 cycles waiting for its MMAs (its own take
+// 3,300, the other slot's come between), 1,000 of argmin, 2,530 of update and
+// 1,900 of input; reading all 16 codeword rows of an update ahead spills and
+// was slower, two batches ahead of four is what 128 registers hold.
+namespace pr128 {
+constexpr int kRing = 5;
+constexpr int kWarps = 14;                   // 0 TMA, 1 MMA, 2..5 and 6..9 epilogue groups, 10..13 update helpers
+constexpr int kThreads = kWarps * 32;
+constexpr int kHalf = kCodes / 2;
+constexpr int A_KB = kRows * 128;            // 16 KB: 128 rows x 64 fp16 (128-byte swizzle)
+constexpr int A_HALF = 2 * A_KB;             // hi (or lo): both K blocks
+constexpr int A_SLOT = 2 * A_HALF;           // 64 KB
+constexpr int A_AUG = kRows * 32;            // 4 KB per slot
+constexpr int B_PIECE = kHalf * 128;         // 16 KB
+constexpr int B_AUG = kHalf * 32;            // 4 KB
+constexpr int OFF_AAUG = 2 * A_SLOT;
+constexpr int OFF_B = OFF_AAUG + 2 * A_AUG;
+constexpr int OFF_BAUG = OFF_B + kRing * B_PIECE;
+constexpr int OFF_BAR = OFF_BAUG + 2 * B_AUG;
+constexpr int BAR_FULL = 0, BAR_EMPTY = 5, BAR_READY = 10, BAR_READY_H = 12, BAR_ACC = 14, BAR_DRAIN = 16, BAR_HAND = 17,
+              BAR_MXE = 25, BAR_MXH = 33, BAR_IN = 41, kBars = 49;
+// per slot and row two words: chosen index | row shift << 8 (then the helper's
+// partial maximum), the slot's partial maximum
+constexpr int OFF_HX = OFF_BAR + 8 * 50;
+constexpr int OFF_IN = OFF_HX + 2 * kRows * 8;   // per slot and quadrant: what the helper's input half holds
+constexpr int OFF_SLOT = OFF_IN + 32;
+constexpr int OFF_LO = OFF_SLOT + 16;        // per slot: the round whose first-stage lo operand is nonzero (leader)
+constexpr int OFF_ABORT = OFF_LO + 16;
+constexpr int SMEM = OFF_ABORT + 16;
+constexpr int kLarge = 1, kInexact = 2;      // input halves: a value of 2^12 or more; a nonzero lo operand
+static_assert(OFF_B % 1024 == 0 && SMEM <= 232448, "shared memory");
+}  // namespace pr128
+
+template <int ESZ>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pr128::kThreads, 1)
+k_rvq128_pair(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_aug, const RvqArgs a,
+              int units_per_group, int n_units, FastDiv div_unit)
+{
+    using namespace pr128;
+    constexpr int D = 128;
+    constexpr int XC = D * ESZ / 16;             // 16-byte chunks per input row
+    extern __shared__ __align__(1024) uint8_t smem_1k[];     // no room for alignment slack
+    uint8_t *base = smem_1k;
+    const uint32_t sbase = smem_u32(base);
+    if (sbase & 1023u) {                         // never, by the declaration: nothing below may run then
+        if (threadIdx.x == 0)
+            atomicOr(a.status, FKV_ST_TIMEOUT);
+        return;
+    }
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(base + OFF_ABORT);
+    volatile int *lo_stamp = reinterpret_cast<volatile int *>(base + OFF_LO);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_rank();
+    auto bar = [&](int i) { return sbase + OFF_BAR + 8u * i; };
+    if (tid == 0) {
+        // a_ready, a_ready_h: a warp's lane each, both CTAs; hand, mx_e, mx_h, in: one warp
+        for (int i = 0; i < kBars; ++i)
+            mbar_init(bar(i), i >= BAR_HAND ? 32 : (i >= BAR_READY && i < BAR_ACC ? 8 : 1));
+        lo_stamp[0] = 0;
+        lo_stamp[1] = 0;
+        *abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&tmap);
+        prefetch_tmap(&tmap_aug);
+    }
+    if (warp == 1)
+        tmem_alloc_pair(sbase + OFF_SLOT, 512);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(base + OFF_SLOT);
+    const int S = a.S;
+    const int64_t nvec = a.batch * a.n_pos;
+    auto cgroup = [&](int g) { return a.pooled ? static_cast<int>(a.div_heads.div(static_cast<unsigned>(g))) : g; };
+    // the clusters take the units in turn, so that at any time they work on a few
+    // codebook groups, whose operands L2 then serves; in this cluster's own count
+    // (units 0 .. nu-1), slot k of round j takes unit 2 j + k
+    const int cid = blockIdx.x >> 1, nc = gridDim.x >> 1;
+    const int nu = (n_units - cid + nc - 1) / nc;
+    auto group_of = [&](int i) { return static_cast<int>(div_unit.div(static_cast<unsigned>(cid + i * nc))); };
+
+    // this row of a unit: its codebook group's head group, its input row and its
+    // record slot (null past the data)
+    struct Unit {
+        int g;
+        const uint4 *src;
+        uint8_t *dst;
+    };
+    auto unit_of = [&](int i, int row) {
+        const int u = cid + i * nc;
+        Unit w;
+        w.g = group_of(i);
+        const int64_t v = (static_cast<int64_t>(u - w.g * units_per_group) * 2 + rank) * kRows + row;
+        w.src = nullptr;
+        w.dst = nullptr;
+        if (v < nvec) {
+            const int l = static_cast<int>(a.div_heads.div(static_cast<unsigned>(w.g))), h = w.g - l * a.n_heads;
+            const int64_t b = vec_seq(a, v), t = v - b * a.n_pos;
+            w.src = reinterpret_cast<const uint4 *>(
+                static_cast<const uint8_t *>(a.x) +
+                (l * a.s_layer + b * a.s_batch + h * a.s_head + (a.t0 + t) * a.s_pos) * ESZ);
+            w.dst = static_cast<uint8_t *>(a.sym) + (b * a.n_layers + l) * a.stream_stride + (a.rec0 + t) * a.R +
+                    a.kv_off + h * S;
+        }
+        return w;
+    };
+
+    if (warp == 0) {
+        // ---------------------------------------------------- TMA producer (both CTAs)
+        if (lane == 0) {
+            // pieces of a slot's stage: q = 0 hi of K block 0 (with the norm
+            // operand, the two buffers in turn), 1 its lo, 2 hi of K block 1, 3 its lo
+            int b = 0, aug = 0;
+            uint32_t ph = 0, used[kRing] = {0, 0, 0, 0, 0};      // loads issued into each ring slot
+            bool ok = true;
+            for (int ur = 0; ur < nu && ok; ur += 2) {
+                for (int s = 0; s < S && ok; ++s) {
+                    for (int u = ur; u < min(ur + 2, nu) && ok; ++u) {
+                        const int gs = cgroup(group_of(u)) * S + s;
+                        for (int q = 0; q < 4; ++q) {
+                            if (!wait_or_abort(bar(BAR_EMPTY + b), ph ^ 1, a.status, abort_flag)) {
+                                ok = false;
+                                break;
+                            }
+                            const uint32_t full = map_cta(bar(BAR_FULL + b), 0);
+                            if (rank == 0)
+                                mbar_arrive_expect_tx(bar(BAR_FULL + b), 2u * (B_PIECE + (q == 0 ? B_AUG : 0)));
+                            tma_load_pair(sbase + OFF_B + b * B_PIECE, &tmap, (q >> 1) * 64,
+                                          gs * 2 * kCodes + (q & 1) * kCodes + static_cast<int>(rank) * kHalf, full);
+                            if (q == 0) {
+                                // free: the piece waited for above, five back, is past the
+                                // stage that used this buffer two stages ago
+                                tma_load_pair(sbase + OFF_BAUG + aug * B_AUG, &tmap_aug, 0,
+                                              gs * (kCodes / 4) + static_cast<int>(rank) * (kHalf / 4), full);
+                                aug ^= 1;
+                            }
+                            ++used[b];
+                            if (++b == kRing) {
+                                b = 0;
+                                ph ^= 1;
+                            }
+                        }
+                    }
+                }
+            }
+            // no copy may still be landing in shared memory when a CTA exits (as in
+            // k_rvq64_pair)
+            if (rank == 0) {
+                for (int i = 0; i < kRing; ++i)
+                    if (used[i])
+                        mbar_wait(bar(BAR_FULL + i), (used[i] - 1) & 1, a.status);
+            } else if (!ok) {
+                const uint64_t t0 = globaltimer_ns();
+                while (globaltimer_ns() - t0 < 2000000) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------------------------------------------- MMA issuer (leader)
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = idesc_f16_f32(2 * kRows, kCodes);
+            uint32_t ph = 0, aph = 0, hph = 0;            // parities of a_ready and a_ready_h per slot, bit k
+            int b = 0, aug = 0, pc = 0;
+            bool ok = true;
+            for (int ur = 0; ur < nu && ok; ur += 2) {
+                ++pc;
+                const int act = min(2, nu - ur);
+                for (int s = 0; s < S && ok; ++s) {
+                    for (int k = 0; k < act && ok; ++k) {
+                        for (int q = 0; q < 4; ++q) {
+                            if (q == 0) {
+                                ok = wait_cluster(bar(BAR_READY + k), (aph >> k) & 1, a.status, abort_flag);
+                                aph ^= 1u << k;
+                                if (ok && s > 0) {        // the helpers' half of the update
+                                    ok = wait_or_abort(bar(BAR_READY_H + k), (hph >> k) & 1, a.status, abort_flag);
+                                    hph ^= 1u << k;
+                                }
+                            }
+                            ok = ok && wait_or_abort(bar(BAR_FULL + b), ph, a.status, abort_flag);
+                            if (!ok)
+                                break;
+                            tc_fence_after();
+                            const bool lo = s > 0 || lo_stamp[k] == pc;
+                            const uint32_t bb = sbase + OFF_B + b * B_PIECE;
+                            const uint32_t ab = sbase + k * A_SLOT + (q >> 1) * A_KB;
+                            const uint32_t acc = tmem + k * 256;
+                            if (q == 0) {   // codeword norms first (K = 16, no swizzle)
+                                umma_f16_pair(acc, sdesc_core16(sbase + OFF_AAUG + k * A_AUG),
+                                              sdesc_core16(sbase + OFF_BAUG + aug * B_AUG), idesc, 0);
+                                aug ^= 1;
+                            }
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk) {
+                                const uint64_t db = sdesc_sw128(bb + kk * 32);
+                                umma_f16_pair(acc, sdesc_sw128(ab + kk * 32), db, idesc, 1);     // hi*hi or hi*lo
+                                if ((q & 1) == 0 && lo)
+                                    umma_f16_pair(acc, sdesc_sw128(ab + A_HALF + kk * 32), db, idesc, 1);   // lo*hi
+                            }
+                            if (q == 3)
+                                umma_commit_pair(bar(BAR_ACC + k));
+                            umma_commit_pair(bar(BAR_EMPTY + b));     // the ring slot is free once these MMAs are done
+                            if (++b == kRing) {
+                                b = 0;
+                                ph ^= 1;
+                            }
+                        }
+                    }
+                }
+            }
+            // every MMA has completed before tensor memory is released
+            umma_commit_pair(bar(BAR_DRAIN));
+            mbar_wait(bar(BAR_DRAIN), 0, a.status);
+        }
+    } else if (warp >= 10) {
+        // ---------------------------------------------------- update helpers
+        // warp 10 + i serves quadrant (10 + i) & 3 of both slots: the second K
+        // block (dimensions 64..127) of its 32 rows, of every unit's input and
+        // every update
+        const int quad = warp & 3;
+        const int row = quad * 32 + lane;
+        uint8_t *hx0 = base + OFF_HX;
+        const uint32_t ready = map_cta(bar(BAR_READY_H), 0);
+        uint32_t hp = 0, xp = 0;                  // parities per slot, bit k
+        bool ok = true;
+        for (int ur = 0; ur < nu && ok; ur += 2) {
+            const int act = min(2, nu - ur);
+            for (int k = 0; k < act; ++k) {
+                const Unit w = unit_of(ur + k, row);
+                const float se = pow2f(-__ldg(&a.escale_h[w.g * S]));
+                // the tile is free once the slot's last stage before has been multiplied
+                // (its update's hand-over, or the wait here a unit ago, came after the
+                // phase before that one)
+                ok = ur == 0 || wait_or_abort(bar(BAR_ACC + k), (static_cast<uint32_t>(ur >> 1) * S - 1) & 1, a.status,
+                                              abort_flag);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok)
+                    break;
+                uint8_t *ahi = base + k * A_SLOT + A_KB;
+                float mx = 0.0f;
+                uint32_t nz = 0;
+                load_rows64<ESZ>(ahi, ahi + A_HALF, quad, w.src ? w.src + XC / 2 : nullptr, a.dtype, se, mx, nz);
+                const int what = (__any_sync(0xFFFFFFFFu, !(mx < 4096.0f)) ? kLarge : 0) |
+                                 (__any_sync(0xFFFFFFFFu, nz != 0) ? kInexact : 0);
+                if (lane == 0)
+                    *reinterpret_cast<volatile int *>(base + OFF_IN + 4 * (4 * k + quad)) = what;
+                fence_proxy_async_smem();
+                mbar_arrive(bar(BAR_IN + 4 * k + quad));
+            }
+            for (int s = 0; s + 1 < S && ok; ++s) {
+                for (int k = 0; k < act; ++k) {
+                    const int g = group_of(ur + k);
+                    const int e = __ldg(&a.escale_h[g * S + s]), e_next = __ldg(&a.escale_h[g * S + s + 1]);
+                    ok = wait_or_abort(bar(BAR_HAND + 4 * k + quad), (hp >> k) & 1, a.status, abort_flag);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok)
+                        break;
+                    hp ^= 1u << k;
+                    uint32_t *hx = reinterpret_cast<uint32_t *>(hx0 + (k * kRows + row) * 8);
+                    const int bidx = static_cast<int>(hx[0] & 0xFFu);
+                    const int er = static_cast<int>(hx[0] >> 8);
+                    uint8_t *ahi = base + k * A_SLOT + A_KB;
+                    uint8_t *alo = ahi + A_HALF;
+                    const float f = -pow2f(-e - er);
+                    const float *cbs = a.cb32 + static_cast<int64_t>(cgroup(g) * S + s) * kCodes * D;
+                    if (e_next == e) {
+                        if (__all_sync(0xFFFFFFFFu, er == 0))
+                            update_rows_t<true>(ahi, alo, quad, cbs + 64, bidx, f);
+                        else
+                            update_rows_t<false>(ahi, alo, quad, cbs + 64, bidx, f);
+                    } else {
+                        const float4 *gc = reinterpret_cast<const float4 *>(cbs + bidx * D) + 16;
+                        float mx = 0.0f;
+#pragma unroll 2
+                        for (int c = 0; c < 8; ++c) {
+                            float t[8];
+                            load_add_chunk(ahi, alo, row, c, __ldg(gc + 2 * c), __ldg(gc + 2 * c + 1), f, t);
+#pragma unroll
+                            for (int i = 0; i < 8; i += 2)
+                                mx = max3f(mx, fabsf(t[i]), fabsf(t[i + 1]));
+                            store_chunk(ahi, alo, row, c, t);
+                        }
+                        // the row's maximum over both halves: exchange with the slot's warp
+                        hx[0] = __float_as_uint(mx);
+                        mbar_arrive(bar(BAR_MXH + 4 * k + quad));
+                        ok = wait_or_abort(bar(BAR_MXE + 4 * k + quad), (xp >> k) & 1, a.status, abort_flag);
+                        ok = __all_sync(0xFFFFFFFFu, ok);
+                        if (!ok)
+                            break;
+                        xp ^= 1u << k;
+                        mx = fmaxf(mx, __uint_as_float(hx[1]));
+                        int E = 0;
+                        if (mx > 0.0f)
+                            frexpf(mx, &E);
+                        const int tot = E + er + e - e_next;
+                        const int er2 = tot > v2::kRowLog ? tot - v2::kRowLog : 0;
+                        const float gsc = pow2f(er + e - e_next - er2);
+#pragma unroll 2
+                        for (int c = 0; c < 8; ++c) {
+                            float t[8];
+                            load_chunk(ahi, alo, row, c, t);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                t[i] *= gsc;
+                            store_chunk(ahi, alo, row, c, t);
+                        }
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0)
+                        arrive_cluster(ready + 8 * k);
+                }
+            }
+        }
+    } else {
+        // ---------------------------------------------------- epilogue groups
+        const int k = (warp - 2) >> 2;           // tile slot 0 or 1
+        const int quad = warp & 3;                // TMEM lane quadrant of this warp
+        const int row = quad * 32 + lane;
+        const uint32_t trow = tmem + k * 256 + (static_cast<uint32_t>(quad * 32) << 16);
+        uint8_t *ahi = base + k * A_SLOT;
+        uint8_t *alo = ahi + A_HALF;
+        uint8_t *aaug = base + OFF_AAUG + k * A_AUG;
+        const uint32_t ready = map_cta(bar(BAR_READY + k), 0);
+        const uint32_t lo_at = map_cta(sbase + OFF_LO + 4 * k, 0);
+        uint32_t fph = 0, xph = 0, iph = 0;
+        int pc = 0;
+        bool ok = true;
+        for (int u = k; u < nu && ok; u += 2) {
+            const Unit cur = unit_of(u, row);
+            const int g = cur.g;
+            const bool valid = cur.src != nullptr;
+            // the row's operand t = x 2^-(e + er), er >= 0 keeping |t| below 2^12
+            int e = __ldg(&a.escale_h[g * S]);
+            int er;
+            ++pc;
+            {
+                const uint4 *src = cur.src;
+                const float se = pow2f(-e);
+                float mx = 0.0f;
+                uint32_t nz = 0;
+                load_rows64<ESZ>(ahi, alo, quad, src, a.dtype, se, mx, nz);
+                // the helper's half
+                ok = wait_or_abort(bar(BAR_IN + 4 * k + quad), iph, a.status, abort_flag);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok)
+                    break;
+                iph ^= 1;
+                const int what = *reinterpret_cast<volatile int *>(base + OFF_IN + 4 * (4 * k + quad));
+                nz |= static_cast<uint32_t>(what & kInexact);
+                er = 0;
+                if (__any_sync(0xFFFFFFFFu, !(mx < 4096.0f) || (what & kLarge) != 0)) {
+                    // a row of larger magnitude (the usual case has none): its lane stores
+                    // it again, shifted
+                    __syncwarp();
+                    auto chunk = [&](int c, float *f) {
+                        uint4 x[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+                        if (valid) {
+                            x[0] = __ldg(src + c * (ESZ / 2));
+                            if (ESZ == 4)
+                                x[1] = __ldg(src + c * 2 + 1);
+                        }
+                        unpack8<ESZ>(x, a.dtype, 0, f);
+                    };
+                    float rm = 0.0f;
+#pragma unroll 1
+                    for (int c = 0; c < 16; ++c) {
+                        float f[8];
+                        chunk(c, f);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            rm = fmaxf(rm, fabsf(f[i] * se));
+                    }
+                    er = row_shift(rm);
+                    if (er != 0) {
+                        const float sr = pow2f(-er);
+#pragma unroll 1
+                        for (int c = 0; c < 16; ++c) {
+                            float f[8];
+                            chunk(c, f);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                f[i] = f[i] * se * sr;
+                            nz |= store_chunk(ahi + (c >> 3) * A_KB, alo + (c >> 3) * A_KB, row, c & 7, f);
+                        }
+                    }
+                }
+                write_aug_row(aaug, row, er);
+                const bool lo = __any_sync(0xFFFFFFFFu, nz != 0);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    if (lo) {
+                        store_cluster(lo_at, pc);
+                        arrive_cluster<true>(ready);
+                    } else {
+                        arrive_cluster(ready);
+                    }
+                }
+            }
+            if (u + 2 < nu) {
+                // the slot's next input row into L2 while this unit runs
+                const Unit nxt = unit_of(u + 2, row);
+                if (nxt.src)
+#pragma unroll
+                    for (int c = 0; c < XC; c += 8)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt.src + c));
+            }
+            uint64_t idx = 0;
+            for (int s = 0; s < S; ++s) {
+                const int e_next = s + 1 < S ? __ldg(&a.escale_h[g * S + s + 1]) : e;
+                ok = wait_or_abort(bar(BAR_ACC + k), fph, a.status, abort_flag);
+                // the tensor-memory loads below are warp-collective: the warp
+                // goes on, or leaves, as one
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok)
+                    break;
+                fph ^= 1;
+                tc_fence_after();
+                bool amb;
+                float vu;
+                int bidx = argmin_row4(trow, &amb, &vu);
+                if (__any_sync(0xFFFFFFFFu, amb)) {   // warp-collective loads: every lane takes part
+                    const int jj = exact_argmin_tmem(trow);
+                    if (amb)
+                        bidx = jj;
+                }
+                tc_fence_before();
+                idx |= static_cast<uint64_t>(bidx) << (8 * s);
+                if (s + 1 < S) {
+                    // t <- t - c 2^(-e-er) (t is the row in units of 2^-(e+er)),
+                    // c the chosen codeword's float32 row; this warp takes the first
+                    // K block, the quadrant's helper the second
+                    uint32_t *hx = reinterpret_cast<uint32_t *>(base + OFF_HX + (k * kRows + row) * 8);
+                    hx[0] = static_cast<uint32_t>(bidx) | (static_cast<uint32_t>(er) << 8);
+                    mbar_arrive(bar(BAR_HAND + 4 * k + quad));
+                    const float f = -pow2f(-e - er);
+                    const float *cbs = a.cb32 + static_cast<int64_t>(cgroup(g) * S + s) * kCodes * D;
+                    if (e_next == e) {
+                        if (__all_sync(0xFFFFFFFFu, er == 0))
+                            update_rows_t<true>(ahi, alo, quad, cbs, bidx, f);
+                        else
+                            update_rows_t<false>(ahi, alo, quad, cbs, bidx, f);
+                    } else {
+                        const float4 *gc = reinterpret_cast<const float4 *>(cbs + bidx * D);
+                        float mx = 0.0f;
+#pragma unroll 2
+                        for (int c = 0; c < 8; ++c) {
+                            float t[8];
+                            load_add_chunk(ahi, alo, row, c, __ldg(gc + 2 * c), __ldg(gc + 2 * c + 1), f, t);
+#pragma unroll
+                            for (int i = 0; i < 8; i += 2)
+                                mx = max3f(mx, fabsf(t[i]), fabsf(t[i + 1]));
+                            store_chunk(ahi, alo, row, c, t);
+                        }
+                        // the row's maximum over both halves: exchange with the helper
+                        hx[1] = __float_as_uint(mx);
+                        mbar_arrive(bar(BAR_MXE + 4 * k + quad));
+                        ok = wait_or_abort(bar(BAR_MXH + 4 * k + quad), xph, a.status, abort_flag);
+                        ok = __all_sync(0xFFFFFFFFu, ok);
+                        if (!ok)
+                            break;
+                        xph ^= 1;
+                        mx = fmaxf(mx, __uint_as_float(hx[0]));
+                        int E = 0;
+                        if (mx > 0.0f)
+                            frexpf(mx, &E);
+                        const int tot = E + er + e - e_next;
+                        const int er2 = tot > v2::kRowLog ? tot - v2::kRowLog : 0;
+                        const float gsc = pow2f(er + e - e_next - er2);
+#pragma unroll 2
+                        for (int c = 0; c < 8; ++c) {
+                            float t[8];
+                            load_chunk(ahi, alo, row, c, t);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                t[i] *= gsc;
+                            store_chunk(ahi, alo, row, c, t);
+                        }
+                        er = er2;
+                        write_aug_row(aaug, row, er);
+                    }
+                    e = e_next;
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0)
+                        arrive_cluster(ready);
+                }
+            }
+            if (!ok)
+                break;
+            if (valid)
+                store_indices(cur.dst, idx, S);
+        }
+    }
+    // neither CTA leaves, or gives tensor memory back, while the other may still
+    // arrive on its barriers or read its shared memory
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    if (warp == 1) {
+        __syncwarp();
+        tmem_dealloc_pair(tmem, 512);
+    }
+    cluster_sync();
+}
+
+// ===================================================================
 // The failure path of the kernels above, on barriers that never complete.
 // Warp 1 holds TMEM as the MMA warp does; warp 0's lane 0 waits on bar 0,
 // which nothing arrives on, gives up after limit_ns and raises the abort
@@ -1395,6 +2510,30 @@ cudaError_t launch_rvq64(const CUtensorMap &tmap, const RvqArgs &a, int ppg, int
     return cudaGetLastError();
 }
 
+// Whether a group of `tiles` tiles runs on CTA pairs.  A pair takes its tiles
+// from one group, so an odd count leaves half of the group's last unit empty:
+// from five tiles on that costs less than the pair gains, and it costs nothing
+// while every unit has a cluster to itself.  Otherwise (one tile a group is a
+// decode step's append) each SM takes its own tiles.  Measured, old and pair:
+// 64 groups of 1 tile of 128-dimensional heads 49.7 / 39.7 us for K and V, 256
+// groups 78.8 / 98.8; 144 groups of 3 tiles of 64-dimensional heads 53.1 / 64.3.
+bool pair_tiles(int64_t tiles, int64_t groups, int sms)
+{
+    return tiles % 2 == 0 || tiles >= 5 || groups * ((tiles + 1) / 2) <= sms / 2;
+}
+
+template <int ESZ, int NB>
+cudaError_t launch_rvq64_pair(const fkv_cbset &cb, const RvqArgs &a, int upg, int n_units, unsigned clusters,
+                              cudaStream_t st)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_rvq64_pair<ESZ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, pr::SMEM);
+    if (e != cudaSuccess)
+        return e;
+    k_rvq64_pair<ESZ, NB><<<2 * clusters, pr::kThreads, pr::SMEM, st>>>(cb.tmap_half, cb.tmap_aug, a, upg, n_units,
+                                                                   FastDiv::make(static_cast<unsigned>(upg)));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int64_t t0, int64_t t1,
                               void *sym, int64_t stream_stride, int64_t rec0, cudaStream_t st)
 {
@@ -1428,6 +2567,9 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
     const int64_t nvec = a.batch * a.n_pos;
     if (nvec <= 0)
         return cudaSuccess;
+    a.small = nvec <= 0x7FFFFFFF;
+    a.div_pos = FastDiv::make(a.small ? static_cast<unsigned>(a.n_pos) : 1u);
+    a.div_heads = FastDiv::make(static_cast<unsigned>(a.n_heads));
     const int64_t tiles = (nvec + kRows - 1) / kRows;
     const int64_t blocks = tiles * c->Ly * c->H;
     if (tiles > 0x7FFFFFFF || blocks > 0x7FFFFFFF)
@@ -1444,6 +2586,15 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
             return e;
         const unsigned grid = static_cast<unsigned>(n_pairs < sms ? n_pairs : sms);
         const int pp = static_cast<int>(ppg), np = static_cast<int>(n_pairs);
+        if (pair_tiles(tiles, c->Ly * c->H, sms)) {
+            const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
+            const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
+            if (c->KC == 1024)
+                return x->dtype == FKV_F32 ? launch_rvq64_pair<4, 4>(cb, a, upg, nu, clusters, st)
+                                           : launch_rvq64_pair<2, 4>(cb, a, upg, nu, clusters, st);
+            return x->dtype == FKV_F32 ? launch_rvq64_pair<4, 1>(cb, a, upg, nu, clusters, st)
+                                       : launch_rvq64_pair<2, 1>(cb, a, upg, nu, clusters, st);
+        }
         if (c->KC == 1024)
             return x->dtype == FKV_F32 ? launch_rvq64<4, 4>(cb.tmap, a, pp, np, grid, st)
                                        : launch_rvq64<2, 4>(cb.tmap, a, pp, np, grid, st);
@@ -1459,6 +2610,17 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
         if (e != cudaSuccess)
             return e;
+        if (pair_tiles(tiles, c->Ly * c->H, sms)) {
+            const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
+            const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
+            const auto kern = x->dtype == FKV_F32 ? k_rvq128_pair<4> : k_rvq128_pair<2>;
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pr128::SMEM);
+            if (e != cudaSuccess)
+                return e;
+            kern<<<2 * clusters, pr128::kThreads, pr128::SMEM, st>>>(cb.tmap_half, cb.tmap_aug, a, upg, nu,
+                                                                     FastDiv::make(static_cast<unsigned>(upg)));
+            return cudaGetLastError();
+        }
         const unsigned grid = static_cast<unsigned>(n_pairs < sms ? n_pairs : sms);
         const int np = static_cast<int>(n_pairs);
         if (x->dtype == FKV_F32) {

@@ -330,3 +330,16 @@ def test_config3_full_size_sampled(fkv, oracle_mod):
     ctx, sym, K, V = _sampled_check(fkv, oracle_mod, synth.CFG3, 3000)
     del K, V, sym
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("base", [1, 3])
+@pytest.mark.parametrize("layers,positions", [(1, 1), (1, 129), (1, 257), (1, 700), (8, 1), (8, 127), (8, 300), (8, 513)])
+def test_tile_counts_of_paired_and_single_tiles(fkv, oracle_mod, base, layers, positions):
+    """Tiles of 128 vectors per head group around the kernels' edges (1, 2, 3, 5
+    and 6 tiles, full and not) with few groups and with more groups than CTA
+    pairs, so that both the paired kernels and the one-tile ones run: every
+    index against the oracle."""
+    b = {1: synth.CFG1, 3: synth.CFG3}[base]
+    cfg = synth.small_config(b, 4000 + 100 * base + layers + positions, n_layers=layers, batch=1, seq=36 + positions,
+                             n_heads=11)
+    check_config_full(fkv, oracle_mod, cfg)
