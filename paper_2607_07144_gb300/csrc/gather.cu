@@ -351,21 +351,34 @@ __host__ __device__ inline int read_tables_bytes(int N, int L)
 // warps + warp, + gridDim.x * warps, ...  Three blocks per SM (80 registers,
 // a few spilled to L1) beat two without spills: 1.12 against 1.20 ms for
 // 262,144 Llama-shaped records.
-template <typename Sym>
+//
+// BLOCK: a whole block per request instead, its threads sharing the spans and
+// the dimension groups, for the few requests of one retrieval, which a warp
+// each would leave on a few SMs with a long serial tail: 96 GPT-2-shaped
+// records 5.9 us against 9.1.
+template <typename Sym, bool BLOCK>
 __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a)
 {
     extern __shared__ __align__(16) uint8_t dsm[];
     const fkvdec::Tables t = fkvdec::load(a.dec, a.T, a.N, a.L, dsm);
     Sym *srec = reinterpret_cast<Sym *>(dsm + read_tables_bytes(a.N, a.L));
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kTeam = BLOCK ? kReadWarps * 32 : 32;      // threads on one request
+    const int warp = BLOCK ? 0 : threadIdx.x >> 5, lane = threadIdx.x & (kTeam - 1);
+    constexpr int kTeams = BLOCK ? 1 : kReadWarps;
+    auto team_sync = [] {
+        if (BLOCK)
+            __syncthreads();
+        else
+            __syncwarp();
+    };
     const int H = a.n_heads, D = a.D, R = a.R, L = a.L;
     const int64_t out_vec = static_cast<int64_t>(2) * H * D;
     const int gsh = D == 128 ? 4 : 3;             // log2 of the 8-dimension groups per head
     const int items = 2 * H << gsh;
     Sym *my = srec + warp * kMaxRecord;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kReadWarps + warp; i < a.n_req;
-         i += static_cast<int64_t>(gridDim.x) * kReadWarps) {
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kTeams + warp; i < a.n_req;
+         i += static_cast<int64_t>(gridDim.x) * kTeams) {
         int64_t q = i, st, rec;
         if (a.order) {
             const int4 e = a.order[i];
@@ -377,7 +390,7 @@ __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a
             rec = a.req[2 * q + 1];
         }
         if (st < 0 || st >= a.n_streams || rec < 0 || rec >= a.n_rec) {
-            for (int64_t i = lane; i < out_vec / 2; i += 32)
+            for (int64_t i = lane; i < out_vec / 2; i += kTeam)
                 store2(a.out, a.dtype, q * out_vec + 2 * i, 0.0f, 0.0f);
             if (lane == 0)
                 atomicOr(a.status, FKV_ST_RANGE);
@@ -387,7 +400,7 @@ __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a
         const int64_t sym0 = rec * R;
         const int64_t u0 = sym0 / L, u1 = (sym0 + R - 1) / L;
         bool bad = false;
-        for (int64_t u = u0 + lane; u <= u1; u += 32) {
+        for (int64_t u = u0 + lane; u <= u1; u += kTeam) {
             const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
             const int last = static_cast<int>(u * L - sym0) + m - 1;
             bad |= !fkvdec::decode_point(t, a.pts[st * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
@@ -400,10 +413,10 @@ __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a
         }
         if (bad)
             atomicOr(a.status, FKV_ST_CORRUPT);
-        __syncwarp();
+        team_sync();
         const int l = static_cast<int>(st % a.n_layers);
 #pragma unroll 2
-        for (int g = lane; g < items; g += 32) {
+        for (int g = lane; g < items; g += kTeam) {
             const int kv = g >= (H << gsh) ? 1 : 0;
             const int gi = kv ? g - (H << gsh) : g;
             const int hh = gi >> gsh, d0 = (gi - (hh << gsh)) * 8;
@@ -440,7 +453,7 @@ __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a
             }
             store8(a.out, a.dtype, q * out_vec + (static_cast<int64_t>(kv) * H + hh) * D + d0, x, y);
         }
-        __syncwarp();                             // the next request reuses `my`
+        team_sync();                              // the next request reuses `my`
     }
 }
 
@@ -695,6 +708,16 @@ __global__ void __launch_bounds__(256) k_order_scatter(const int64_t *__restrict
 // L2 one request per warp.
 constexpr int64_t kStagedPerLayer = 512;
 
+// Up to this many requests (a warp each, about what is resident at once: three
+// blocks of eight warps on each of 152 SMs) run together, so that grouping
+// them by layer changes nothing but costs four launches: 96 records 10.2 us
+// without them and with a block each, 23.7 before.
+constexpr int64_t kUnordered = 3648;
+
+// Up to this many requests (a block each, resident at once) a request gets a
+// block of its own.
+constexpr int64_t kBlockEach = 456;
+
 static bool read_staged(const fkv_ctx *c, int64_t n_req)
 {
     return n_req >= kStagedPerLayer * c->Ly;
@@ -714,7 +737,7 @@ int64_t read_order_ints(const fkv_ctx *c, int64_t n_req)
     if (n_req <= 0 || n_req > 0x7FFFFFFF || 2 * (c->Ly + 1) > 12 * 1024)
         return 0;
     if (!read_staged(c, n_req))
-        return 4 * n_req + c->Ly + 1;
+        return n_req <= kUnordered ? 0 : 4 * n_req + c->Ly + 1;
     const int64_t R = static_cast<int64_t>(c->H) * (c->cb[0].stages + c->cb[1].stages);
     const int64_t esz = c->KC == 256 ? 1 : 2;
     return read_scr_ints(c, n_req) + (n_req * R * esz + 3) / 4;
@@ -823,8 +846,11 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
         return cudaSuccess;
     const int esz = c->KC == 256 ? 1 : 2;
     const int smem = read_tables_bytes(a.N, a.L) + kReadWarps * kMaxRecord * esz;
-    const void *kern = esz == 1 ? reinterpret_cast<const void *>(k_read_kv<uint8_t>)
-                                : reinterpret_cast<const void *>(k_read_kv<uint16_t>);
+    const bool block = n_req <= kBlockEach;
+    const void *kern = esz == 1 ? (block ? reinterpret_cast<const void *>(k_read_kv<uint8_t, true>)
+                                         : reinterpret_cast<const void *>(k_read_kv<uint8_t, false>))
+                                : (block ? reinterpret_cast<const void *>(k_read_kv<uint16_t, true>)
+                                         : reinterpret_cast<const void *>(k_read_kv<uint16_t, false>));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess)
         return e;
@@ -856,7 +882,7 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kReadWarps * 32, smem);
     if (e != cudaSuccess)
         return e;
-    int64_t blocks = (n_req + kReadWarps - 1) / kReadWarps;
+    int64_t blocks = block ? n_req : (n_req + kReadWarps - 1) / kReadWarps;
     const int64_t resident = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
     if (blocks > resident)
         blocks = resident;
