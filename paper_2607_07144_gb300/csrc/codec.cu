@@ -272,6 +272,32 @@ k_span_encode(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, int64_
     }
 }
 
+// The same for many short streams (a decode step's append): the threads count
+// through all streams' spans, so that a block, its table load and its warps
+// serve as many spans as it has threads, and read their symbols in place.
+// 2,048 streams of 48 symbols: 4.8 us, 8.4 with a block (and its table load) a
+// stream; from half a block's spans on, a block a stream loses little.
+template <bool HALF, typename Sym>
+__global__ void __launch_bounds__(kThreads)
+k_span_encode_flat(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, unsigned spans, unsigned total,
+                   fkvd::FastDiv div_spans, double2 *__restrict__ pts, int64_t pt_stride, const EncArgs a,
+                   unsigned *status)
+{
+    __shared__ double2 sV[enc_table_len<HALF, Sym>()];
+    load_vertices<HALF>(sV, a);
+    __syncthreads();
+    const unsigned t = blockIdx.x * kThreads + threadIdx.x;
+    if (t >= total)
+        return;
+    const unsigned stream = div_spans.div(t), s = t - stream * spans;
+    const int64_t b = static_cast<int64_t>(s) * a.L;
+    const int m = static_cast<int>(min(static_cast<int64_t>(a.L), n - b));
+    const double2 p = encode_anchored<HALF>(sym + stream * sym_stride + b, m, sV, a, RatioMul(a.r));
+    if (isnan(p.x))   // a symbol >= N
+        atomicOr(status, FKV_ST_CORRUPT);
+    pts[stream * pt_stride + s] = p;
+}
+
 // ------------------------------------------------------------- decoding
 // (arithmetic in decode_core.cuh: exact Q1.62 walk, no division)
 
@@ -1121,6 +1147,15 @@ cudaError_t span_encode_t(const fkv_ctx *c, const Sym *sym, int64_t n_streams, i
         return cudaSuccess;
     if (blocks > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
+    // streams of at most half a block's spans share blocks
+    if (spans <= kThreads / 2 && n_streams * spans <= 0x7FFFFFFF) {
+        const auto flat = c->r == 0.5 ? k_span_encode_flat<true, Sym> : k_span_encode_flat<false, Sym>;
+        const unsigned total = static_cast<unsigned>(n_streams * spans);
+        flat<<<(total + kThreads - 1) / kThreads, kThreads, 0, st>>>(
+            sym, n, sym_stride, static_cast<unsigned>(spans), total, fkvd::FastDiv::make(static_cast<unsigned>(spans)),
+            reinterpret_cast<double2 *>(pts), pt_stride, enc_args(c), c->d_status);
+        return cudaGetLastError();
+    }
     const auto kern = c->r == 0.5 ? k_span_encode<true, Sym> : k_span_encode<false, Sym>;
     kern<<<static_cast<unsigned>(blocks), kThreads, 0, st>>>(sym, n, sym_stride, spans, static_cast<int>(bps),
                                                              reinterpret_cast<double2 *>(pts), pt_stride, enc_args(c),
