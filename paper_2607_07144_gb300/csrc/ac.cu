@@ -21,8 +21,9 @@
 //
 // Measured at 96 streams of 17,784 symbols (N = 256, adaptive, one GB300):
 // encode 1.38 ms (160 cycles a symbol; 19.8 ms with divisions, bit loops and
-// the model on the chain), decode 4.37 ms (500 cycles; 26.9 ms).  Testing a
-// lane's eight symbols at once instead of by halves takes fewer dependent
+// the model on the chain), decode 3.96 ms (450 cycles; 26.9 ms; 4.37 with the
+// code words and reciprocals by shuffle and the bits in two branches).  Testing
+// a lane's eight symbols at once instead of by halves takes fewer dependent
 // steps but more instructions, and one warp issues too few: 4.85 ms.
 #include "fkv_internal.h"
 
@@ -255,17 +256,22 @@ k_ac_encode(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, int N, i
 // with floor(w cum / T) <= val - lo, which is w cum <= (val - lo + 1) T - 1
 // without a division: every lane tests its first symbol (the owner is the last
 // lane that passes) and, at the same time, searches its own symbols by halves
-// and works out the interval of the one it finds (the quotients by T from a
-// reciprocal that lane k of the batch prepared for the batch's symbol k); the
-// owner's interval and symbol then come by shuffle.  The bits to come sit in a
-// 64-bit window refilled without a branch; the code words are fetched 32 at a
-// time, one batch ahead.
-template <typename Sym, int CPL>
+// and works out the interval of the one it finds (the quotients by T from
+// reciprocals prepared 32 symbols at a time); the owner's interval and symbol
+// then come by shuffle.  The bits to come sit in a 64-bit window refilled
+// without a branch from 64 code words in shared memory, of which 32 symbols
+// use at most 32 (SMALL: N + n < 2^28, so that a symbol settles fewer than 32
+// bits: an interval of 2^30 or more leaves at least 4, which doubles at most
+// 30 times).  Larger counts take a symbol's bits in two steps.
+template <typename Sym, int CPL, bool SMALL>
 __global__ void __launch_bounds__(32)
 k_ac_decode(const uint32_t *__restrict__ words, int64_t word_stride, const int64_t *__restrict__ nbits, int64_t n,
             int N, int adaptive, Sym *__restrict__ sym, int64_t sym_stride, unsigned *status)
 {
     constexpr unsigned kAll = 0xFFFFFFFFu;
+    constexpr int kWords = SMALL ? 64 : 128;      // a batch of 32 symbols uses at most half
+    __shared__ uint32_t code[kWords];
+    __shared__ unsigned long long recip[32];
     const int lane = threadIdx.x;
     const int64_t stream = blockIdx.x;
     const uint32_t *in = words + stream * word_stride;
@@ -284,41 +290,50 @@ k_ac_decode(const uint32_t *__restrict__ words, int64_t word_stride, const int64
         const uint32_t w = __ldg(in + q);
         return left >= 32 ? w : w & (0xFFFFFFFFu << (32 - static_cast<int>(left)));
     };
-    int64_t wq = lane;                            // this lane's word of the batch after next
-    uint32_t cur = word_at(wq), ahead = word_at(wq + 32);
-    wq += 64;
+    // code[] holds words base .. base + kWords - 1 (word q at q mod kWords), the
+    // 32 after them are on their way in `ahead`
+    for (int i = lane; i < kWords; i += 32)
+        code[i] = word_at(i);
+    int64_t wq = kWords + lane;
+    uint32_t ahead = word_at(wq);
+    __syncwarp();
     uint32_t cum[CPL + 1];                        // counts below symbols lane CPL + j
 #pragma unroll
     for (int j = 0; j <= CPL; ++j)
         cum[j] = min(lane * CPL + j, N);
-    uint32_t lo = 0, hi = 0xFFFFFFFFu, val = __shfl_sync(kAll, cur, 0);
-    unsigned long long win = static_cast<unsigned long long>(__shfl_sync(kAll, cur, 1)) << 32;  // bits to come
+    uint32_t lo = 0, hi = 0xFFFFFFFFu, val = code[0];
+    unsigned long long win = static_cast<unsigned long long>(code[1]) << 32;   // bits to come
     int have = 32;                                // of them valid, from the top: at least 32 between uses
-    int taken = 2;                                // words of cur already in the window
+    unsigned taken = 2;                           // words already in the window
+    unsigned loaded = kWords;                     // words that code[] has held
     auto use = [&](int len) {                     // drop len <= 32 bits
-        const uint32_t w = __shfl_sync(kAll, cur, taken);
+        const uint32_t w = code[taken & (kWords - 1)];
         win <<= len;
         have -= len;
         const bool refill = have < 32;
         win |= refill ? static_cast<unsigned long long>(w) << (32 - have) : 0ull;
         have += refill ? 32 : 0;
-        taken += refill ? 1 : 0;
-        if (taken == 32) {
-            taken = 0;
-            cur = ahead;
-            ahead = word_at(wq);
-            wq += 32;
-        }
+        taken += refill ? 1u : 0u;
     };
     uint32_t T = N;
-    unsigned long long Mb = 0xFFFFFFFFFFFFFFFFull / T;
+    unsigned long long M = 0xFFFFFFFFFFFFFFFFull / T;
     for (int64_t k0 = 0; k0 < n; k0 += 32) {
         const int len = static_cast<int>(min(static_cast<int64_t>(32), n - k0));
+        __syncwarp();
         if (adaptive)
-            Mb = 0xFFFFFFFFFFFFFFFFull / (T + lane);
+            recip[lane] = 0xFFFFFFFFFFFFFFFFull / (T + lane);
+        // keep half of code[] ahead of the window
+        while (loaded - taken <= kWords - 32) {
+            code[(loaded + lane) & (kWords - 1)] = ahead;
+            loaded += 32;
+            wq += 32;
+            ahead = word_at(wq);
+        }
+        __syncwarp();
         uint32_t pending = 0;
         for (int k = 0; k < len; ++k) {
-            const unsigned long long M = adaptive ? __shfl_sync(kAll, Mb, k) : Mb;
+            if (adaptive)
+                M = recip[k];
             const uint32_t d = hi - lo, v = val - lo;
             const unsigned long long R = static_cast<unsigned long long>(v) * T + (T - 1);
             auto passes = [&](uint32_t x) { return static_cast<unsigned long long>(d) * x + x <= R; };
@@ -355,10 +370,9 @@ k_ac_decode(const uint32_t *__restrict__ words, int64_t word_stride, const int64
             const int e = straddles(lo, hi);
             lo = (lo << e) & 0x7FFFFFFFu;
             hi = shl_in(hi, 0xFFFFFFFFu, e) | 0x80000000u;
-            const int sh = s + e;
-            if (sh <= 32) {
-                val = shl_in(val, static_cast<uint32_t>(win >> 32), sh);
-                use(sh);
+            if (SMALL) {
+                val = shl_in(val, static_cast<uint32_t>(win >> 32), s + e);
+                use(s + e);
             } else {
                 val = shl_in(val, static_cast<uint32_t>(win >> 32), s);
                 use(s);
@@ -400,8 +414,10 @@ cudaError_t ac_decode_t(const fkv_ctx *c, const uint32_t *words, int64_t word_st
 {
     if (n_streams > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
-    k_ac_decode<Sym, kPerLane<Sym>><<<static_cast<unsigned>(n_streams), 32, 0, st>>>(
-        words, word_stride, nbits, n, c->N, adaptive, sym, sym_stride, c->d_status);
+    const auto kern = n + c->N < (int64_t(1) << 28) ? k_ac_decode<Sym, kPerLane<Sym>, true>
+                                                    : k_ac_decode<Sym, kPerLane<Sym>, false>;
+    kern<<<static_cast<unsigned>(n_streams), 32, 0, st>>>(words, word_stride, nbits, n, c->N, adaptive, sym, sym_stride,
+                                                          c->d_status);
     return cudaGetLastError();
 }
 
