@@ -4,13 +4,15 @@
 // the nearest codeword of its (layer, head or pooled layer, K/V, stage)
 // codebook, the residual dropping the chosen codeword after each stage.
 //
-// Two persistent, warp-specialised kernels, one CTA per SM: k_rvq64 for
-// 64-dimensional heads (256 or 1024 codewords per stage) and k_rvq128 for
-// 128-dimensional heads (256).  Warp 0 streams the stage codebook by TMA, warp
-// 1 issues tcgen05.mma (M = 128, N = 256, K = 16) into fp32 accumulators in
-// tensor memory, and two 4-warp epilogue groups each walk one 128-vector tile
-// through the stages: exact argmin read out of tensor memory with
-// tcgen05.ld.red, then the residual update in the fp16 hi/lo operand tiles.
+// Persistent, warp-specialised kernels, one CTA per SM, for 64-dimensional
+// heads (256 or 1024 codewords per stage) and 128-dimensional ones (256): warp
+// 0 streams the stage codebook by TMA, warp 1 issues tcgen05.mma (N = 256, K =
+// 16) into fp32 accumulators in tensor memory, and 4-warp epilogue groups each
+// walk one 128-vector tile through the stages: exact argmin read out of tensor
+// memory with tcgen05.ld.red, then the residual update in the fp16 hi/lo
+// operand tiles.  k_rvq64_pair and k_rvq128_pair run on CTA pairs (M = 256);
+// k_rvq64 and k_rvq128 (M = 128) take the shapes whose tiles do not pair up
+// (pair_tiles), a decode step's append above all.
 #include <type_traits>
 
 #include "fkv_internal.h"
@@ -871,12 +873,14 @@ k_rvq64(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int pairs_per
 //
 // GPT-2-shaped cache, 1,138,176 vectors of K (4 stages) and of V (2): 486 us
 // against 633 for k_rvq64, and with 1024-codeword codebooks 1,013 against
-// 1,192 (85 % of the time the 13 MMAs of a block take alone).  At four stages a
+// 1,192 (1,960 cycles a block, of which its 13 MMAs take 1,664).  At four stages a
 // slot's round is 1,560 cycles of input, 3,200 waiting for its MMAs, 1,270 of
 // argmin and 2/3 x 2,600 of update: instruction issue and L2 latency of the
-// epilogue, not the tensor pipe, still bound it.  Cluster-scope releases on
-// every arrival cost 572 us, contiguous unit ranges per cluster 538 (their
-// codebooks spread over all groups), the argmin's two-load pipelining 613.
+// epilogue, not the tensor pipe, still bound it.  On the way: 689 us with
+// cluster-scope releases on every arrival and rows loaded lane by lane, 551
+// without; 613 with the argmin's loads pipelined by two (more registers), 538
+// with its three-input minima; 476 with the units strided over the clusters
+// instead of a contiguous range each (whose codebooks spread over all groups).
 namespace pr {
 constexpr int kSlots = 3;
 constexpr int kBufs = 3;
