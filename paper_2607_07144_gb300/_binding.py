@@ -105,19 +105,23 @@ def lib():
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():
+        # the handle alone: building a Stream object takes 3 us of a call's 15
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t: torch.Tensor):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _rows(t: torch.Tensor, unit: int = 1) -> int:
     """Row stride of a [rows, ...] tensor in units of `unit` elements; a
     single row has no meaningful stride, so report its own extent."""
     if t.shape[0] <= 1:
-        return max(1, t[0].numel() // unit if t.shape[0] else 1)
+        return max(1, t.numel() // unit)
     return t.stride(0) // unit
 
 
@@ -142,16 +146,11 @@ def cache_view(t: torch.Tensor, host: bool = False) -> _Cache:
     """fkv_cache view of a tensor shaped [n_layers, batch, n_heads, seq, dim]
     (any strides with a contiguous last dimension): a CUDA tensor, or with
     host=True a CPU tensor (pinned for full transfer speed)."""
-    if t.dim() != 5 or t.stride(4) != 1 or t.is_cuda == host:
+    st = t.stride()
+    if len(st) != 5 or st[4] != 1 or t.is_cuda == host:
         raise ValueError("cache must be a %s tensor [layers, batch, heads, seq, dim] with contiguous dim"
                          % ("CPU" if host else "CUDA"))
-    c = _Cache()
-    c.data = t.data_ptr()
-    c.dtype = _DTYPE[t.dtype]
-    c.batch = t.shape[1]
-    c.seq = t.shape[3]
-    c.stride_layer, c.stride_batch, c.stride_head, c.stride_pos = t.stride(0), t.stride(1), t.stride(2), t.stride(3)
-    return c
+    return _Cache(t.data_ptr(), _DTYPE[t.dtype], t.shape[1], t.shape[3], st[0], st[1], st[2], st[3])
 
 
 class Context:

@@ -1176,14 +1176,11 @@ cudaError_t launch_span_encode(const fkv_ctx *c, const void *sym, int64_t n_stre
 cudaError_t decode_grid(const fkv_ctx *c, const void *kern, int smem, int64_t n_chunks, unsigned *grid,
                         int threads = kThreads)
 {
-    int sms = 0, per_sm = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    int per_sm = 0;
+    const cudaError_t e = kernel_use(c, kern, threads, smem, &per_sm);
     if (e != cudaSuccess)
         return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-    if (e != cudaSuccess)
-        return e;
-    int64_t g = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
+    int64_t g = static_cast<int64_t>(c->sms) * (per_sm > 0 ? per_sm : 1);
     if (g > n_chunks)
         g = n_chunks;
     *grid = static_cast<unsigned>(g);
@@ -1207,11 +1204,8 @@ cudaError_t span_decode_t(const fkv_ctx *c, const double *pts, int64_t n_streams
     const void *kern = direct ? reinterpret_cast<const void *>(k_span_decode<Sym>)
                               : reinterpret_cast<const void *>(k_span_decode_staged<Sym>);
     const int smem = tables_bytes(c->N, c->L) + (direct ? 0 : dec_stage_bytes<Sym>(c->L));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     unsigned grid = 0;
-    e = decode_grid(c, kern, smem, n_chunks, &grid, TPB);
+    cudaError_t e = decode_grid(c, kern, smem, n_chunks, &grid, TPB);
     if (e != cudaSuccess)
         return e;
     const double2 *p2 = reinterpret_cast<const double2 *>(pts);
@@ -1250,12 +1244,8 @@ cudaError_t span_decode_planar_t(const fkv_ctx *c, const double *pts, int64_t n_
     if (n > 0x7FFFFFFF || n_chunks > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
     const int smem = tables_bytes(c->N, c->L) + R * static_cast<int>(sizeof(unsigned));
-    cudaError_t e = cudaFuncSetAttribute(k_span_decode_planar<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
-    if (e != cudaSuccess)
-        return e;
     unsigned grid = 0;
-    e = decode_grid(c, reinterpret_cast<const void *>(k_span_decode_planar<Sym>), smem, n_chunks, &grid, TPB);
+    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_span_decode_planar<Sym>), smem, n_chunks, &grid, TPB);
     if (e != cudaSuccess)
         return e;
     k_span_decode_planar<Sym><<<grid, TPB, smem, st>>>(
@@ -1294,9 +1284,6 @@ cudaError_t launch_suffix_search(const fkv_ctx *c, const double *pts, int64_t n_
     const double t = 2.0 * rl;
     const double thr2 = t * t;
     const int smem = tables_bytes(c->N, c->L);
-    e = cudaFuncSetAttribute(k_suffix_search, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     unsigned grid = 0;
     e = decode_grid(c, reinterpret_cast<const void *>(k_suffix_search), smem, cdiv(n_streams * spans, kThreads),
                     &grid);
@@ -1318,11 +1305,8 @@ cudaError_t read_t(const fkv_ctx *c, const double *pts, int64_t n_streams, int64
     if (blocks == 0)
         return cudaSuccess;
     const int smem = tables_bytes(c->N, c->L);
-    cudaError_t e = cudaFuncSetAttribute(k_read<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     unsigned grid = 0;
-    e = decode_grid(c, reinterpret_cast<const void *>(k_read<Sym>), smem, blocks, &grid, TPB);
+    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_read<Sym>), smem, blocks, &grid, TPB);
     if (e != cudaSuccess)
         return e;
     k_read<Sym><<<grid, TPB, smem, st>>>(
@@ -1427,11 +1411,8 @@ cudaError_t lossy_decode_t(const fkv_ctx *c, const LossyArgs &a, int64_t n_strea
     if (bps > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
     const int smem = c->N * 32 + ((kThreads * c->L * static_cast<int>(sizeof(Sym)) + 32 + 15) & ~15);
-    cudaError_t e = cudaFuncSetAttribute(k_lossy_decode<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     unsigned grid = 0;
-    e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_decode<Sym>), smem, n_chunks, &grid);
+    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_decode<Sym>), smem, n_chunks, &grid);
     if (e != cudaSuccess)
         return e;
     k_lossy_decode<Sym><<<grid, kThreads, smem, st>>>(a, n, spans, static_cast<int>(bps), n_chunks, sym, sym_stride,
@@ -1447,11 +1428,8 @@ cudaError_t lossy_read_t(const fkv_ctx *c, const LossyArgs &a, int64_t n_streams
     if (blocks == 0)
         return cudaSuccess;
     const int smem = c->N * 32;
-    cudaError_t e = cudaFuncSetAttribute(k_lossy_read<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     unsigned grid = 0;
-    e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_read<Sym>), smem, blocks, &grid);
+    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_read<Sym>), smem, blocks, &grid);
     if (e != cudaSuccess)
         return e;
     k_lossy_read<Sym><<<grid, kThreads, smem, st>>>(a, n_streams, n, req, n_req, out, lossy_walk(c),
@@ -1469,14 +1447,10 @@ cudaError_t launch_truncate(const fkv_ctx *c, const double *pts, int64_t n_strea
     const int64_t T = spans > keep_exact ? spans - keep_exact : 0;
     const int64_t words = cdiv(2 * T * bits, 32);
     if (n_streams > 0 && words > 0) {
-        int sms = 0;
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        if (e != cudaSuccess)
-            return e;
-        const int64_t blocks = min(cdiv(n_streams * cdiv(T, 32), kThreads / 32), static_cast<int64_t>(sms) * 8);
+        const int64_t blocks = min(cdiv(n_streams * cdiv(T, 32), kThreads / 32), static_cast<int64_t>(c->sms) * 8);
         k_truncate<<<static_cast<unsigned>(blocks), kThreads, 0, st>>>(pts, pt_stride, n_streams, T, bits, codes,
                                                                         code_stride, words);
-        e = cudaGetLastError();
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return e;
     }
@@ -1515,9 +1489,6 @@ namespace {
 template <typename Sym>
 cudaError_t ragged_decoder_grid(const fkv_ctx *c, const void *kern, int smem, unsigned *grid)
 {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     return decode_grid(c, kern, smem, 1ll << 40, grid, dec_threads<Sym>());
 }
 

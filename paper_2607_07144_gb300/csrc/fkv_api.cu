@@ -292,6 +292,40 @@ const char *check_lossy(const fkv_ctx *ctx, int64_t n_streams, int64_t n, int bi
 
 }  // namespace
 
+cudaError_t kernel_use(const fkv_ctx *c, const void *fn, int threads, size_t smem, int *per_sm)
+{
+    for (int i = 0; i < c->n_uses; ++i) {
+        const fkv_kernel_use &u = c->uses[i];
+        if (u.fn == fn && u.smem == static_cast<int>(smem) && u.threads == threads) {
+            if (per_sm)
+                *per_sm = u.per_sm;
+            return cudaSuccess;
+        }
+    }
+    cudaError_t e;
+    if (smem > 0) {
+        // the limit, less 1 KB for a kernel's own static arrays, whatever this context needs
+        const int most = kMaxDynSmem - 1024 > static_cast<int>(smem) ? kMaxDynSmem - 1024 : static_cast<int>(smem);
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess)
+            return e;
+    }
+    fkv_kernel_use u;
+    u.fn = fn;
+    u.smem = static_cast<int>(smem);
+    u.threads = threads;
+    if (per_sm) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&u.per_sm, fn, threads, smem);
+        if (e != cudaSuccess)
+            return e;
+    }
+    if (c->n_uses < static_cast<int>(sizeof(c->uses) / sizeof(c->uses[0])))
+        c->uses[c->n_uses++] = u;
+    if (per_sm)
+        *per_sm = u.per_sm;
+    return cudaSuccess;
+}
+
 extern "C" {
 
 double fkv_packing_ratio(int N)
@@ -339,7 +373,8 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
     ctx->N = N;
     ctx->r = r;
     ctx->L = span_len;
-    if (cudaGetDevice(&ctx->device) != cudaSuccess)
+    if (cudaGetDevice(&ctx->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess)
         return bail(FKV_ECUDA);
 
     // vertex table (the encoders give a symbol >= N a NaN vertex)

@@ -45,11 +45,22 @@ struct fkv_decconst {
     int sect_sh;                   // floor(2^16 log2(1/r))
 };
 
+// A kernel as a context launches it: its dynamic shared memory and how many
+// of its blocks fit an SM.
+struct fkv_kernel_use {
+    const void *fn = nullptr;
+    int smem = 0, threads = 0, per_sm = 0;
+};
+
 struct fkv_ctx {
     int N = 0;
     double r = 0.0;
     int L = 0;
     int device = 0;
+    int sms = 0;                   // SMs of the device
+    // kernels this context has launched (calls on one context are serialised)
+    mutable fkv_kernel_use uses[32];
+    mutable int n_uses = 0;
     double2 *d_V = nullptr;        // [N] vertices; first of one allocation with d_T, d_dec, d_status and d_pre
     fkv_decconst *d_dec = nullptr; // decoder constants (device copy)
     longlong2 *d_T = nullptr;      // [L][N] (1-r) r^j V(c) in Q1.62
@@ -86,6 +97,14 @@ struct fkv_streams {
 };
 
 // ---------------------------------------------------------------- launches
+// Ready `fn` for launches with `smem` bytes of dynamic shared memory and
+// `threads` threads a block, once per context; *per_sm (if not null) receives
+// the blocks that fit an SM.  Setting the attribute and the occupancy query on
+// every call cost small calls 2 to 5 us of their 12 to 20 on the host.  The
+// attribute is raised to the device's limit, so that contexts of different
+// tables do not lower it for one another.
+cudaError_t kernel_use(const fkv_ctx *c, const void *fn, int threads, size_t smem, int *per_sm);
+
 // codec.cu
 // Dynamic shared memory the codec's decoding kernels take for (N, L): the
 // decoder tables plus one chunk of staged symbols.

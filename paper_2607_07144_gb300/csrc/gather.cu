@@ -589,6 +589,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_read_gather(const ReadGatherArg
                     q[u] = __ldg(&a.order[e].x);
                 }
             }
+            // the next round's index words and requests into L1 meanwhile
+#pragma unroll
+            for (int u = kU; u < 2 * kU; ++u) {
+                const int64_t e = start + j + u * vpi;
+                if (j + u * vpi < j1) {
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(scr + e * R + a.off + h * S));
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(&a.order[e]));
+                }
+            }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 if (j + u * vpi >= j1)
@@ -789,20 +798,13 @@ cudaError_t launch_rvq_decode(const fkv_ctx *c, int kv, const void *sym, int lay
     const bool wide = reinterpret_cast<uintptr_t>(sym) % (Sv * esz) == 0 && a.ib % Sv == 0 && a.il % Sv == 0 &&
                       a.ih % Sv == 0 && a.ir % Sv == 0 && a.ioff % Sv == 0;
     const void *kern = gather_kernel_for(a.S, wide, c->KC);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem > 48 * 1024 ? smem : 48 * 1024));
-    if (e != cudaSuccess)
-        return e;
     // persistent: as many blocks as fit at once, each taking an equal share
-    int sms = 0, per_sm = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (e != cudaSuccess)
-        return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
+    int per_sm = 0;
+    cudaError_t e = kernel_use(c, kern, kThreads, smem, &per_sm);
     if (e != cudaSuccess)
         return e;
     const int64_t work = static_cast<int64_t>(c->Ly) * c->H * parts * nvec;
-    int64_t blocks = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
+    int64_t blocks = static_cast<int64_t>(c->sms) * (per_sm > 0 ? per_sm : 1);
     if (blocks > work)
         blocks = work;
     void *args[] = {&a};
@@ -851,12 +853,10 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
                                          : reinterpret_cast<const void *>(k_read_kv<uint8_t, false>))
                                 : (block ? reinterpret_cast<const void *>(k_read_kv<uint16_t, true>)
                                          : reinterpret_cast<const void *>(k_read_kv<uint16_t, false>));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     // persistent: as many blocks as fit at once, or one per eight requests
-    int sms = 0, per_sm = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    int per_sm = 0;
+    const int sms = c->sms;
+    cudaError_t e = kernel_use(c, kern, kReadWarps * 32, smem, &per_sm);
     if (e != cudaSuccess)
         return e;
     if (order && n_streams <= 0x7FFFFFFF && n_rec <= 0x7FFFFFFF) {
@@ -879,9 +879,6 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
         if (read_staged(c, n_req))
             a.scr = order + read_scr_ints(c, n_req);
     }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kReadWarps * 32, smem);
-    if (e != cudaSuccess)
-        return e;
     int64_t blocks = block ? n_req : (n_req + kReadWarps - 1) / kReadWarps;
     const int64_t resident = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
     if (blocks > resident)
@@ -898,11 +895,8 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
         const int tsm = read_tables_bytes(a.N, a.L);
         const void *sk = esz == 1 ? reinterpret_cast<const void *>(k_read_syms<uint8_t>)
                                   : reinterpret_cast<const void *>(k_read_syms<uint16_t>);
-        e = cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm);
-        if (e != cudaSuccess)
-            return e;
         int sper = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sper, sk, 256, tsm);
+        e = kernel_use(c, sk, 256, tsm, &sper);
         if (e != cudaSuccess)
             return e;
         int spr = (a.R + a.L - 1) / a.L + (a.R % a.L ? 1 : 0);
@@ -937,12 +931,8 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
         const size_t gsm = static_cast<size_t>(S) * c->KC * Dp * 4;
         const bool wide = a.R % S == 0 && g.off % S == 0;
         const void *gk = read_gather_kernel_for(S, wide, c->KC);
-        e = cudaFuncSetAttribute(gk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(gsm > 48 * 1024 ? gsm : 48 * 1024));
-        if (e != cudaSuccess)
-            return e;
         int gper = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gper, gk, kThreads, gsm);
+        e = kernel_use(c, gk, kThreads, gsm, &gper);
         if (e != cudaSuccess)
             return e;
         void *gargs[] = {&g};

@@ -2504,10 +2504,10 @@ cudaError_t launch_wait_check(unsigned *status, uint64_t limit_ns, int *out_dev,
 }
 
 template <int ESZ, int NB>
-cudaError_t launch_rvq64(const CUtensorMap &tmap, const RvqArgs &a, int ppg, int n_pairs, unsigned grid,
-                         cudaStream_t st)
+cudaError_t launch_rvq64(const fkv_ctx *c, const CUtensorMap &tmap, const RvqArgs &a, int ppg, int n_pairs,
+                         unsigned grid, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_rvq64<ESZ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, v2::SMEM);
+    const cudaError_t e = kernel_use(c, reinterpret_cast<const void *>(k_rvq64<ESZ, NB>), v2::kThreads, v2::SMEM, nullptr);
     if (e != cudaSuccess)
         return e;
     k_rvq64<ESZ, NB><<<grid, v2::kThreads, v2::SMEM, st>>>(tmap, a, ppg, n_pairs);
@@ -2527,10 +2527,11 @@ bool pair_tiles(int64_t tiles, int64_t groups, int sms)
 }
 
 template <int ESZ, int NB>
-cudaError_t launch_rvq64_pair(const fkv_cbset &cb, const RvqArgs &a, int upg, int n_units, unsigned clusters,
-                              cudaStream_t st)
+cudaError_t launch_rvq64_pair(const fkv_ctx *c, const fkv_cbset &cb, const RvqArgs &a, int upg, int n_units,
+                              unsigned clusters, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_rvq64_pair<ESZ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, pr::SMEM);
+    const cudaError_t e = kernel_use(c, reinterpret_cast<const void *>(k_rvq64_pair<ESZ, NB>), pr::kThreads, pr::SMEM,
+                                     nullptr);
     if (e != cudaSuccess)
         return e;
     k_rvq64_pair<ESZ, NB><<<2 * clusters, pr::kThreads, pr::SMEM, st>>>(cb.tmap_half, cb.tmap_aug, a, upg, n_units,
@@ -2584,41 +2585,36 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         const int64_t n_pairs = ppg * c->Ly * c->H;
         if (n_pairs > 0x7FFFFFFF)
             return cudaErrorInvalidConfiguration;
-        int sms = 0;
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        if (e != cudaSuccess)
-            return e;
+        const int sms = c->sms;
         const unsigned grid = static_cast<unsigned>(n_pairs < sms ? n_pairs : sms);
         const int pp = static_cast<int>(ppg), np = static_cast<int>(n_pairs);
         if (pair_tiles(tiles, c->Ly * c->H, sms)) {
             const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
             const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
             if (c->KC == 1024)
-                return x->dtype == FKV_F32 ? launch_rvq64_pair<4, 4>(cb, a, upg, nu, clusters, st)
-                                           : launch_rvq64_pair<2, 4>(cb, a, upg, nu, clusters, st);
-            return x->dtype == FKV_F32 ? launch_rvq64_pair<4, 1>(cb, a, upg, nu, clusters, st)
-                                       : launch_rvq64_pair<2, 1>(cb, a, upg, nu, clusters, st);
+                return x->dtype == FKV_F32 ? launch_rvq64_pair<4, 4>(c, cb, a, upg, nu, clusters, st)
+                                           : launch_rvq64_pair<2, 4>(c, cb, a, upg, nu, clusters, st);
+            return x->dtype == FKV_F32 ? launch_rvq64_pair<4, 1>(c, cb, a, upg, nu, clusters, st)
+                                       : launch_rvq64_pair<2, 1>(c, cb, a, upg, nu, clusters, st);
         }
         if (c->KC == 1024)
-            return x->dtype == FKV_F32 ? launch_rvq64<4, 4>(cb.tmap, a, pp, np, grid, st)
-                                       : launch_rvq64<2, 4>(cb.tmap, a, pp, np, grid, st);
-        return x->dtype == FKV_F32 ? launch_rvq64<4, 1>(cb.tmap, a, pp, np, grid, st)
-                                   : launch_rvq64<2, 1>(cb.tmap, a, pp, np, grid, st);
+            return x->dtype == FKV_F32 ? launch_rvq64<4, 4>(c, cb.tmap, a, pp, np, grid, st)
+                                       : launch_rvq64<2, 4>(c, cb.tmap, a, pp, np, grid, st);
+        return x->dtype == FKV_F32 ? launch_rvq64<4, 1>(c, cb.tmap, a, pp, np, grid, st)
+                                   : launch_rvq64<2, 1>(c, cb.tmap, a, pp, np, grid, st);
     } else {
         // 128-dimensional heads: 256 codewords per stage, the tiles of all
         // head groups paired in order
         const int64_t n_pairs = (tiles * c->Ly * c->H + 1) / 2;
         if (n_pairs > 0x7FFFFFFF)
             return cudaErrorInvalidConfiguration;
-        int sms = 0;
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        if (e != cudaSuccess)
-            return e;
+        const int sms = c->sms;
         if (pair_tiles(tiles, c->Ly * c->H, sms)) {
             const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
             const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
             const auto kern = x->dtype == FKV_F32 ? k_rvq128_pair<4> : k_rvq128_pair<2>;
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pr128::SMEM);
+            const cudaError_t e = kernel_use(c, reinterpret_cast<const void *>(kern), pr128::kThreads, pr128::SMEM,
+                                             nullptr);
             if (e != cudaSuccess)
                 return e;
             kern<<<2 * clusters, pr128::kThreads, pr128::SMEM, st>>>(cb.tmap_half, cb.tmap_aug, a, upg, nu,
@@ -2627,17 +2623,11 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         }
         const unsigned grid = static_cast<unsigned>(n_pairs < sms ? n_pairs : sms);
         const int np = static_cast<int>(n_pairs);
-        if (x->dtype == FKV_F32) {
-            e = cudaFuncSetAttribute(k_rvq128<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, v3::SMEM);
-            if (e != cudaSuccess)
-                return e;
-            k_rvq128<4><<<grid, v3::kThreads, v3::SMEM, st>>>(cb.tmap, a, np);
-        } else {
-            e = cudaFuncSetAttribute(k_rvq128<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, v3::SMEM);
-            if (e != cudaSuccess)
-                return e;
-            k_rvq128<2><<<grid, v3::kThreads, v3::SMEM, st>>>(cb.tmap, a, np);
-        }
+        const auto kern = x->dtype == FKV_F32 ? k_rvq128<4> : k_rvq128<2>;
+        const cudaError_t e = kernel_use(c, reinterpret_cast<const void *>(kern), v3::kThreads, v3::SMEM, nullptr);
+        if (e != cudaSuccess)
+            return e;
+        kern<<<grid, v3::kThreads, v3::SMEM, st>>>(cb.tmap, a, np);
     }
     return cudaGetLastError();
 }
