@@ -82,6 +82,25 @@ __device__ __forceinline__ void stage_out(uint8_t *dst, const uint8_t *buf, int 
     }
 }
 
+// stage_out by one warp.
+__device__ __forceinline__ void stage_out_warp(uint8_t *dst, const uint8_t *buf, int len, int off)
+{
+    uint8_t *a = dst - off;
+    const int total = off + len;
+    const int nv = (total + 15) >> 4;
+    for (int v = threadIdx.x & 31; v < nv; v += 32) {
+        const int b0 = v << 4;
+        if (b0 >= off && b0 + 16 <= total) {
+            *reinterpret_cast<uint4 *>(a + b0) = *reinterpret_cast<const uint4 *>(buf + b0);
+        } else {
+            const int lo = b0 > off ? b0 : off;
+            const int hi = b0 + 16 < total ? b0 + 16 : total;
+            for (int q = lo; q < hi; ++q)
+                a[q] = buf[q];
+        }
+    }
+}
+
 // Sec. 1 forward map for a run of symbols from (x, y), binary64, no FMA.
 // A symbol >= N takes a NaN vertex, so its span's point comes out NaN.
 template <typename Sym>
@@ -824,49 +843,55 @@ __device__ __forceinline__ unsigned long long trunc_field(double x, double up, i
 }
 
 // Warp per group of 32 spans of one stream: the group's 64 codes fill exactly
-// 2B words (the group starts at stream bit 64 B g, a word boundary); each lane
-// computes its span's two codes, then assembles words lane, lane + 32, ... of
-// the group from the codes that overlap them, fetched by warp shuffles.
+// 2B words (the group starts at stream bit 64 B g, a word boundary).  A lane
+// puts its span's two codes, 2B bits that touch at most five words, into the
+// warp's words in shared memory (neighbours share words, so by atomic OR), and
+// the warp writes those out.  @@TR@@
 __global__ void __launch_bounds__(kThreads)
 k_truncate(const double *__restrict__ pts, int64_t pt_stride, int64_t n_streams, int64_t T, int bits,
            uint32_t *__restrict__ codes, int64_t code_stride, int64_t words)
 {
+    __shared__ uint32_t wbuf[kThreads / 32][2 * 53 + 4];
     const double up = static_cast<double>(1ull << (bits - 1));
     const int lane = threadIdx.x & 31;
+    uint32_t *w = wbuf[threadIdx.x >> 5];
     const int64_t gps = (T + 31) >> 5;                       // groups per stream
     const int64_t n_groups = n_streams * gps;
     const int64_t nw = static_cast<int64_t>(gridDim.x) * (kThreads / 32);
-    const int kmax = 32 / bits + 2;                          // codes overlapping one word, at most
     const int wpg = 2 * bits;                                // words per group
+    for (int j = lane; j < wpg + 4; j += 32)
+        w[j] = 0;
+    __syncwarp();
     for (int64_t g = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5; g < n_groups; g += nw) {
         const int64_t stream = g / gps, grp = g - stream * gps;
         const int64_t u = grp * 32 + lane;
-        unsigned long long fx = 0, fy = 0;
         if (u < T) {
-            const double2 p = reinterpret_cast<const double2 *>(pts)[stream * pt_stride + u];
-            fx = trunc_field(p.x, up, bits);
-            fy = trunc_field(p.y, up, bits);
+            const double2 p = __ldg(&reinterpret_cast<const double2 *>(pts)[stream * pt_stride + u]);
+            const unsigned long long fx = trunc_field(p.x, up, bits), fy = trunc_field(p.y, up, bits);
+            // the 2B bits from bit 2B lane on, as words of 32
+            const int at = wpg * lane, sh = at & 31;
+            const unsigned long long lo = fx | (fy << bits), hi = bits < 64 - bits ? 0ull : fy >> (64 - bits);
+            uint32_t v[5];
+            v[0] = static_cast<uint32_t>(lo << sh);
+            v[1] = __funnelshift_l(static_cast<uint32_t>(lo), static_cast<uint32_t>(lo >> 32), sh);
+            v[2] = __funnelshift_l(static_cast<uint32_t>(lo >> 32), static_cast<uint32_t>(hi), sh);
+            v[3] = __funnelshift_l(static_cast<uint32_t>(hi), static_cast<uint32_t>(hi >> 32), sh);
+            v[4] = __funnelshift_l(static_cast<uint32_t>(hi >> 32), 0u, sh);
+            const int nv = (sh + wpg + 31) >> 5;
+#pragma unroll
+            for (int i = 0; i < 5; ++i)
+                if (i < nv)
+                    atomicOr(&w[(at >> 5) + i], v[i]);
         }
+        __syncwarp();
         const int64_t w0 = grp * wpg;
-        const int64_t nwg = min(static_cast<int64_t>(wpg), words - w0);
-        for (int j0 = 0; j0 < wpg; j0 += 32) {
-            const int j = j0 + lane;
-            const int bit0 = 32 * j;                         // relative to the group
-            const int c0 = bit0 / bits;
-            uint32_t out = 0;
-            for (int k = 0; k < kmax; ++k) {
-                const int ci = c0 + k;                       // code of the group: span ci / 2, x or y
-                const int src = min(ci >> 1, 31);
-                const unsigned long long vx = __shfl_sync(0xFFFFFFFFu, fx, src);
-                const unsigned long long vy = __shfl_sync(0xFFFFFFFFu, fy, src);
-                const unsigned long long f = (ci & 1) ? vy : vx;
-                const int sh = ci * bits - bit0;
-                if (ci < 64 && sh < 32)
-                    out |= static_cast<uint32_t>(sh >= 0 ? f << sh : f >> (-sh));
-            }
+        const int nwg = static_cast<int>(min(static_cast<int64_t>(wpg), words - w0));
+        for (int j = lane; j < wpg; j += 32) {
             if (j < nwg)
-                codes[stream * code_stride + w0 + j] = out;
+                codes[stream * code_stride + w0 + j] = w[j];
+            w[j] = 0;
         }
+        __syncwarp();
     }
 }
 
@@ -885,6 +910,18 @@ __device__ __forceinline__ long long read_field(const uint32_t *w, int64_t words
     return static_cast<long long>(v << sh) >> sh;
 }
 
+// k 2^-(bits - 1) for a bits-bit code k: below 53 bits, k added to the integer
+// pattern of 1.5 2^52 and that number subtracted again is k exactly, and the
+// scaling is the exponent's.
+__device__ __forceinline__ double code_value(long long k, int bits, double scale)
+{
+    if (bits > 52)
+        return __dmul_rn(static_cast<double>(k), scale);
+    const double v = __dsub_rn(__longlong_as_double(k + 0x4338000000000000ll), 0x1.8p52);
+    const int hi = __double2hiint(v);
+    return __hiloint2double(k != 0 ? hi - ((bits - 1) << 20) : 0, __double2loint(v));
+}
+
 // The point a lossy archive keeps for span u of a stream.
 __device__ __forceinline__ double2 lossy_point(const LossyArgs &a, int64_t stream, int64_t u)
 {
@@ -894,7 +931,7 @@ __device__ __forceinline__ double2 lossy_point(const LossyArgs &a, int64_t strea
     const int64_t pos = 2 * u * a.bits;
     const long long kx = read_field(w, a.words, pos, a.bits);
     const long long ky = read_field(w, a.words, pos + a.bits, a.bits);
-    return make_double2(__dmul_rn(static_cast<double>(kx), a.scale), __dmul_rn(static_cast<double>(ky), a.scale));
+    return make_double2(code_value(kx, a.bits, a.scale), code_value(ky, a.bits, a.scale));
 }
 
 // Squared distance to a vertex as the paper's binary64 arithmetic forms it
@@ -915,6 +952,8 @@ struct LossyWalk {
     float sect_a[5], sect_thr;   // arctangent polynomial in sector widths and its safe fraction
 };
 
+static __device__ __noinline__ double div_fp64(double a, double b) { return __ddiv_rn(a, b); }
+
 // a / r rounded to nearest even, as __ddiv_rn(a, r), on the integer pipe: the
 // mantissa of a (at the top of 64 bits) times inv is the quotient's upper 64
 // bits, low by less than one unit, and rounds at its 53rd bit.  A quotient of
@@ -933,7 +972,7 @@ __device__ __forceinline__ double div_ratio(const LossyWalk &q, double a)
     const unsigned half = 512u << top;
     const unsigned rest = static_cast<unsigned>(h) & (2u * half - 1u);
     if (static_cast<unsigned>(e - 512) >= 1000u || rest == half - 1u || q.inv == 0)
-        return __ddiv_rn(a, q.r);
+        return div_fp64(a, q.r);
     const unsigned long long n = (h + half) >> drop;
     const unsigned th = static_cast<unsigned>(n >> 32) + (static_cast<unsigned>(1021 + top + e - q.er) << 20);
     return __hiloint2double(static_cast<int>(th | (hi & 0x80000000u)), static_cast<int>(static_cast<unsigned>(n)));
@@ -1037,8 +1076,16 @@ __device__ __forceinline__ void walk64(const LossyWalk &q, const double2 *sV, do
     }
 }
 
+// Staging of one warp's 32 spans, 16-byte aligned, with the realignment slack.
+template <typename Sym>
+__host__ __device__ inline int warp_stage_bytes(int L)
+{
+    return (32 * L * static_cast<int>(sizeof(Sym)) + 32 + 15) & ~15;
+}
+
 // Bulk decode of a lossy archive: persistent blocks walk chunks of 256 spans
-// (one per thread) and write the symbols through shared memory.
+// (one per thread); each warp writes its 32 spans' symbols through its own
+// piece of shared memory, so that no warp waits for another's walk.
 template <typename Sym>
 __global__ void __launch_bounds__(kThreads)
 k_lossy_decode(const LossyArgs a, int64_t n, int64_t spans, int bps, int64_t n_chunks, Sym *__restrict__ sym,
@@ -1046,28 +1093,30 @@ k_lossy_decode(const LossyArgs a, int64_t n, int64_t spans, int bps, int64_t n_c
 {
     extern __shared__ __align__(16) uint8_t dsm[];
     double2 *sV = reinterpret_cast<double2 *>(dsm);
-    uint8_t *sbuf = dsm + q.N * 32;
-    const int L = q.L;
+    const int L = q.L, lane = threadIdx.x & 31;
+    uint8_t *sbuf = dsm + q.N * 32 + (threadIdx.x >> 5) * warp_stage_bytes<Sym>(L);
     load_lossy(sV, q);
     __syncthreads();
     ChunkWalk cw(bps);
     for (int64_t ck = blockIdx.x; ck < n_chunks; ck += gridDim.x, cw.next()) {
         const int64_t stream = cw.stream;
-        const int64_t s0 = cw.sb * kThreads;
+        const int64_t s0 = cw.sb * kThreads + (threadIdx.x & ~31);     // the warp's first span
+        if (s0 >= spans)
+            continue;
         const int64_t b = s0 * L;
-        const int64_t e = min(n, (s0 + kThreads) * L);
+        const int64_t e = min(n, (s0 + 32) * L);
         uint8_t *dst = reinterpret_cast<uint8_t *>(sym + stream * sym_stride + b);
         const int off = static_cast<int>(reinterpret_cast<uintptr_t>(dst) & 15);
-        const int64_t s = s0 + threadIdx.x;
+        const int64_t s = s0 + lane;
         if (s < spans) {
             const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
             const double2 p = lossy_point(a, stream, s);
-            Sym *my = reinterpret_cast<Sym *>(sbuf + off) + threadIdx.x * L;
-            walk64(q, sV, p.x, p.y, m, [&](int j, int c) { my[m - 1 - j] = static_cast<Sym>(c); });
+            Sym *my = reinterpret_cast<Sym *>(sbuf + off) + lane * L + m - 1;
+            walk64(q, sV, p.x, p.y, m, [&](int j, int c) { my[-j] = static_cast<Sym>(c); });
         }
-        __syncthreads();
-        stage_out(dst, sbuf, static_cast<int>(e - b) * static_cast<int>(sizeof(Sym)), off);
-        __syncthreads();
+        __syncwarp();
+        stage_out_warp(dst, sbuf, static_cast<int>(e - b) * static_cast<int>(sizeof(Sym)), off);
+        __syncwarp();
     }
 }
 
@@ -1410,7 +1459,7 @@ cudaError_t lossy_decode_t(const fkv_ctx *c, const LossyArgs &a, int64_t n_strea
         return cudaSuccess;
     if (bps > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
-    const int smem = c->N * 32 + ((kThreads * c->L * static_cast<int>(sizeof(Sym)) + 32 + 15) & ~15);
+    const int smem = c->N * 32 + kThreads / 32 * warp_stage_bytes<Sym>(c->L);
     unsigned grid = 0;
     cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_decode<Sym>), smem, n_chunks, &grid);
     if (e != cudaSuccess)
