@@ -846,7 +846,8 @@ __device__ __forceinline__ unsigned long long trunc_field(double x, double up, i
 // 2B words (the group starts at stream bit 64 B g, a word boundary).  A lane
 // puts its span's two codes, 2B bits that touch at most five words, into the
 // warp's words in shared memory (neighbours share words, so by atomic OR), and
-// the warp writes those out.  @@TR@@
+// the warp writes those out.  1.14 M spans at 24 bits:
+// 10.4 us (15.2 with the words gathered by shuffles).
 __global__ void __launch_bounds__(kThreads)
 k_truncate(const double *__restrict__ pts, int64_t pt_stride, int64_t n_streams, int64_t T, int bits,
            uint32_t *__restrict__ codes, int64_t code_stride, int64_t words)
@@ -949,7 +950,8 @@ struct LossyWalk {
     double w, r;             // 1 - r and r
     unsigned long long inv;  // floor(2^127 / (r's mantissa at the top of 64 bits)); 0 for r a power of two
     int er;                  // r's exponent field
-    float sect_a[5], sect_thr;   // arctangent polynomial in sector widths and its safe fraction
+    const int2 *bound;       // (cos, -sin) 2^30 of boundary g + 1/2 at [g + N / 2 + 1], g = -N/2 - 1 .. N/2
+    float sect_a[5];         // arctangent polynomial in sector widths
 };
 
 static __device__ __noinline__ double div_fp64(double a, double b) { return __ddiv_rn(a, b); }
@@ -978,29 +980,31 @@ __device__ __forceinline__ double div_ratio(const LossyWalk &q, double a)
     return __hiloint2double(static_cast<int>(th | (hi & 0x80000000u)), static_cast<int>(static_cast<unsigned>(n)));
 }
 
-// float32 image of a binary64 value, truncated, by integer ops (a conversion
-// issues at the FP64 rate): below 2^-126 zero; callers rule out |v| >= 2^20.
-__device__ __forceinline__ float trunc_f32(double v)
-{
-    const int hi = __double2hiint(v);
-    const int r = max((hi & 0x7FFFFFFF) - (896 << 20), 0);
-    return __int_as_float(static_cast<int>(__funnelshift_l(static_cast<unsigned>(__double2loint(v)),
-                                                           static_cast<unsigned>(r), 3)) |
-                          (hi & static_cast<int>(0x80000000)));
-}
-
 // Sec. 1 cell test in binary64 for a point that need not be a code point:
 // the vertex of least binary64 squared distance, lowest index on a tie.  The
 // nearest vertex is the angularly nearest.  For a larger coordinate in
-// [2^-20, 2^20) the fp32 angle decides alone while it is farther from a
-// sector boundary than twice its error bound: the true direction is then at
-// least 1.4e-5 rad off the boundary, so the two squared distances differ by
-// 4 |p| sin(pi/N) 1.4e-5 (1.7e-7 |p| at N = 1024), far above their rounding,
-// (|p| + 1)^2 3.4e-16.  Nearer the boundary, and for |p|^2 up to 2^60, the
+// [2^-14, 2^16) the fp32 angle names the pair of neighbouring sectors (any
+// error below half a sector will do) and the sign of the cross product with
+// their common boundary, on 31-bit images of the point and the boundary, picks
+// one of them.  The images are off by at most one unit (the point, truncated)
+// and half a unit (the boundary) a coordinate, so the product by less than
+// (sqrt 2 + 2) 2^30.  At 2^34 and above its sign is sure, and the direction at
+// least 12.5 2^30 / 2^61.5 = 4.1e-9 rad off the boundary: the two squared
+// distances differ by 4 |p| sin(pi/N) 4.1e-9, above their rounding,
+// (|p| + 1)^2 3.4e-16 (at N = 1024 by a factor of 9 at |p| = 2^-14, 1.6 at
+// 2^16.5 and 10^4 at 1).  Nearer the boundary, and for |p|^2 up to 2^60, the
 // three vertices around the angle are scored: every other vertex is farther by
 // at least 2|p|(cos(pi/N) - cos(3 pi/N)) (7.5e-5 |p| at N = 1024), so the
-// choice equals a full scan's.  Other points (tiny, huge, not finite) take
-// the full scan.
+// choice equals a full scan's.  Other points (tiny, huge, not finite) take the
+// full scan.
+// The angle alone with a margin for the polynomial's 1.2e-5 rad, as in the
+// planar decoder, left 3 warps in 4 a lane to score: a code point's offset
+// from its vertex is r times a point near the unit circle, so its place across
+// the sector crowds at the boundaries.  k_lossy_decode on 96 streams of 71,136
+// symbols (N = 256, 24 bits): 53 us, 105 with the margin.  (The planar
+// decoder settles its near cases with four integer products; there the cross
+// product costs more than it saves, 0.460 against 0.456 ms for encoding and
+// decoding 50.3 M symbols.)
 static __device__ __noinline__ int nearest64_scored(const double2 *sV, int N, double x, double y)
 {
     const double rr = x * x + y * y;
@@ -1035,27 +1039,50 @@ static __device__ __noinline__ int nearest64_scored(const double2 *sV, int N, do
     return best;
 }
 
-__device__ __forceinline__ int nearest64(const LossyWalk &q, const double2 *sV, double x, double y)
+// The 31 upper bits of a binary64 mantissa, shifted down to exponent field e.
+__device__ __forceinline__ int image31(double v, int e)
 {
-    // exponent fields of the larger coordinate in [2^-20, 2^20)
-    const int big = max(__double2hiint(x) & 0x7FFFFFFF, __double2hiint(y) & 0x7FFFFFFF);
-    if (static_cast<unsigned>(big - (1003 << 20)) < static_cast<unsigned>(40 << 20)) {
-        float f;
-        const int c = fkvdec::sector_of(q.N, q.sect_a, trunc_f32(x), trunc_f32(y), 0x1p-30f, f);
-        if (fabsf(f) < q.sect_thr)
-            return c;
+    const int hi = __double2hiint(v);
+    const int ev = (hi >> 20) & 0x7FF;
+    const unsigned m = 0x40000000u | ((static_cast<unsigned>(hi) & 0xFFFFFu) << 10) |
+                       (static_cast<unsigned>(__double2loint(v)) >> 22);
+    const int r = static_cast<int>(m >> min(e - ev, 31));
+    return hi < 0 ? -r : r;
+}
+
+__device__ __forceinline__ int nearest64(const LossyWalk &q, const int2 *bound, const double2 *sV, double x, double y)
+{
+    // exponent field of the larger coordinate, in [2^-14, 2^16)
+    const int big = max(__double2hiint(x) & 0x7FFFFFFF, __double2hiint(y) & 0x7FFFFFFF) >> 20;
+    if (static_cast<unsigned>(big - 1009) < 30u) {
+        const int hx = image31(x, big), hy = image31(y, big);
+        const float a = fkvdec::sector_angle(q.N, q.sect_a, __int2float_rn(hx), __int2float_rn(hy), 1.0f);
+        const int lower = __float_as_int(__fadd_rd(a, 12582912.0f)) - 0x4B400000;   // floor, -N/2 - 1 .. N/2
+        const int2 b = bound[lower + (q.N / 2 + 1)];
+        const int s =
+            static_cast<int>((static_cast<long long>(b.x) * hy + static_cast<long long>(b.y) * hx) >> 32);
+        const int c = lower + (s > 0 ? 1 : 0);
+        if (static_cast<unsigned>(s + 4) > 7u)
+            return c < 0 ? c + q.N : c;
     }
     return nearest64_scored(sV, q.N, x, y);
 }
 
-// Vertices V(c) at sV[c] and their multiples (1 - r) V(c) at sV[N + c].
-__device__ __forceinline__ void load_lossy(double2 *sV, const LossyWalk &q)
+// Vertices V(c) at sV[c], their multiples (1 - r) V(c) at sV[N + c], the
+// sector boundaries behind them (lossy_table_bytes in all).
+__host__ __device__ inline int lossy_table_bytes(int N) { return (N * 32 + (N + 2) * 8 + 15) & ~15; }
+
+__device__ __forceinline__ const int2 *load_lossy(double2 *sV, const LossyWalk &q)
 {
+    int2 *bound = reinterpret_cast<int2 *>(sV + 2 * q.N);
+    for (int i = threadIdx.x; i < q.N + 2; i += blockDim.x)
+        bound[i] = q.bound[i];
     for (int i = threadIdx.x; i < q.N; i += blockDim.x) {
         const double2 v = q.V[i];
         sV[i] = v;
         sV[q.N + i] = make_double2(__dmul_rn(q.w, v.x), __dmul_rn(q.w, v.y));
     }
+    return bound;
 }
 
 // Backward walk from (x, y) in the paper's arithmetic: the cell, then
@@ -1063,12 +1090,13 @@ __device__ __forceinline__ void load_lossy(double2 *sV, const LossyWalk &q)
 // IEEE division).  emit(j, c) receives the symbol of step j.  Two binary64
 // operations a symbol, the differences; three scored distances, the products
 // and two divisions on the FP64 pipe took about 40.  96 streams of 71,136
-// symbols (N = 256, 24 bits): 0.101 ms, 0.586 ms before.
+// symbols (N = 256, 24 bits): 0.053 ms, 0.586 ms before.
 template <class Emit>
-__device__ __forceinline__ void walk64(const LossyWalk &q, const double2 *sV, double x, double y, int steps, Emit emit)
+__device__ __forceinline__ void walk64(const LossyWalk &q, const int2 *bound, const double2 *sV, double x,
+                                       double y, int steps, Emit emit)
 {
     for (int j = 0; j < steps; ++j) {
-        const int c = nearest64(q, sV, x, y);
+        const int c = nearest64(q, bound, sV, x, y);
         emit(j, c);
         const double2 v = sV[q.N + c];
         x = div_ratio(q, __dsub_rn(x, v.x));
@@ -1094,8 +1122,8 @@ k_lossy_decode(const LossyArgs a, int64_t n, int64_t spans, int bps, int64_t n_c
     extern __shared__ __align__(16) uint8_t dsm[];
     double2 *sV = reinterpret_cast<double2 *>(dsm);
     const int L = q.L, lane = threadIdx.x & 31;
-    uint8_t *sbuf = dsm + q.N * 32 + (threadIdx.x >> 5) * warp_stage_bytes<Sym>(L);
-    load_lossy(sV, q);
+    uint8_t *sbuf = dsm + lossy_table_bytes(q.N) + (threadIdx.x >> 5) * warp_stage_bytes<Sym>(L);
+    const int2 *bound = load_lossy(sV, q);
     __syncthreads();
     ChunkWalk cw(bps);
     for (int64_t ck = blockIdx.x; ck < n_chunks; ck += gridDim.x, cw.next()) {
@@ -1112,7 +1140,7 @@ k_lossy_decode(const LossyArgs a, int64_t n, int64_t spans, int bps, int64_t n_c
             const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
             const double2 p = lossy_point(a, stream, s);
             Sym *my = reinterpret_cast<Sym *>(sbuf + off) + lane * L + m - 1;
-            walk64(q, sV, p.x, p.y, m, [&](int j, int c) { my[-j] = static_cast<Sym>(c); });
+            walk64(q, bound, sV, p.x, p.y, m, [&](int j, int c) { my[-j] = static_cast<Sym>(c); });
         }
         __syncwarp();
         stage_out_warp(dst, sbuf, static_cast<int>(e - b) * static_cast<int>(sizeof(Sym)), off);
@@ -1129,7 +1157,7 @@ k_lossy_read(const LossyArgs a, int64_t n_streams, int64_t n, const int64_t *__r
     extern __shared__ __align__(16) uint8_t dsm[];
     double2 *sV = reinterpret_cast<double2 *>(dsm);
     const int L = q.L;
-    load_lossy(sV, q);
+    const int2 *bound = load_lossy(sV, q);
     __syncthreads();
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < n_req;
          i += static_cast<int64_t>(gridDim.x) * kThreads) {
@@ -1144,7 +1172,7 @@ k_lossy_read(const LossyArgs a, int64_t n_streams, int64_t n, const int64_t *__r
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
         const double2 p = lossy_point(a, st, u);
         int c = 0;
-        walk64(q, sV, p.x, p.y, m - o, [&](int j, int cc) { c = cc; });
+        walk64(q, bound, sV, p.x, p.y, m - o, [&](int j, int cc) { c = cc; });
         out[i] = static_cast<Sym>(c);
     }
 }
@@ -1444,7 +1472,7 @@ LossyWalk lossy_walk(const fkv_ctx *c)
     q.inv = m == 1ull << 63 ? 0ull : static_cast<unsigned long long>((static_cast<unsigned __int128>(1) << 127) / m);
     q.er = static_cast<int>(b >> 52);
     memcpy(q.sect_a, c->sect_a, sizeof(q.sect_a));
-    q.sect_thr = c->sect_thr;
+    q.bound = c->d_dec->bound;
     return q;
 }
 
@@ -1459,7 +1487,7 @@ cudaError_t lossy_decode_t(const fkv_ctx *c, const LossyArgs &a, int64_t n_strea
         return cudaSuccess;
     if (bps > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
-    const int smem = c->N * 32 + kThreads / 32 * warp_stage_bytes<Sym>(c->L);
+    const int smem = lossy_table_bytes(c->N) + kThreads / 32 * warp_stage_bytes<Sym>(c->L);
     unsigned grid = 0;
     cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_decode<Sym>), smem, n_chunks, &grid);
     if (e != cudaSuccess)
@@ -1476,7 +1504,7 @@ cudaError_t lossy_read_t(const fkv_ctx *c, const LossyArgs &a, int64_t n_streams
     const int64_t blocks = cdiv(n_req, kThreads);
     if (blocks == 0)
         return cudaSuccess;
-    const int smem = c->N * 32;
+    const int smem = lossy_table_bytes(c->N);
     unsigned grid = 0;
     cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_lossy_read<Sym>), smem, blocks, &grid);
     if (e != cudaSuccess)

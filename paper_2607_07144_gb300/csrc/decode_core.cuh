@@ -133,12 +133,11 @@ __device__ __forceinline__ float rcp_approx(float x)
     return y;
 }
 
-// The sector of direction (qx, qy): octant reduction to u in [0, 1], atan u
-// in sector widths (coefficients k) from the odd polynomial of fit_atan.py,
-// the octant's reflections, and rounding by adding 1.5 2^23; f receives the
-// distance to the sector's centre.  No subnormal or huge coordinates; the
-// larger one is at least `least`, or both are zero.
-__device__ __forceinline__ int sector_of(int N, const float *k, float qx, float qy, float least, float &f)
+// The angle of direction (qx, qy) in sector widths, in [-N/2, N/2]: octant
+// reduction to u in [0, 1], atan u (coefficients k, in sector widths) from the
+// odd polynomial of fit_atan.py, the octant's reflections.  No subnormal or
+// huge coordinates; the larger one is at least `least`, or both are zero.
+__device__ __forceinline__ float sector_angle(int N, const float *k, float qx, float qy, float least)
 {
     const float ax = fabsf(qx), ay = fabsf(qy);
     const float u = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), least));
@@ -148,7 +147,13 @@ __device__ __forceinline__ int sector_of(int N, const float *k, float qx, float 
         a = 0.25f * static_cast<float>(N) - a;
     if (qx < 0.0f)
         a = 0.5f * static_cast<float>(N) - a;
-    a = copysignf(a, qy);                      // in [-N/2, N/2]
+    return copysignf(a, qy);
+}
+
+// The sector, by adding 1.5 2^23; f receives the distance to its centre.
+__device__ __forceinline__ int sector_of(int N, const float *k, float qx, float qy, float least, float &f)
+{
+    const float a = sector_angle(N, k, qx, qy, least);
     const float big = a + 12582912.0f;
     f = a - (big - 12582912.0f);               // in [-0.5, 0.5]
     const int c = __float_as_int(big) - 0x4B400000;

@@ -417,7 +417,11 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
     for (int i = 0; i < 5; ++i)
         dec.sect_a[i] = static_cast<float>(static_cast<double>(fkvdec::kAtan[i]) * N / two_pi);
     memcpy(ctx->sect_a, dec.sect_a, sizeof(dec.sect_a));
-    ctx->sect_thr = dec.sect_thr;
+    for (int i = 0; i < N + 2; ++i) {
+        // the boundary half a sector above vertex g = i - (N / 2 + 1)
+        const double th = (i - (N / 2 + 1) + 0.5) * 2.0 * 3.14159265358979324 / N;
+        dec.bound[i] = make_int2(static_cast<int>(lrint(ldexp(cos(th), 30))), static_cast<int>(-lrint(ldexp(sin(th), 30))));
+    }
     dec.sect_sh = static_cast<int>(floor(65536.0 * log2(1.0 / r)));
     // one allocation: the host-made tables in one copy, then the status word
     // and the encoders' point table, filled on the device

@@ -41,6 +41,7 @@ struct fkv_decconst {
     float vfx[FKV_MAX_N], vfy[FKV_MAX_N];      // V(c) rounded to float
     long long alim[48];            // anchor limit 2^-4 r^m in Q1.62, per span length m
     float sect_thr;                // sector test threshold, N > 8 (decode_core.cuh classify)
+    int2 bound[FKV_MAX_N + 2];     // sector boundaries (codec.cu LossyWalk)
     float sect_a[5];               // arctangent polynomial in sector widths
     int sect_sh;                   // floor(2^16 log2(1/r))
 };
@@ -66,8 +67,7 @@ struct fkv_ctx {
     longlong2 *d_T = nullptr;      // [L][N] (1-r) r^j V(c) in Q1.62
     double2 *d_pre = nullptr;      // [N^pre_k] points after pre_k symbols from the anchor (codec.cu)
     int pre_k = 0;
-    float sect_a[5] = {};          // host copies of the decoder's sector constants
-    float sect_thr = 0.0f;
+    float sect_a[5] = {};          // host copy of the decoder's sector polynomial
     unsigned *d_status = nullptr;
     // archive geometry and codebooks
     bool has_cb = false;

@@ -191,3 +191,23 @@ def test_any_ratio_encodes_and_decodes_as_the_oracle(fkv, oracle_mod, N, r):
         pts = ctx.span_encode(torch.from_numpy(sym).cuda())
         assert ctx.sync_status() == -5
         assert torch.isnan(pts[0, 0]).all() and not torch.isnan(pts[0, 1]).any()
+
+
+@pytest.mark.parametrize("N", [3, 4, 9, 256, 1023, 1024])
+def test_points_beside_sector_boundaries_and_of_any_size(fkv, oracle_mod, N):
+    """Tail points a few 1e-16 to 1e-7 rad off the sector boundaries, around
+    the boundary of the 31-bit cross product's certainty, and magnitudes around
+    the ends of the range in which it is used: every symbol is the oracle's."""
+    ctx = fkv.Context(N)
+    rng = np.random.default_rng(N)
+    g = np.arange(N)
+    th = [(g + 0.5) * 2 * np.pi / N + s * d for d in (0.0, 1e-15, 1e-10, 1.9e-9, 6e-9, 1.6e-8, 1e-7) for s in (-1, 1)]
+    th = np.concatenate(th)
+    mag = 2.0 ** rng.choice([-30, -15, -14, -13.5, -1, -0.01, 0, 0.5, 15.5, 15.9, 16, 16.4, 17, 31], th.size)
+    pts = np.stack([mag * np.cos(th), mag * np.sin(th)], axis=1)
+    pts = np.concatenate([pts, [[0, 0], [0.0, -0.0], [-1, 0], [-1, -0.0], [0, 1], [0, -1], [1, 0]]])
+    n, keep = pts.shape[0] * ctx.L, pts.shape[0]
+    T, words, ts = ctx.lossy_geometry(n, 24, keep)
+    codes = torch.zeros((1, max(words, 1)), dtype=torch.int32, device="cuda")
+    dec = ctx.lossy_decode(codes, torch.from_numpy(pts[None]).cuda(), n, 24, keep).cpu().numpy()
+    assert np.array_equal(dec[0].astype(np.int32), oracle_mod.lossy_decode(pts, n, N, ctx.r, ctx.L, 24, keep))
