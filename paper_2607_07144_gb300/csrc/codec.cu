@@ -131,6 +131,10 @@ struct EncArgs {
 
 // Calls, so that the compiler does not run the rare case for every lane.
 static __device__ __noinline__ double mul_fp64(double a, double b) { return __dmul_rn(a, b); }
+static __device__ __noinline__ double mul_add_fp64(double r, double d, double v)
+{
+    return __dadd_rn(v, __dmul_rn(r, d));
+}
 static __device__ __noinline__ long long floor_fp64(double x) { return __double2ll_rd(x); }
 
 // r d rounded to nearest even, as __dmul_rn(r, d), on the integer pipe: the
@@ -150,12 +154,10 @@ struct RatioMul {
         m11 = (b << 11) | (1ull << 63);
         er = static_cast<int>(b >> 52);
     }
-    __device__ __forceinline__ double operator()(double d) const
+    // The rounded mantissa of r d, 2^52 .. 2^53, and *top, the product's
+    // top bit: |r d| = mantissa 2^(e + er + top - 2098), e d's exponent field.
+    __device__ __forceinline__ unsigned long long mantissa(unsigned hi, unsigned lo, int &top) const
     {
-        const unsigned hi = static_cast<unsigned>(__double2hiint(d)), lo = static_cast<unsigned>(__double2loint(d));
-        const int e = static_cast<int>((hi >> 20) & 0x7FFu);
-        if (static_cast<unsigned>(e - 512) >= 588u)
-            return mul_fp64(r, d);
         const unsigned dh = __funnelshift_l(lo, hi, 11) | 0x80000000u, dl = lo << 11;
         const unsigned rh = static_cast<unsigned>(m11 >> 32), rl = static_cast<unsigned>(m11);
         const unsigned long long p00 = static_cast<unsigned long long>(dl) * rl;
@@ -163,13 +165,76 @@ struct RatioMul {
         const unsigned long long b = static_cast<unsigned long long>(dl) * rh + static_cast<unsigned>(a);
         unsigned long long h = static_cast<unsigned long long>(dh) * rh + (a >> 32) + (b >> 32);
         h |= (static_cast<unsigned>(b) | static_cast<unsigned>(p00)) != 0u ? 1ull : 0ull;
-        const int top = static_cast<int>(h >> 63);
+        top = static_cast<int>(h >> 63);
         const int drop = 10 + top;
         const unsigned odd = (static_cast<unsigned>(h) >> drop) & 1u;
         h += (512u << top) - 1u + odd;
-        h >>= drop;                              // 53 bits, or 2^53 after a carry
+        return h >> drop;
+    }
+    __device__ __forceinline__ double operator()(double d) const
+    {
+        const unsigned hi = static_cast<unsigned>(__double2hiint(d)), lo = static_cast<unsigned>(__double2loint(d));
+        const int e = static_cast<int>((hi >> 20) & 0x7FFu);
+        if (static_cast<unsigned>(e - 512) >= 588u)
+            return mul_fp64(r, d);
+        int top;
+        const unsigned long long h = mantissa(hi, lo, top);
         const unsigned th = static_cast<unsigned>(h >> 32) + (static_cast<unsigned>(e + er - 1024 + top) << 20);
         return __hiloint2double(static_cast<int>(th | (hi & 0x80000000u)), static_cast<int>(static_cast<unsigned>(h)));
+    }
+    // v + r d, both operations rounded to nearest even, for |v| in [0.7, 1]:
+    // the sum as well on the integer pipe, in units of 2^-62.  v is a whole
+    // number of them; the product, below 1/2, keeps in its last bit whether
+    // bits under it were dropped, and since the sum is above 1/8 at least six
+    // bits lie between that bit and the place of rounding, which it therefore
+    // never turns.  Larger and far smaller products take the FP64 operations.
+    __device__ __forceinline__ double plus(double v, double d) const
+    {
+        const unsigned hi = static_cast<unsigned>(__double2hiint(d)), lo = static_cast<unsigned>(__double2loint(d));
+        int top;
+        const unsigned long long h = mantissa(hi, lo, top);
+        const unsigned sh = 2044u - (((hi >> 20) & 0x7FFu) + static_cast<unsigned>(er + top));
+        if (sh > 63u)
+            return mul_add_fp64(r, d, v);
+        const unsigned long long w = h << 8;
+        unsigned long long t = w >> sh;
+        t |= t << sh != w ? 1ull : 0ull;
+        const unsigned vhi = static_cast<unsigned>(__double2hiint(v)), vlo = static_cast<unsigned>(__double2loint(v));
+        const unsigned long long vm = static_cast<unsigned long long>((vhi & 0xFFFFFu) | 0x100000u) << 32 | vlo;
+        unsigned long long q = vm << (((vhi >> 20) & 0x7FFu) - 1013u);
+        q = static_cast<int>(vhi ^ hi) < 0 ? q - t : q + t;
+        const int lz = __clz(static_cast<int>(static_cast<unsigned>(q >> 32))) - 1;   // 0 .. 3
+        q <<= lz;
+        q += 511u + ((static_cast<unsigned>(q) >> 10) & 1u);
+        q >>= 10;
+        const unsigned qh = static_cast<unsigned>(q >> 32) + (static_cast<unsigned>(1022 - lz) << 20);
+        return __hiloint2double(static_cast<int>(qh | (vhi & 0x80000000u)), static_cast<int>(static_cast<unsigned>(q)));
+    }
+};
+
+// Shared vertex table of the bulk encoders: for r = 1/2 the multiples 2^j V(c)
+// at [j N + c], j = 0 .. L; else V(c) with the larger coordinate first, and
+// whether that is y.
+template <bool HALF, typename Sym>
+struct EncTable {
+    double2 v[HALF ? 4 * (kMaxSpan + 1) : vtab_len<Sym>()];
+    uint8_t turned[HALF ? 16 : vtab_len<Sym>()];
+    __device__ __forceinline__ void load(const EncArgs &a)
+    {
+        if (HALF) {
+            for (int i = threadIdx.x; i < (a.L + 1) * a.N; i += blockDim.x) {
+                const double2 p = a.V[i % a.N];
+                const double up = __longlong_as_double(static_cast<long long>(1023 + i / a.N) << 52);
+                v[i] = make_double2(p.x * up, p.y * up);
+            }
+        } else {
+            for (int i = threadIdx.x; i < a.N; i += blockDim.x) {
+                const double2 p = a.V[i];
+                const bool turn = (__double2hiint(p.y) & 0x7FFFFFFF) > (__double2hiint(p.x) & 0x7FFFFFFF);
+                v[i] = turn ? make_double2(p.y, p.x) : p;
+                turned[i] = turn;
+            }
+        }
     }
 };
 
@@ -177,10 +242,12 @@ struct RatioMul {
 // walked, the product on the integer pipe.  With r = 1/2 (HALF) the product
 // is exact, and the walk keeps S = 2^j p (scaling by powers of two commutes
 // with the roundings): S <- 2^(j+1) V + (S - 2^j V), two operations a
-// coordinate; sV then holds 2^j V(c) at [j N + c], j = 0 .. L.
+// coordinate.  Else the sum in the vertex's larger coordinate (at least
+// cos(pi/4) of its unit length) is on the integer pipe too: three FP64
+// operations a symbol, the point's coordinates turned to the vertex's order.
 template <bool HALF, typename Sym>
-__device__ __forceinline__ double2 encode_anchored(const Sym *s, int m, const double2 *sV, const EncArgs &a,
-                                                   const RatioMul &mul)
+__device__ __forceinline__ double2 encode_anchored(const Sym *s, int m, const EncTable<HALF, Sym> &tab,
+                                                   const EncArgs &a, const RatioMul &mul)
 {
     const unsigned N = static_cast<unsigned>(a.N);
     double x = 0.0, y = 0.0;
@@ -204,19 +271,29 @@ __device__ __forceinline__ double2 encode_anchored(const Sym *s, int m, const do
         x = __dmul_rn(x, up);
         y = __dmul_rn(y, up);
     }
+    unsigned turned = 0;
     for (; k < m; ++k) {
         unsigned c = s[k];
         bad |= c >= N;
         c = min(c, N - 1);
         if (HALF) {
-            const double2 v = sV[k * N + c], w = sV[(k + 1) * N + c];
+            const double2 v = tab.v[k * N + c], w = tab.v[(k + 1) * N + c];
             x = __dadd_rn(w.x, __dsub_rn(x, v.x));
             y = __dadd_rn(w.y, __dsub_rn(y, v.y));
         } else {
-            const double2 v = sV[c];
-            x = __dadd_rn(v.x, mul(__dsub_rn(x, v.x)));
-            y = __dadd_rn(v.y, mul(__dsub_rn(y, v.y)));
+            const double2 v = tab.v[c];
+            const unsigned f = tab.turned[c];
+            const bool turn = f != turned;
+            turned = f;
+            const double u = turn ? y : x, w = turn ? x : y;
+            x = mul.plus(v.x, __dsub_rn(u, v.x));
+            y = __dadd_rn(v.y, mul(__dsub_rn(w, v.y)));
         }
+    }
+    if (turned) {
+        const double u = x;
+        x = y;
+        y = u;
     }
     if (HALF) {
         const double down = __longlong_as_double(static_cast<long long>(1023 - m) << 52);
@@ -225,21 +302,6 @@ __device__ __forceinline__ double2 encode_anchored(const Sym *s, int m, const do
     }
     const double nan = __longlong_as_double(-1ll);
     return bad ? make_double2(nan, nan) : make_double2(x, y);
-}
-
-// Shared vertex table of the bulk encoders: V, or for r = 1/2 its 2^j multiples.
-template <bool HALF, typename Sym>
-__host__ __device__ constexpr int enc_table_len() { return HALF ? 4 * (kMaxSpan + 1) : vtab_len<Sym>(); }
-
-template <bool HALF>
-__device__ __forceinline__ void load_vertices(double2 *sV, const EncArgs &a)
-{
-    const int rows = HALF ? a.L + 1 : 1;
-    for (int i = threadIdx.x; i < rows * a.N; i += blockDim.x) {
-        const double2 v = a.V[i % a.N];
-        const double up = __longlong_as_double(static_cast<long long>(1023 + i / a.N) << 52);
-        sV[i] = HALF ? make_double2(v.x * up, v.y * up) : v;
-    }
 }
 
 // The table of points after k symbols from the anchor: entry i's symbols are
@@ -259,22 +321,25 @@ __global__ void __launch_bounds__(kThreads) k_pre_table(const double2 *__restric
     pre[i] = encode_span(s, k, V, N, r, 0.0, 0.0);
 }
 
-// Bulk encoding, one span per thread.  Bound by the FP64 pipe: four binary64
-// operations for each symbol after the table's, so (6 - 2) 4 = 16 a span for
-// N = 256 where the plain walk takes 36.  128 streams of 392,784 symbols: 0.278 ms
-// (92 % of that pipe), 0.593 ms without either, 0.397 ms with the table alone;
-// 16.8 M ragged symbols of N = 16, 0.111 ms against 0.204.
+// Bulk encoding, one span per thread.  Bound by the FP64 pipe and, a quarter
+// below it, by instruction issue: three binary64 operations for each symbol
+// after the table's, so (6 - 2) 3 = 12 a span for N = 256 where the plain walk
+// takes 36.  128 streams of 392,784 symbols: 0.226 ms; 0.593 ms by the plain
+// walk, 0.397 with the table, 0.278 with the products on the integer pipe too,
+// 0.234 with all but the NaN and table comparisons off the FP64 pipe.
+// Persistent blocks with warp-wide staging: 0.258.  16.8 M ragged symbols of
+// N = 16: 0.091 ms against 0.204.
 template <bool HALF, typename Sym>
 __global__ void __launch_bounds__(kThreads)
 k_span_encode(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, int64_t spans, int bps,
               double2 *__restrict__ pts, int64_t pt_stride, const EncArgs a, unsigned *status)
 {
     __shared__ __align__(16) uint8_t sbuf[stage_bytes<Sym>()];
-    __shared__ double2 sV[enc_table_len<HALF, Sym>()];
+    __shared__ EncTable<HALF, Sym> tab;
     const int L = a.L;
     const int64_t stream = blockIdx.x / bps;
     const int64_t s0 = static_cast<int64_t>(blockIdx.x % bps) * kThreads;
-    load_vertices<HALF>(sV, a);
+    tab.load(a);
     const int64_t b = s0 * L;
     const int64_t e = min(n, (s0 + kThreads) * L);
     const int off = stage_in(sbuf, reinterpret_cast<const uint8_t *>(sym + stream * sym_stride + b),
@@ -284,8 +349,8 @@ k_span_encode(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, int64_
     if (s < spans) {
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
         const Sym *my = reinterpret_cast<const Sym *>(sbuf + off) + threadIdx.x * L;
-        const double2 p = encode_anchored<HALF>(my, m, sV, a, RatioMul(a.r));
-        if (isnan(p.x))   // a symbol >= N
+        const double2 p = encode_anchored<HALF>(my, m, tab, a, RatioMul(a.r));
+        if (__double2hiint(p.x) == -1)   // NaN: a symbol >= N
             atomicOr(status, FKV_ST_CORRUPT);
         pts[stream * pt_stride + s] = p;
     }
@@ -302,8 +367,8 @@ k_span_encode_flat(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, u
                    fkvd::FastDiv div_spans, double2 *__restrict__ pts, int64_t pt_stride, const EncArgs a,
                    unsigned *status)
 {
-    __shared__ double2 sV[enc_table_len<HALF, Sym>()];
-    load_vertices<HALF>(sV, a);
+    __shared__ EncTable<HALF, Sym> tab;
+    tab.load(a);
     __syncthreads();
     const unsigned t = blockIdx.x * kThreads + threadIdx.x;
     if (t >= total)
@@ -311,8 +376,8 @@ k_span_encode_flat(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, u
     const unsigned stream = div_spans.div(t), s = t - stream * spans;
     const int64_t b = static_cast<int64_t>(s) * a.L;
     const int m = static_cast<int>(min(static_cast<int64_t>(a.L), n - b));
-    const double2 p = encode_anchored<HALF>(sym + stream * sym_stride + b, m, sV, a, RatioMul(a.r));
-    if (isnan(p.x))   // a symbol >= N
+    const double2 p = encode_anchored<HALF>(sym + stream * sym_stride + b, m, tab, a, RatioMul(a.r));
+    if (__double2hiint(p.x) == -1)   // NaN: a symbol >= N
         atomicOr(status, FKV_ST_CORRUPT);
     pts[stream * pt_stride + s] = p;
 }
@@ -722,10 +787,10 @@ __global__ void __launch_bounds__(kThreads)
 k_span_encode_ragged(const Sym *__restrict__ sym, const int64_t *__restrict__ so, int64_t n_streams,
                      double2 *__restrict__ pts, const int64_t *__restrict__ po, const EncArgs a, unsigned *status)
 {
-    __shared__ double2 sV[enc_table_len<HALF, Sym>()];
+    __shared__ EncTable<HALF, Sym> tab;
     const int L = a.L;
     const RatioMul mul(a.r);
-    load_vertices<HALF>(sV, a);
+    tab.load(a);
     __syncthreads();
     ragged_check(so, po, n_streams, L, status);
     const int64_t g0 = __ldg(&po[0]), g1 = __ldg(&po[n_streams]);
@@ -739,8 +804,8 @@ k_span_encode_ragged(const Sym *__restrict__ sym, const int64_t *__restrict__ so
         if (s < 0 || s * L >= n)
             continue;                       // a slot past the stream's last span
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
-        const double2 p = encode_anchored<HALF>(sym + __ldg(&so[i]) + s * L, m, sV, a, mul);
-        if (isnan(p.x))
+        const double2 p = encode_anchored<HALF>(sym + __ldg(&so[i]) + s * L, m, tab, a, mul);
+        if (__double2hiint(p.x) == -1)
             atomicOr(status, FKV_ST_CORRUPT);
         pts[g] = p;
     }

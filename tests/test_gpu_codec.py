@@ -223,3 +223,17 @@ def test_symbol_codec_stress_full_size(fkv, oracle_mod, N, dist):
     got = ctx.read(pts, n, req)
     assert torch.equal(got, sym[req[:, 0], req[:, 1]])
     assert ctx.sync_status() == 0
+
+
+@pytest.mark.parametrize("N", [3, 5, 6, 8, 9, 33, 100, 255])
+def test_many_random_spans_encode_bit_exact(fkv, oracle_mod, N):
+    """The encoder's products and half of its sums leave the FP64 pipe: enough
+    spans that roundings up, down and to even, both signs, both orders of a
+    vertex's coordinates and products too large or too small for the integer
+    sum all occur."""
+    ctx = _ctx(fkv, N)
+    n = 20000 * ctx.L
+    sym = _rand_streams(N, 2, n, 77 + N)
+    pts = ctx.span_encode(torch.from_numpy(sym).cuda())
+    want = _oracle_points(oracle_mod, sym, N, ctx.r, ctx.L)
+    assert np.array_equal(pts.cpu().numpy().view(np.uint64), want.view(np.uint64))
