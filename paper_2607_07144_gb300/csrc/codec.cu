@@ -418,7 +418,7 @@ struct ChunkWalk {
 // dec_threads spans (chunk = stream * bps + span block), blockIdx.x,
 // + gridDim.x, ...; each thread stores its span's symbols directly, so the
 // chunks need no block barrier.
-template <typename Sym>
+template <typename Sym, fkvdec::Cell CELL>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_span_decode(const double2 *__restrict__ pts, int64_t n, int64_t pt_stride, int64_t spans, int bps,
               int64_t n_chunks, Sym *__restrict__ sym, int64_t sym_stride, const fkv_decconst *__restrict__ dc,
@@ -442,7 +442,7 @@ k_span_decode(const double2 *__restrict__ pts, int64_t n, int64_t pt_stride, int
         if (s < spans) {
             const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
             dst += m - 1;
-            if (!fkvdec::decode_point(t, p, m, __ldg(&dc->alim[m]), [&] {
+            if (!fkvdec::decode_point<CELL>(t, p, m, __ldg(&dc->alim[m]), [&] {
                     return [=](int j, int c) { dst[-j] = static_cast<Sym>(c); };
                 }))
                 atomicOr(status, FKV_ST_CORRUPT);
@@ -453,7 +453,7 @@ k_span_decode(const double2 *__restrict__ pts, int64_t n, int64_t pt_stride, int
 
 // Decode 256 spans of one stream (chunk `ck` of the n_streams * bps chunks)
 // into sbuf (one span per thread, symbol i of the chunk at sbuf[i]).
-template <typename Sym>
+template <fkvdec::Cell CELL, typename Sym>
 __device__ __forceinline__ void decode_chunk(const fkvdec::Tables &t, const double2 *__restrict__ pts, int64_t n,
                                              int64_t pt_stride, int64_t spans, int64_t stream, int64_t s0,
                                              Sym *sbuf, const fkv_decconst *__restrict__ dc, int L,
@@ -463,7 +463,7 @@ __device__ __forceinline__ void decode_chunk(const fkvdec::Tables &t, const doub
     if (s < spans) {
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
         Sym *my = sbuf + threadIdx.x * L + m - 1;
-        if (!fkvdec::decode_point(t, pts[stream * pt_stride + s], m, __ldg(&dc->alim[m]), [&] {
+        if (!fkvdec::decode_point<CELL>(t, pts[stream * pt_stride + s], m, __ldg(&dc->alim[m]), [&] {
                 return [=](int j, int c) { my[-j] = static_cast<Sym>(c); };
             }))
             atomicOr(status, FKV_ST_CORRUPT);
@@ -475,7 +475,7 @@ __device__ __forceinline__ void decode_chunk(const fkvdec::Tables &t, const doub
 // since a thread's own span would otherwise be a run of scattered byte
 // stores.  Persistent: chunk = stream * bps + span block, blockIdx.x,
 // + gridDim.x, ...
-template <typename Sym>
+template <typename Sym, fkvdec::Cell CELL>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_span_decode_staged(const double2 *__restrict__ pts, int64_t n, int64_t pt_stride, int64_t spans, int bps,
               int64_t n_chunks, Sym *__restrict__ sym, int64_t sym_stride, const fkv_decconst *__restrict__ dc,
@@ -494,7 +494,7 @@ k_span_decode_staged(const double2 *__restrict__ pts, int64_t n, int64_t pt_stri
         const int64_t e = min(n, (s0 + TPB) * L);
         uint8_t *dst = reinterpret_cast<uint8_t *>(sym + stream * sym_stride + b);
         const int off = static_cast<int>(reinterpret_cast<uintptr_t>(dst) & 15);
-        decode_chunk(t, pts, n, pt_stride, spans, stream, s0, reinterpret_cast<Sym *>(sbuf + off), dc, L, status);
+        decode_chunk<CELL>(t, pts, n, pt_stride, spans, stream, s0, reinterpret_cast<Sym *>(sbuf + off), dc, L, status);
         __syncthreads();
         stage_out(dst, sbuf, static_cast<int>(e - b) * static_cast<int>(sizeof(Sym)), off);
         __syncthreads();
@@ -510,7 +510,7 @@ k_span_decode_staged(const double2 *__restrict__ pts, int64_t n, int64_t pt_stri
 // offset plus record x stages, stepping back one symbol of the record (and a
 // record at its start) per symbol.  Positions inside a stream are 32-bit (the
 // launcher keeps a stream below 2^31 symbols) and the span's last record comes
-// from a multiply-high division.
+// from a multiply-high division.  Codebooks come with N = 256 or 1024: sectors.
 template <typename Sym>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_span_decode_planar(const double2 *__restrict__ pts, unsigned n_rec, int64_t pt_stride, unsigned spans, int bps,
@@ -551,7 +551,7 @@ k_span_decode_planar(const double2 *__restrict__ pts, unsigned n_rec, int64_t pt
             const unsigned q = first + m - 1;             // the span's last symbol
             const unsigned rec = div_r.div(q);
             const int o = static_cast<int>(q - rec * static_cast<unsigned>(R));
-            if (!fkvdec::decode_point(t, p, m, m == L ? lim_full : __ldg(&dc->alim[m]), [&] {
+            if (!fkvdec::decode_point<fkvdec::kSectors>(t, p, m, m == L ? lim_full : __ldg(&dc->alim[m]), [&] {
                     return [=, o = o, rec = rec](int, int c) mutable {
                         const unsigned S = o < nk ? SK : SV;
                         base[poff[o] + rec * S] = static_cast<Sym>(c);
@@ -585,9 +585,26 @@ struct SuffixQuery {
     int len;
 };
 
+// Whether the last symbols of the span stored as p are the query: step j of
+// the walk recovers the query's symbol len - 1 - j.  A call: few points are
+// candidates, and inlined the walks' registers halve the scan's warps.
+static __device__ __noinline__ bool ends_in(const fkvdec::Tables &t, double2 p, const SuffixQuery &qy)
+{
+    long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
+    bool eq = true;
+    auto same = [&](int j, int c) { eq = eq && c == qy.sym[qy.len - 1 - j]; };
+    if (t.N > 8)
+        fkvdec::walk<fkvdec::kSectors>(t, X, Y, qy.len, same);
+    else if (t.N == 4)
+        fkvdec::walk<fkvdec::kAxes>(t, X, Y, qy.len, same);
+    else
+        fkvdec::walk<fkvdec::kScores>(t, X, Y, qy.len, same);
+    return eq;
+}
+
 __global__ void __launch_bounds__(kThreads)
 k_suffix_search(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, int64_t pt_stride, int64_t spans,
-                const SuffixQuery qy, double thr, double thr2, const double2 *__restrict__ V, double r,
+                const __grid_constant__ SuffixQuery qy, double thr, double thr2, const double2 *__restrict__ V, double r,
                 const fkv_decconst *__restrict__ dc, const longlong2 *__restrict__ T, int N, int L,
                 long long *__restrict__ out, long long cap, unsigned long long *__restrict__ counts)
 {
@@ -650,11 +667,7 @@ k_suffix_search(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, i
                 const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
                 if (d2 <= thr2) {
                     atomicAdd(&counts[1], 1ull);
-                    long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-                    bool eq = true;
-                    // step j recovers the span's symbol m - 1 - j, the query's l - 1 - j
-                    fkvdec::walk(t, X, Y, l, [&](int j, int c) { eq = eq && c == qy.sym[l - 1 - j]; });
-                    if (eq) {
+                    if (ends_in(t, p, qy)) {
                         const unsigned long long slot = atomicAdd(&counts[0], 1ull);
                         if (static_cast<long long>(slot) < cap) {
                             out[2 * slot] = su[i];
@@ -670,7 +683,7 @@ k_suffix_search(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, i
 // Sec. 2 random access: one request per thread, decoding only its span down
 // to the requested offset.  Persistent: a block loads the decoder tables once
 // and takes requests blockIdx.x * TPB + threadIdx.x, + gridDim.x * TPB, ...
-template <typename Sym>
+template <typename Sym, fkvdec::Cell CELL>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_read(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, int64_t pt_stride,
        const int64_t *__restrict__ req, int64_t n_req, Sym *__restrict__ out,
@@ -679,23 +692,37 @@ k_read(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, int64_t pt
     extern __shared__ __align__(16) uint8_t dsm[];
     const fkvdec::Tables t = fkvdec::load(dc, T, N, L, dsm);
     __syncthreads();
-    constexpr int TPB = dec_threads<Sym>();
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * TPB + threadIdx.x; q < n_req;
-         q += static_cast<int64_t>(gridDim.x) * TPB) {
-        const int64_t st = req[2 * q], pos = req[2 * q + 1];
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * dec_threads<Sym>();
+    int64_t q = static_cast<int64_t>(blockIdx.x) * dec_threads<Sym>() + threadIdx.x;
+    int64_t st = 0, pos = 0;
+    if (q < n_req) {
+        st = req[2 * q];
+        pos = req[2 * q + 1];
+    }
+    while (q < n_req) {
+        // the next request is on its way during this one's walk
+        const int64_t qn = q + stride;
+        int64_t stn = 0, posn = 0;
+        if (qn < n_req) {
+            stn = req[2 * qn];
+            posn = req[2 * qn + 1];
+        }
         if (st < 0 || st >= n_streams || pos < 0 || pos >= n) {
             out[q] = static_cast<Sym>(~0u);
             atomicOr(status, FKV_ST_RANGE);
-            continue;
+        } else {
+            const int64_t u = pos / L;
+            const int o = static_cast<int>(pos - u * L);
+            const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
+            const double2 p = pts[st * pt_stride + u];
+            long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
+            int sym = 0;
+            fkvdec::walk<CELL>(t, X, Y, m - o, [&](int j, int c) { sym = c; });
+            out[q] = static_cast<Sym>(sym);
         }
-        const int64_t u = pos / L;
-        const int o = static_cast<int>(pos - u * L);
-        const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
-        const double2 p = pts[st * pt_stride + u];
-        long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
-        int sym = 0;
-        fkvdec::walk(t, X, Y, m - o, [&](int j, int c) { sym = c; });
-        out[q] = static_cast<Sym>(sym);
+        q = qn;
+        st = stn;
+        pos = posn;
     }
 }
 
@@ -811,7 +838,30 @@ k_span_encode_ragged(const Sym *__restrict__ sym, const int64_t *__restrict__ so
     }
 }
 
-template <typename Sym>
+// Receiver of a walk that stores m symbols from dst, last to first; WORDS: bytes
+// go out as the aligned words they make up.
+template <bool WORDS, typename Sym>
+__device__ __forceinline__ auto span_writer(Sym *dst, int m)
+{
+    if constexpr (!WORDS) {
+        return [=](int j, int c) { dst[m - 1 - j] = static_cast<Sym>(c); };
+    } else {
+        return [=, acc = 0u](int j, int c) mutable {
+            acc = (acc << 8) | static_cast<unsigned>(c);
+            uint8_t *at = dst + (m - 1 - j);
+            const unsigned in_word = static_cast<unsigned>(reinterpret_cast<uintptr_t>(at)) & 3u;
+            if (in_word == 0u && j >= 3) {
+                *reinterpret_cast<unsigned *>(at) = acc;
+            } else if (in_word == 0u || j == m - 1) {
+                const int cnt = min(j + 1, 4 - static_cast<int>(in_word));
+                for (int k = 0; k < cnt; ++k)
+                    at[k] = static_cast<uint8_t>(acc >> (8 * k));
+            }
+        };
+    }
+}
+
+template <typename Sym, fkvdec::Cell CELL, bool WORDS>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_span_decode_ragged(const double2 *__restrict__ pts, const int64_t *__restrict__ po, int64_t n_streams,
                      Sym *__restrict__ sym, const int64_t *__restrict__ so, const fkv_decconst *__restrict__ dc,
@@ -832,17 +882,15 @@ k_span_decode_ragged(const double2 *__restrict__ pts, const int64_t *__restrict_
         if (s < 0 || s * L >= n)
             continue;
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
-        Sym *dst = sym + __ldg(&so[i]) + s * L + m - 1;
-        if (!fkvdec::decode_point(t, pts[g], m, __ldg(&dc->alim[m]), [&] {
-                return [=](int j, int c) { dst[-j] = static_cast<Sym>(c); };
-            }))
+        Sym *dst = sym + __ldg(&so[i]) + s * L;
+        if (!fkvdec::decode_point<CELL>(t, pts[g], m, __ldg(&dc->alim[m]), [&] { return span_writer<WORDS>(dst, m); }))
             atomicOr(status, FKV_ST_CORRUPT);
     }
 }
 
 // Random access into a ragged batch: request q = (stream, position), the
 // position checked against that stream's own length.
-template <typename Sym>
+template <typename Sym, fkvdec::Cell CELL>
 __global__ void __launch_bounds__(dec_threads<Sym>())
 k_read_ragged(const double2 *__restrict__ pts, const int64_t *__restrict__ po, const int64_t *__restrict__ so,
               int64_t n_streams, const int64_t *__restrict__ req, int64_t n_req, Sym *__restrict__ out,
@@ -866,7 +914,7 @@ k_read_ragged(const double2 *__restrict__ pts, const int64_t *__restrict__ po, c
         const double2 p = pts[__ldg(&po[st]) + u];
         long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
         int c = 0;
-        fkvdec::walk(t, X, Y, m - o, [&](int, int cc) { c = cc; });
+        fkvdec::walk<CELL>(t, X, Y, m - o, [&](int, int cc) { c = cc; });
         out[q] = static_cast<Sym>(c);
     }
 }
@@ -1343,21 +1391,20 @@ cudaError_t span_decode_t(const fkv_ctx *c, const double *pts, int64_t n_streams
         return cudaErrorInvalidConfiguration;
     // spans of up to 8 symbols: each thread stores its own; longer ones: staged
     const bool direct = c->L <= 8;
-    const void *kern = direct ? reinterpret_cast<const void *>(k_span_decode<Sym>)
-                              : reinterpret_cast<const void *>(k_span_decode_staged<Sym>);
+    auto kern = direct ? k_span_decode<Sym, fkvdec::kSectors> : k_span_decode_staged<Sym, fkvdec::kSectors>;
+    if constexpr (sizeof(Sym) == 1) {
+        if (c->N == 4)
+            kern = direct ? k_span_decode<Sym, fkvdec::kAxes> : k_span_decode_staged<Sym, fkvdec::kAxes>;
+        else if (c->N <= 8)
+            kern = direct ? k_span_decode<Sym, fkvdec::kScores> : k_span_decode_staged<Sym, fkvdec::kScores>;
+    }
     const int smem = tables_bytes(c->N, c->L) + (direct ? 0 : dec_stage_bytes<Sym>(c->L));
     unsigned grid = 0;
-    cudaError_t e = decode_grid(c, kern, smem, n_chunks, &grid, TPB);
+    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(kern), smem, n_chunks, &grid, TPB);
     if (e != cudaSuccess)
         return e;
-    const double2 *p2 = reinterpret_cast<const double2 *>(pts);
-    if (direct)
-        k_span_decode<Sym><<<grid, TPB, smem, st>>>(p2, n, pt_stride, spans, static_cast<int>(bps), n_chunks, sym,
-                                                         sym_stride, c->d_dec, c->d_T, c->N, c->L, c->d_status);
-    else
-        k_span_decode_staged<Sym><<<grid, TPB, smem, st>>>(p2, n, pt_stride, spans, static_cast<int>(bps), n_chunks,
-                                                                sym, sym_stride, c->d_dec, c->d_T, c->N, c->L,
-                                                                c->d_status);
+    kern<<<grid, TPB, smem, st>>>(reinterpret_cast<const double2 *>(pts), n, pt_stride, spans, static_cast<int>(bps),
+                                  n_chunks, sym, sym_stride, c->d_dec, c->d_T, c->N, c->L, c->d_status);
     return cudaGetLastError();
 }
 
@@ -1446,12 +1493,17 @@ cudaError_t read_t(const fkv_ctx *c, const double *pts, int64_t n_streams, int64
     const int64_t blocks = cdiv(n_req, TPB);
     if (blocks == 0)
         return cudaSuccess;
+    auto kern = k_read<Sym, fkvdec::kSectors>;
+    if constexpr (sizeof(Sym) == 1) {
+        if (c->N <= 8)
+            kern = c->N == 4 ? k_read<Sym, fkvdec::kAxes> : k_read<Sym, fkvdec::kScores>;
+    }
     const int smem = tables_bytes(c->N, c->L);
     unsigned grid = 0;
-    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(k_read<Sym>), smem, blocks, &grid, TPB);
+    cudaError_t e = decode_grid(c, reinterpret_cast<const void *>(kern), smem, blocks, &grid, TPB);
     if (e != cudaSuccess)
         return e;
-    k_read<Sym><<<grid, TPB, smem, st>>>(
+    kern<<<grid, TPB, smem, st>>>(
         reinterpret_cast<const double2 *>(pts), n_streams, n, pt_stride, req, n_req, out, c->d_dec, c->d_T,
         c->N, c->L, c->d_status);
     return cudaGetLastError();
@@ -1652,15 +1704,29 @@ template <typename Sym>
 cudaError_t decode_ragged_t(const fkv_ctx *c, const double *pts, const int64_t *po, int64_t n_streams, Sym *sym,
                             const int64_t *so, cudaStream_t st)
 {
+    auto kern = k_span_decode_ragged<Sym, fkvdec::kSectors, false>;
+    if constexpr (sizeof(Sym) == 1) {
+        // words pay from longer spans on: 134 M symbols as words and as bytes,
+        // sectors: 0.385 / 0.349 ms at 12 symbols a span, 0.358 / 0.394 at 16,
+        // 0.354 / 0.546 at 22; scores: 0.658 / 0.630 at 24, 0.533 / 0.717 at 31
+        // (their walk, not the stores, bounds the shorter ones)
+        const bool words = c->L >= (c->N <= 8 && c->N != 4 ? 28 : 16);
+        if (c->N == 4)
+            kern = words ? k_span_decode_ragged<Sym, fkvdec::kAxes, true>
+                         : k_span_decode_ragged<Sym, fkvdec::kAxes, false>;
+        else if (c->N <= 8)
+            kern = words ? k_span_decode_ragged<Sym, fkvdec::kScores, true>
+                         : k_span_decode_ragged<Sym, fkvdec::kScores, false>;
+        else if (words)
+            kern = k_span_decode_ragged<Sym, fkvdec::kSectors, true>;
+    }
     const int smem = tables_bytes(c->N, c->L);
     unsigned grid = 0;
-    cudaError_t e = ragged_decoder_grid<Sym>(c, reinterpret_cast<const void *>(k_span_decode_ragged<Sym>), smem,
-                                             &grid);
+    cudaError_t e = ragged_decoder_grid<Sym>(c, reinterpret_cast<const void *>(kern), smem, &grid);
     if (e != cudaSuccess)
         return e;
-    k_span_decode_ragged<Sym><<<grid, dec_threads<Sym>(), smem, st>>>(reinterpret_cast<const double2 *>(pts), po,
-                                                                      n_streams, sym, so, c->d_dec, c->d_T, c->N,
-                                                                      c->L, c->d_status);
+    kern<<<grid, dec_threads<Sym>(), smem, st>>>(reinterpret_cast<const double2 *>(pts), po, n_streams, sym, so,
+                                                 c->d_dec, c->d_T, c->N, c->L, c->d_status);
     return cudaGetLastError();
 }
 
@@ -1668,17 +1734,21 @@ template <typename Sym>
 cudaError_t read_ragged_t(const fkv_ctx *c, const double *pts, const int64_t *po, const int64_t *so,
                           int64_t n_streams, const int64_t *req, int64_t n_req, Sym *out, cudaStream_t st)
 {
+    auto kern = k_read_ragged<Sym, fkvdec::kSectors>;
+    if constexpr (sizeof(Sym) == 1) {
+        if (c->N <= 8)
+            kern = c->N == 4 ? k_read_ragged<Sym, fkvdec::kAxes> : k_read_ragged<Sym, fkvdec::kScores>;
+    }
     const int smem = tables_bytes(c->N, c->L);
     unsigned grid = 0;
-    cudaError_t e = ragged_decoder_grid<Sym>(c, reinterpret_cast<const void *>(k_read_ragged<Sym>), smem, &grid);
+    cudaError_t e = ragged_decoder_grid<Sym>(c, reinterpret_cast<const void *>(kern), smem, &grid);
     if (e != cudaSuccess)
         return e;
     const int64_t need = cdiv(n_req, dec_threads<Sym>());
     if (static_cast<int64_t>(grid) > need)
         grid = static_cast<unsigned>(need);
-    k_read_ragged<Sym><<<grid, dec_threads<Sym>(), smem, st>>>(reinterpret_cast<const double2 *>(pts), po, so,
-                                                               n_streams, req, n_req, out, c->d_dec, c->d_T, c->N,
-                                                               c->L, c->d_status);
+    kern<<<grid, dec_threads<Sym>(), smem, st>>>(reinterpret_cast<const double2 *>(pts), po, so, n_streams, req, n_req,
+                                                 out, c->d_dec, c->d_T, c->N, c->L, c->d_status);
     return cudaGetLastError();
 }
 

@@ -174,34 +174,41 @@ __device__ __forceinline__ int classify_sector(const Tables &t, long long X, lon
     return d > 0 ? c : (d < 0 ? c1 : min(c, c1));
 }
 
-__device__ __forceinline__ int classify(const Tables &t, long long X, long long Y)
+__device__ __forceinline__ int classify_axes(long long X, long long Y)
 {
-    const int N = t.N;
-    if (N == 4) {
-        const long long ax = X < 0 ? -X : X, ay = Y < 0 ? -Y : Y;
-        if (ax >= ay)
-            return X >= 0 ? 0 : 2;
-        return Y >= 0 ? 1 : 3;
-    }
+    const long long ax = X < 0 ? -X : X, ay = Y < 0 ? -Y : Y;
+    if (ax >= ay)
+        return X >= 0 ? 0 : 2;
+    return Y >= 0 ? 1 : 3;
+}
+
+template <int N>
+__device__ __forceinline__ int classify_scores(const Tables &t, long long X, long long Y)
+{
     float qx, qy;
     direction(X, Y, qx, qy);
-    if (N <= 8) {
-        float b1 = -INFINITY, b2 = -INFINITY;
-        int bi = 0;
-        for (int c = 0; c < N; ++c) {
-            const float s = fmaf(qx, t.vf[c].x, qy * t.vf[c].y);
-            if (s > b1) {
-                b2 = b1;
-                b1 = s;
-                bi = c;
-            } else if (s > b2) {
-                b2 = s;
-            }
+    float b1 = -INFINITY, b2 = -INFINITY;
+    int bi = 0;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        const float s = fmaf(qx, t.vf[c].x, qy * t.vf[c].y);
+        if (s > b1) {
+            b2 = b1;
+            b1 = s;
+            bi = c;
+        } else if (s > b2) {
+            b2 = s;
         }
-        if (b1 - b2 > 0x1p-18f * (fabsf(qx) + fabsf(qy)))
-            return bi;
-        return classify_exact_all(t, X, Y);
     }
+    if (b1 - b2 > 0x1p-18f * (fabsf(qx) + fabsf(qy)))
+        return bi;
+    return classify_exact_all(t, X, Y);
+}
+
+__device__ __forceinline__ int classify_angle(const Tables &t, long long X, long long Y)
+{
+    float qx, qy;
+    direction(X, Y, qx, qy);
     return classify_sector(t, X, Y, qx, qy);
 }
 
@@ -235,23 +242,46 @@ __device__ __forceinline__ long long to_q62(double v)
 // step j = 0 .. steps-1 emits the symbol at offset m-1-j of the span.
 // `emit(j, c)` receives each symbol.  Any Q, of any size: random reads,
 // retrieval, and spans that are no code point.
-template <class Emit>
-__device__ __forceinline__ void walk(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
+template <class Classify, class Emit>
+__device__ __forceinline__ void walk_by(const Tables &t, long long &X, long long &Y, int steps, Classify classify,
+                                        Emit emit)
 {
-    const int N = t.N;
-    for (int j = 0; j < steps; ++j) {
-        const int c = classify(t, X, Y);
+    const longlong2 *T = t.T;
+    for (int j = 0; j < steps; ++j, T += t.N) {
+        const int c = classify(X, Y);
         emit(j, c);
-        const longlong2 w = t.T[j * N + c];
+        const longlong2 w = T[c];
         X = static_cast<long long>(static_cast<unsigned long long>(X) - static_cast<unsigned long long>(w.x));
         Y = static_cast<long long>(static_cast<unsigned long long>(Y) - static_cast<unsigned long long>(w.y));
+    }
+}
+
+// The cell test of an alphabet: sectors (N > 8), the axes (N = 4), scores.
+enum Cell { kSectors, kAxes, kScores };
+
+template <Cell CELL, class Emit>
+__device__ __forceinline__ void walk(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
+{
+    auto by = [&](auto classify) { walk_by(t, X, Y, steps, classify, emit); };
+    if (CELL == kSectors) {
+        by([&](long long x, long long y) { return classify_angle(t, x, y); });
+    } else if (CELL == kAxes) {
+        by([](long long x, long long y) { return classify_axes(x, y); });
+    } else {
+        switch (t.N) {
+        case 3: by([&](long long x, long long y) { return classify_scores<3>(t, x, y); }); break;
+        case 5: by([&](long long x, long long y) { return classify_scores<5>(t, x, y); }); break;
+        case 6: by([&](long long x, long long y) { return classify_scores<6>(t, x, y); }); break;
+        case 7: by([&](long long x, long long y) { return classify_scores<7>(t, x, y); }); break;
+        default: by([&](long long x, long long y) { return classify_scores<8>(t, x, y); }); break;
+        }
     }
 }
 
 template <class Emit>
 static __device__ __noinline__ void walk_any(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
 {
-    walk(t, X, Y, steps, emit);
+    walk<kSectors>(t, X, Y, steps, emit);
 }
 
 // The walk of a code point for N > 8, where Voronoi regions are sectors.  A
@@ -288,13 +318,18 @@ __device__ __forceinline__ void walk_sectors(const Tables &t, long long &X, long
 // Decode the m symbols of the span stored as p.  start() gives the receiver
 // emit(j, c) of a walk from its beginning; false when the walk does not end at
 // the anchor (|Q_0| <= lim), the symbols then being those of the general walk.
-template <class Start>
+// The decoders and random reads are compiled for each cell test.  With all of
+// them in one kernel, chosen at each symbol, 134 M symbols took 0.402 ms for
+// N = 3 (0.326 by itself), 0.224 for N = 4 (0.170), 0.672 for N = 8 (0.549),
+// 0.416 for N = 256 (0.413); 4.2 M random reads 0.648 / 0.297 / 0.459 / 0.111
+// (0.432 / 0.218 / 0.402 / 0.110).
+template <Cell CELL, class Start>
 __device__ __forceinline__ bool decode_point(const Tables &t, double2 p, int m, long long lim, Start start)
 {
     long long X = to_q62(p.x), Y = to_q62(p.y);
     auto off = [&] { return X > lim || X < -lim || Y > lim || Y < -lim; };
-    if (t.N <= 8) {
-        walk(t, X, Y, m, start());
+    if (CELL != kSectors) {
+        walk<CELL>(t, X, Y, m, start());
         return !off();
     }
     walk_sectors(t, X, Y, m, start());

@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kReadWarps * 32, 3) k_read_kv(const ReadArgs a
         for (int64_t u = u0 + lane; u <= u1; u += kTeam) {
             const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
             const int last = static_cast<int>(u * L - sym0) + m - 1;
-            bad |= !fkvdec::decode_point(t, a.pts[st * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
+            bad |= !fkvdec::decode_point<fkvdec::kSectors>(t, a.pts[st * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
                 return [=](int j, int c) {
                     const int pos = last - j;
                     if (pos >= 0 && pos < R)
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(256) k_read_syms(const ReadArgs a, int spr)
         const int m = static_cast<int>(min(static_cast<int64_t>(L), n - u * L));
         const int last = static_cast<int>(u * L - sym0) + m - 1;
         Sym *dst = scr + i * R;
-        if (!fkvdec::decode_point(t, a.pts[e.y * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
+        if (!fkvdec::decode_point<fkvdec::kSectors>(t, a.pts[e.y * a.pt_stride + u], m, __ldg(&a.dec->alim[m]), [&] {
                 return [=](int j, int c) {
                     const int pos = last - j;
                     if (pos >= 0 && pos < R)

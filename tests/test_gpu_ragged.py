@@ -102,3 +102,30 @@ def test_ragged_inconsistent_offsets_report_range(fkv):
     with pytest.raises(fkv.FkvError) as ei:
         ctx.span_encode_ragged(sym, so, po, pts=pts.view(-1)[1:])          # points not 16-byte aligned
     assert ei.value.code == -1
+
+
+@pytest.mark.parametrize("N,L", [(3, 28), (3, 27), (4, 16), (4, 15), (4, 44), (5, 31), (6, 27), (7, 25), (8, 24),
+                                 (9, 22), (16, 16), (16, 15)])
+def test_ragged_decode_writes_its_own_bytes_only(fkv, oracle_mod, N, L):
+    """Every alphabet of its own cell test, spans on both sides of where bytes
+    are stored as words, streams of every length and alignment: what is decoded
+    equals the symbols, no byte outside is touched, and reads agree."""
+    ctx = fkv.Context(N, span_len=L)
+    rng = np.random.default_rng(100 * N + L)
+    ln = np.array(list(range(1, 2 * L + 3)) + [257 * L + 1, 40 * L + 3], np.int64)
+    flat = rng.integers(0, N, size=int(ln.sum())).astype(np.uint8)
+    so, po = ctx.ragged_offsets(ln)
+    pts = ctx.span_encode_ragged(torch.from_numpy(flat).cuda(), so, po)
+    for shift in range(4):
+        out = torch.full((shift + flat.size + 9,), 0xEE, dtype=torch.uint8, device="cuda")
+        ctx.span_decode_ragged(pts, po, so, sym=out[shift:shift + flat.size])
+        h = out.cpu().numpy()
+        assert np.array_equal(h[shift:shift + flat.size], flat)
+        assert np.all(h[:shift] == 0xEE) and np.all(h[shift + flat.size:] == 0xEE)
+    n = int(ln[-2])
+    s = flat[int(ln[:-2].sum()):int(ln[:-2].sum()) + n]
+    p = ctx.span_encode(torch.from_numpy(s.copy()[None]).cuda())
+    assert np.array_equal(ctx.span_decode(p, n).cpu().numpy()[0], s)
+    req = torch.stack([torch.zeros(n, dtype=torch.int64), torch.arange(n)], 1).cuda()
+    assert np.array_equal(ctx.read(p, n, req).cpu().numpy(), s)
+    assert ctx.sync_status() == 0
