@@ -177,3 +177,29 @@ def test_record_reads_in_any_order(fkv):
         assert torch.equal(out[ti(np.flatnonzero(ok)), 0], Kr[ti(l), ti(b), :, ti(t)])
         assert torch.equal(out[ti(np.flatnonzero(ok)), 1], Vr[ti(l), ti(b), :, ti(t)])
         assert torch.count_nonzero(out[ti(np.flatnonzero(bad))]) == 0
+
+
+@pytest.mark.parametrize("n_req", [1, 456, 457, 3648, 3649, 4095])
+def test_record_reads_at_the_edges_of_each_path(fkv, n_req):
+    """A block a request, a warp a request in the order given, and grouped by
+    layer: the same values, out-of-range requests zeros."""
+    cfg = synth.small_config(synth.CFG1, 317, n_layers=8, batch=2, seq=36 + 41)
+    K = synth.gpu_kv_cache(cfg, 0)
+    V = synth.gpu_kv_cache(cfg, 1)
+    ctx, sym, pts = write_archive(fkv, cfg, K, V)
+    P, ns = cfg.n_archived, cfg.batch * cfg.n_layers
+    Kr, Vr = torch.zeros_like(K), torch.zeros_like(V)
+    ctx.decode_kv(pts, P, Kr, Vr, t0=cfg.t0)
+    rng = np.random.default_rng(n_req)
+    req = np.stack([rng.integers(0, ns, n_req), rng.integers(0, P, n_req)], axis=1)
+    bad = rng.random(n_req) < 0.02
+    bad[-1] = n_req > 1
+    req[bad, 1] = rng.choice([-1, P, 1 << 40], bad.sum())
+    out = torch.full((n_req, 2, cfg.n_heads, cfg.dim), 9.0, dtype=K.dtype, device="cuda")
+    ctx.read_kv(pts, P, torch.from_numpy(req).cuda(), out)
+    assert ctx.sync_status() == (-2 if bad.any() else 0)
+    h = out.cpu()
+    ok = ~bad
+    b, l, t = req[ok, 0] // cfg.n_layers, req[ok, 0] % cfg.n_layers, req[ok, 1] + cfg.t0
+    assert torch.equal(h[ok, 0], Kr.cpu()[l, b, :, t]) and torch.equal(h[ok, 1], Vr.cpu()[l, b, :, t])
+    assert torch.count_nonzero(h[bad]) == 0

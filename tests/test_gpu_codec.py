@@ -237,3 +237,21 @@ def test_many_random_spans_encode_bit_exact(fkv, oracle_mod, N):
     pts = ctx.span_encode(torch.from_numpy(sym).cuda())
     want = _oracle_points(oracle_mod, sym, N, ctx.r, ctx.L)
     assert np.array_equal(pts.cpu().numpy().view(np.uint64), want.view(np.uint64))
+
+
+@pytest.mark.parametrize("N", [4, 16, 256])
+@pytest.mark.parametrize("spans", [1, 127, 128, 129])
+def test_many_short_streams_encode_bit_exact(fkv, oracle_mod, N, spans):
+    """Streams that share blocks and the first that do not, the last span short,
+    strided symbols and points."""
+    ctx = _ctx(fkv, N)
+    L, ns = ctx.L, 37
+    n = spans * L - (L - 1 if spans > 1 else 0)
+    sym = _rand_streams(N, ns, n + 5, spans)
+    d = torch.from_numpy(sym).cuda()[:, :n]
+    pts = torch.full((ns, spans + 2, 2), 7.0, dtype=torch.float64, device="cuda")
+    ctx.span_encode(d, pts=pts[:, :spans])
+    want = _oracle_points(oracle_mod, sym[:, :n], N, ctx.r, L)
+    got = pts.cpu().numpy()
+    assert np.array_equal(got[:, :spans].view(np.uint64), want.view(np.uint64))
+    assert np.all(got[:, spans:] == 7.0) and ctx.sync_status() == 0
