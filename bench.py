@@ -28,7 +28,9 @@ The line also carries, each measured on its own after the timed region:
            the oracle (RVQ indices under the 1e-4 gap rule, stored points bit
            for bit, rebuilt K/V under the rounding rule), with near-tie counts;
   fp64     binary64 add/mul throughput measured by independent chains (the
-           span encoder's roofline denominator), next to the nominal figure;
+           denominator of the span encoder's six operations a symbol, of which it
+           leaves most to a table and the integer pipe), next to the nominal
+           figure;
 and under "kernels" the secondary workloads (a --no-<name> flag skips one):
   gpt2     the GPT-2-shaped full cache (12 layers x 8 x 12 heads x 1024 x 64,
            fp16, K 4 / V 2 stages), the same step on 64-dimensional heads;
@@ -83,15 +85,15 @@ def load_peaks():
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per RVQ launch of
-# the headline workload, from ncu captures of the current k_rvq128 on the same
+# the headline workload, from ncu captures of the current k_rvq128_pair on the same
 # cache cut to 4096 and to 8192 archived positions (the full cache is too large
-# for a multi-metric capture): key launch 1,340,126,208 and 2,458,886,400 B,
-# value launch 1,209,800,960 and 2,317,281,024 B.  Traffic is a fixed part (the
+# for a multi-metric capture): key launch 1,340,242,688 and 2,459,090,688 B,
+# value launch 1,209,741,312 and 2,331,231,488 B.  Traffic is a fixed part (the
 # codebooks) plus a part that grows with the positions, so the two lengths fix
 # a line, extrapolated to the headline length; the figure is the mean of the
-# key and value launches.  Set it to None when k_rvq128 changes until it is
+# key and value launches.  Set it to None when k_rvq128_pair changes until it is
 # captured again.
-RVQ_TRAFFIC_CAPTURES = ((4096, 8192), ((1340126208, 2458886400), (1209800960, 2317281024)))
+RVQ_TRAFFIC_CAPTURES = ((4096, 8192), ((1340242688, 2459090688), (1209741312, 2331231488)))
 
 
 def _rvq_traffic_full(positions=None, captures=RVQ_TRAFFIC_CAPTURES):
@@ -256,8 +258,9 @@ def phase_times(g, reps):
 def archive_rates(cfg, phase, R, P, n_rec, spans, ns, peaks, fp64_ops_per_s):
     """Algorithmic rates of one archive step's kernels (all fixed by the
     method and the workload's shape): RVQ 2*D*256 flop per vector and stage;
-    span encode 1 B in per symbol + 16 B per span out and 6 binary64
-    operations per symbol; the archive read 1 B per symbol + 16 B per span in
+    span encode 1 B in per symbol + 16 B per span out and the map's 6 binary64
+    operations per symbol (the kernel runs 2 of them a symbol on the FP64 pipe
+    at N = 256, so its rate may lie above that pipe's); the archive read 1 B per symbol + 16 B per span in
     and the rebuilt K/V out."""
     D, H = cfg.dim, cfg.n_heads
     nvec = cfg.batch * cfg.n_layers * H * P
@@ -661,7 +664,7 @@ def run_secondary(fkv, args, dev, g):
         del codes, tail, lsym, exact
 
     # Sec. 6 probability-weighted maps: this step's 96 archived index streams
-    # arithmetic-coded with the adaptive add-one model (one warp per stream;
+    # arithmetic-coded with the adaptive add-one model (independent streams;
     # decoding is sequential within a stream), encode and decode
     weighted = None
     if not args.no_weighted and g is not None:
@@ -848,7 +851,7 @@ def secondary_report(res, peaks, fp64, sm_mhz):
             "workload": "gpt2-shaped full KV cache: 12 layers x batch 8 x 12 heads x 1024 tok x 64 dims, fp16; "
                         "4+32 exact window; K 4 / V 2 RVQ stages x 256; N=256, r=r_256, L=6",
             "records_per_s": gx.ns * gx.n_rec / (gx.ms * 1e-3), "ms_per_step": gx.ms, "phase_ms": gx.phase,
-            "rvq_kernel": "k_rvq64", "rvq_ms": rates["rvq"]["ms"], "rvq_tflops": rates["rvq"]["achieved_tflops"],
+            "rvq_kernel": "k_rvq64_pair", "rvq_ms": rates["rvq"]["ms"], "rvq_tflops": rates["rvq"]["achieved_tflops"],
             "rvq_frac": rates["rvq"]["frac"], "span_encode_ms": rates["span_encode"]["ms"],
             "span_encode_frac_fp64_measured": rates["span_encode"]["frac_fp64_measured"],
             "decode_kv_ms": rates["decode_kv"]["ms"], "decode_kv_gbs": rates["decode_kv"]["achieved_gbs"],
@@ -918,7 +921,8 @@ def secondary_report(res, peaks, fp64, sm_mhz):
             "truncate_ms": lx["truncate"], "truncate_bound": "hbm",
             "truncate_gbs": tb / (lx["truncate"] * 1e-3) / 1e9,
             "truncate_frac": tb / (lx["truncate"] * 1e-3) / 1e9 / peaks["hbm_gbs"],
-            "decode_ms": lx["decode"], "decode_bound": "fp64 (binary64 walk with IEEE division, as the paper)",
+            "decode_ms": lx["decode"],
+            "decode_bound": "fp64 (the binary64 walk's differences; cell test and division on the integer pipe)",
             "decode_symbols_per_s": lx["symbols"] / (lx["decode"] * 1e-3),
             "archive_bytes": lx["code_bytes"] + lx["tail_bytes"], "exact_archive_bytes": lx["point_bytes"],
             "symbol_error_rate_truncated_spans": lx["sym_err_truncated"], "status_ok": lx["ok"]}
@@ -926,7 +930,7 @@ def secondary_report(res, peaks, fp64, sm_mhz):
         wx = sec["weighted"]
         kernels["probability-weighted maps (Sec. 6)"] = {
             "workload": "the gpt2 step's 96 archived RVQ index streams (989 records x 72 symbols, N=256), adaptive "
-                        "add-one model, one warp per stream",
+                        "add-one model, one block per stream",
             "encode_ms": wx["encode"], "decode_ms": wx["decode"], "bound": "latency (sequential within a stream)",
             "encode_symbols_per_s": wx["symbols"] / (wx["encode"] * 1e-3),
             "decode_symbols_per_s": wx["symbols"] / (wx["decode"] * 1e-3),
@@ -999,8 +1003,8 @@ def main():
     rates = archive_rates(cfg, res["phase"], res["R"], res["P"], res["n_rec"], res["spans"], res["ns"], peaks,
                           res["fp64"])
     traffic = RVQ_DRAM_BYTES_PER_LAUNCH if args.seq == HEADLINE.seq else None
-    dominant = roofline(rates, peaks, traffic, "k_rvq128 (RVQ assignment, 128-dim heads)")
-    kernels = {"rvq (tcgen05, k_rvq128)": rates["rvq"], "span_encode": rates["span_encode"],
+    dominant = roofline(rates, peaks, traffic, "k_rvq128_pair (RVQ assignment, 128-dim heads)")
+    kernels = {"rvq (tcgen05, k_rvq128_pair)": rates["rvq"], "span_encode": rates["span_encode"],
                "decode_kv (decode + gather)": rates["decode_kv"]}
     kernels.update(secondary_report(res, peaks, res["fp64"], sm_mhz))
     units = res["units"] * world
@@ -1044,8 +1048,9 @@ def main():
         "parity": par,
         "cpu_baseline": cpu,
         "e2e": e2e,
-        # per step: RVQ x4 (K and V archive, K and V of the appended position),
-        # k_span_encode x2 (archive, tail append), k_span_decode_planar,
+        # per step: RVQ x4 (K and V archive: k_rvq128_pair; K and V of the appended
+        # position: k_rvq128), k_span_encode (archive) and k_span_encode_flat
+        # (append), k_span_decode_planar,
         # k_gather x2, the record reads' k_order_count, k_order_scan and
         # k_order_scatter, and k_read_kv (as the ncu launch list shows)
         "gpu_launches": 13 * args.steps,
