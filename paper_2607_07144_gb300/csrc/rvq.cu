@@ -2514,16 +2514,34 @@ cudaError_t launch_rvq64(const fkv_ctx *c, const CUtensorMap &tmap, const RvqArg
     return cudaGetLastError();
 }
 
-// Whether a group of `tiles` tiles runs on CTA pairs.  A pair takes its tiles
-// from one group, so an odd count leaves half of the group's last unit empty:
-// from five tiles on that costs less than the pair gains, and it costs nothing
-// while every unit has a cluster to itself.  Otherwise (one tile a group is a
-// decode step's append) each SM takes its own tiles.  Measured, old and pair:
-// 64 groups of 1 tile of 128-dimensional heads 49.7 / 39.7 us for K and V, 256
-// groups 78.8 / 98.8; 144 groups of 3 tiles of 64-dimensional heads 53.1 / 64.3.
-bool pair_tiles(int64_t tiles, int64_t groups, int sms)
+// Whether a call runs on CTA pairs: `per` units (two tiles of one group) for
+// the busiest of the sms / 2 clusters.  The single-SM kernels take `sms` tile
+// pairs a round, two slots an SM; k_rvq64_pair three units a cluster, so its
+// round is half as long again, and k_rvq128_pair two, so its rounds are the
+// same but only within groups (k_rvq128 pairs the tiles of all groups, an odd
+// group's last one too).  Measured, pair / single SM (16-bit input):
+//   64 dimensions, 1 stage: 0.74 .. 1.01 but for 2 units a cluster (1.11 for
+//   144 groups of 1 tile); more stages: 1.01 .. 1.30 up to 2 units (few units
+//   gain nothing and wait for their partner), 0.75 .. 0.96 at 3 (two rounds
+//   against one), 1.10 .. 1.22 at 4, 0.85 .. 1.08 from 5 to 12, 0.91 .. 0.98
+//   beyond (0.71 .. 0.77 on 4,464 units); a tile a group 1.08 .. 1.56.
+//   1024 codewords: 0.67 .. 1.00 but for 2 units a cluster (up to 1.13).
+//   128 dimensions: 1.05 .. 1.33 when the pairs need a round more; else 0.71 ..
+//   0.97 from 2 stages on; 1 stage 0.80 .. 0.94 at an odd number of units a
+//   cluster, 0.99 .. 1.16 at an even one.
+bool pair_tiles(const fkv_ctx *c, int64_t tiles, int64_t groups, int S)
 {
-    return tiles % 2 == 0 || tiles >= 5 || groups * ((tiles + 1) / 2) <= sms / 2;
+    const int64_t units = groups * ((tiles + 1) / 2), clusters = c->sms / 2;
+    const int64_t per = (units + clusters - 1) / clusters;
+    if (c->D == 64) {
+        if (c->KC == 1024 || S == 1)
+            return per != 2;
+        return tiles > 1 && (per == 3 || per > 12);
+    }
+    const int64_t pairs = (groups * tiles + 1) / 2;
+    if ((per + 1) / 2 > (pairs + 2 * clusters - 1) / (2 * clusters))
+        return false;
+    return S > 1 || per % 2 == 1;
 }
 
 template <int ESZ, int NB>
@@ -2588,7 +2606,7 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         const int sms = c->sms;
         const unsigned grid = static_cast<unsigned>(n_pairs < sms ? n_pairs : sms);
         const int pp = static_cast<int>(ppg), np = static_cast<int>(n_pairs);
-        if (pair_tiles(tiles, c->Ly * c->H, sms)) {
+        if (pair_tiles(c, tiles, c->Ly * c->H, a.S)) {
             const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
             const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
             if (c->KC == 1024)
@@ -2609,7 +2627,7 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         if (n_pairs > 0x7FFFFFFF)
             return cudaErrorInvalidConfiguration;
         const int sms = c->sms;
-        if (pair_tiles(tiles, c->Ly * c->H, sms)) {
+        if (pair_tiles(c, tiles, c->Ly * c->H, a.S)) {
             const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
             const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
             const auto kern = x->dtype == FKV_F32 ? k_rvq128_pair<4> : k_rvq128_pair<2>;

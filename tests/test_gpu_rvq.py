@@ -343,3 +343,35 @@ def test_tile_counts_of_paired_and_single_tiles(fkv, oracle_mod, base, layers, p
     cfg = synth.small_config(b, 4000 + 100 * base + layers + positions, n_layers=layers, batch=1, seq=36 + positions,
                              n_heads=11)
     check_config_full(fkv, oracle_mod, cfg)
+
+
+@pytest.mark.parametrize("dtype,n", [("f32", 512), ("f16", 421), ("bf16", 300)])
+def test_paired_tiles_of_many_groups_with_extreme_rows(fkv, oracle_mod, dtype, n):
+    """Three tile pairs a cluster, which 64-dimensional heads of several stages
+    run on SM pairs: rows far outside and inside the codebooks, codeword-equal
+    and zero rows, and a change of stage scale, in every group."""
+    rng = np.random.default_rng(n)
+    L, H, S = 8, 11, 3
+    cbk = rng.normal(size=(L, H, S, 256, 64)).astype(np.float32)
+    cbk[:, :, 1] *= 0.3
+    cbk[:, :, 2] *= 1e-4
+    big, small = (1e3, 1e-3) if dtype == "f16" else (1e30, 1e-30)
+    x = rng.normal(size=(L, 1, H, n, 64))
+    x[:, :, :, 5:20] *= big
+    x[:, :, :, 130:150] *= small
+    x[:, :, :, 200] = 0.0
+    x[:, 0, :, n - 1] = cbk[:, :, 0, 17]
+    X = torch.from_numpy(x).to(TORCH_DT[dtype]).cuda()
+    ctx = fkv.Context(256, codebooks=(cbk, cbk[:, :, :1]))
+    sym = torch.zeros((L, n * ctx.record_len()), dtype=torch.uint8, device="cuda")
+    ctx.rvq_encode(0, X, 0, n, sym)
+    ctx.rvq_encode(1, X, 0, n, sym)
+    assert ctx.sync_status() == 0
+    x64, s = X.double().cpu().numpy(), sym.cpu().numpy().astype(np.int32)
+    for l in range(0, L, 3):
+        ik, iv = oracle_mod.indices_from_records(s[l], H, S, 1)
+        for h in range(H):
+            for gidx, cb in ((ik, cbk[l, h]), (iv, cbk[l, h, :1])):
+                oi, gap = oracle_mod.rvq_encode(x64[l, 0, h], cb)
+                assert compare_rvq(gidx[h], oi, gap)[0] == 0, (l, h)
+            assert ik[h, n - 1, 0] == 17
