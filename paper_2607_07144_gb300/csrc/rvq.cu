@@ -11,7 +11,7 @@
 // walk one 128-vector tile through the stages: exact argmin read out of tensor
 // memory with tcgen05.ld.red, then the residual update in the fp16 hi/lo
 // operand tiles.  k_rvq64_pair and k_rvq128_pair run on CTA pairs (M = 256);
-// k_rvq64 and k_rvq128 (M = 128) take the shapes whose tiles do not pair up
+// k_rvq64 and k_rvq128 (M = 128) take the shapes that are no faster there
 // (pair_tiles), a decode step's append above all.
 #include <type_traits>
 
