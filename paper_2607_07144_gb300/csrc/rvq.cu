@@ -2524,24 +2524,26 @@ cudaError_t launch_rvq64(const fkv_ctx *c, const CUtensorMap &tmap, const RvqArg
 //   144 groups of 1 tile); more stages: 1.01 .. 1.30 up to 2 units (few units
 //   gain nothing and wait for their partner), 0.75 .. 0.96 at 3 (two rounds
 //   against one), 1.10 .. 1.22 at 4, 0.85 .. 1.08 from 5 to 12, 0.91 .. 0.98
-//   beyond (0.71 .. 0.77 on 4,464 units); a tile a group 1.08 .. 1.56.
+//   beyond (0.71 .. 0.77 on 4,464 units); a tile a group 1.08 .. 1.56; float32
+//   input at 1 unit 0.92 .. 1.05, and 19.3 / 22.9 us for the two launches of a
+//   layer of 12 heads and 988 positions (rows come whole lines at a time).
 //   1024 codewords: 0.67 .. 1.00 but for 2 units a cluster (up to 1.13).
 //   128 dimensions: 1.05 .. 1.33 when the pairs need a round more; else 0.71 ..
 //   0.97 from 2 stages on; 1 stage 0.80 .. 0.94 at an odd number of units a
 //   cluster, 0.99 .. 1.16 at an even one.
-bool pair_tiles(const fkv_ctx *c, int64_t tiles, int64_t groups, int S)
+bool pair_tiles(const fkv_ctx *c, int64_t tiles, int64_t groups, const RvqArgs &a)
 {
     const int64_t units = groups * ((tiles + 1) / 2), clusters = c->sms / 2;
     const int64_t per = (units + clusters - 1) / clusters;
     if (c->D == 64) {
-        if (c->KC == 1024 || S == 1)
+        if (c->KC == 1024 || a.S == 1)
             return per != 2;
-        return tiles > 1 && (per == 3 || per > 12);
+        return tiles > 1 && (per == 3 || per > 12 || (per == 1 && a.dtype == FKV_F32));
     }
     const int64_t pairs = (groups * tiles + 1) / 2;
     if ((per + 1) / 2 > (pairs + 2 * clusters - 1) / (2 * clusters))
         return false;
-    return S > 1 || per % 2 == 1;
+    return a.S > 1 || per % 2 == 1;
 }
 
 template <int ESZ, int NB>
@@ -2606,7 +2608,7 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         const int sms = c->sms;
         const unsigned grid = static_cast<unsigned>(n_pairs < sms ? n_pairs : sms);
         const int pp = static_cast<int>(ppg), np = static_cast<int>(n_pairs);
-        if (pair_tiles(c, tiles, c->Ly * c->H, a.S)) {
+        if (pair_tiles(c, tiles, c->Ly * c->H, a)) {
             const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
             const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
             if (c->KC == 1024)
@@ -2627,7 +2629,7 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
         if (n_pairs > 0x7FFFFFFF)
             return cudaErrorInvalidConfiguration;
         const int sms = c->sms;
-        if (pair_tiles(c, tiles, c->Ly * c->H, a.S)) {
+        if (pair_tiles(c, tiles, c->Ly * c->H, a)) {
             const int upg = static_cast<int>((tiles + 1) / 2), nu = upg * c->Ly * c->H;
             const unsigned clusters = static_cast<unsigned>(nu < sms / 2 ? nu : sms / 2);
             const auto kern = x->dtype == FKV_F32 ? k_rvq128_pair<4> : k_rvq128_pair<2>;
