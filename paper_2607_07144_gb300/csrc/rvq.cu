@@ -866,9 +866,14 @@ k_rvq64(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int pairs_per
 // accumulator n & 1 and ring buffer n mod 3.  Barriers, in the leader unless
 // both CTAs are named: full (the two halves of a buffer have landed), empty
 // (both; the item's MMAs are done), a_ready (the slot's operand rows are
-// written, one arrival per epilogue warp of both CTAs), acc_full (both; per
-// slot, so that every group waits on a barrier of its own phases), acc_free
-// (the accumulator's scores are read).  The epilogue takes the chosen codeword
+// written, one arrival per epilogue warp of both CTAs), acc_full (both; two
+// per slot, for its even and its odd codeword blocks), acc_free (the
+// accumulator's scores are read).  A wait by parity tells only the last phase
+// from the one before, so no barrier may complete twice before all its waiters
+// have seen the first.  For acc_full that takes the two: a round of one unit
+// issues a slot's blocks back to back on the two accumulators, and the MMAs of
+// block u + 1 wait for no read of block u, those of u + 2 (by acc_free) do;
+// between stages a_ready does it.  The epilogue takes the chosen codeword
 // from its float32 row in L2, two rows per instruction.
 //
 // GPT-2-shaped cache, 1,138,176 vectors of K (4 stages) and of V (2): 486 us
@@ -896,8 +901,8 @@ constexpr int B_BUF = 2 * B_TILE + B_AUG;    // 36 KB
 constexpr int OFF_AAUG = kSlots * A_SLOT;
 constexpr int OFF_B = OFF_AAUG + kSlots * A_AUG;
 constexpr int OFF_BAR = OFF_B + kBufs * B_BUF;
-constexpr int BAR_FULL = 0, BAR_EMPTY = 3, BAR_READY = 6, BAR_ACC = 9, BAR_FREE = 12, BAR_DRAIN = 14, kBars = 15;
-constexpr int OFF_SLOT = OFF_BAR + 8 * 16;
+constexpr int BAR_FULL = 0, BAR_EMPTY = 3, BAR_READY = 6, BAR_ACC = 9, BAR_FREE = 15, BAR_DRAIN = 17, kBars = 18;
+constexpr int OFF_SLOT = OFF_BAR + 8 * kBars;
 constexpr int OFF_LO = OFF_SLOT + 16;        // per slot: the round whose first-stage lo operand is nonzero (leader)
 constexpr int OFF_ABORT = OFF_LO + 16;
 constexpr int END = OFF_ABORT + 16;
@@ -1214,7 +1219,7 @@ k_rvq64_pair(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ C
                                 if (lo)
                                     umma_f16_pair(acc, dal, dbh, idesc, 1);
                             }
-                            umma_commit_pair(bar(BAR_ACC + k));
+                            umma_commit_pair(bar(BAR_ACC + 2 * k + (blk & 1)));
                             umma_commit_pair(bar(BAR_EMPTY + b));
                             if (++b == kBufs) {
                                 b = 0;
@@ -1266,7 +1271,7 @@ k_rvq64_pair(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ C
             return w;
         };
         uint32_t n0 = 0;                          // items before this round
-        uint32_t fph = 0;
+        uint32_t fph = 0;                         // parities of the slot's two acc_full
         int pc = 0;
         bool ok = true;
         for (int ur = 0; ur + k < nu && ok; ur += kSlots) {
@@ -1349,13 +1354,13 @@ k_rvq64_pair(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ C
                 int bidx = 0;
                 for (int blk = 0; blk < NB; ++blk) {
                     const uint32_t acc = (n0 + static_cast<uint32_t>((s * NB + blk) * act + k)) & 1;
-                    ok = wait_or_abort(bar(BAR_ACC + k), fph, a.status, abort_flag);
+                    ok = wait_or_abort(bar(BAR_ACC + 2 * k + (blk & 1)), (fph >> (blk & 1)) & 1, a.status, abort_flag);
                     // the tensor-memory loads below are warp-collective: the warp
                     // goes on, or leaves, as one
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok)
                         break;
-                    fph ^= 1;
+                    fph ^= 1u << (blk & 1);
                     tc_fence_after();
                     const uint32_t trow = tmem + acc * 256 + tquad;
                     bool amb;

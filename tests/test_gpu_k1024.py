@@ -211,3 +211,36 @@ def test_full_size_pooled_rvq1024x2(fkv, oracle_mod):
                 hd, _, sn = compare_rvq(gi[h], oi, gap)
                 hard, seen = hard + hd, seen + sn
     assert hard == 0 and seen > 0
+
+
+@pytest.mark.parametrize("dtype,pooled,layers,heads,n",
+                         [("f32", True, 4, 19, 200), ("f16", True, 7, 11, 300), ("bf16", False, 7, 11, 600),
+                          ("f16", True, 7, 11, 641), ("f32", False, 7, 11, 900)])
+def test_partial_rounds_on_pairs_of_sms(fkv, oracle_mod, dtype, pooled, layers, heads, n):
+    """1, 3, 4 and 5 units (two 128-vector tiles of a head) for the busiest of
+    76 SM pairs, three of which run at a time: rounds of three units, then of
+    one or two, whose codeword blocks follow one another on the same tile.
+    Codewords of different 256-blocks that are equal must give the lowest."""
+    rng = np.random.default_rng(n)
+    Hc = 1 if pooled else heads
+    cb = rng.normal(size=(layers, Hc, 2, 1024, 64)).astype(np.float32)
+    cb[:, :, 1] *= 0.4
+    cb[:, :, 0, 1000] = cb[:, :, 0, 3]
+    cb[:, :, 0, 700] = cb[:, :, 0, 300]
+    x = rng.normal(size=(layers, 1, heads, n, 64))
+    x[:, 0, :, 0] = cb[:, :, 0, 1000]
+    x[:, 0, :, n - 1] = cb[:, :, 0, 700]
+    X = torch.from_numpy(x).to(TORCH_DT[dtype]).cuda()
+    ctx = fkv.Context(1024, codebooks=(cb, cb[:, :, :1]), pooled=pooled, n_heads=heads)
+    sym = torch.full((layers, n * ctx.record_len()), -1, dtype=ctx.sym_dtype, device="cuda")
+    ctx.rvq_encode(0, X, 0, n, sym)
+    ctx.rvq_encode(1, X, 0, n, sym)
+    assert ctx.sync_status() == 0
+    x64, s = X.double().cpu().numpy(), sym.cpu().numpy().astype(np.int32)
+    for l in range(layers):
+        ik, iv = oracle_mod.indices_from_records(s[l], heads, 2, 1)
+        assert np.all(ik[:, 0, 0] == 3) and np.all(ik[:, n - 1, 0] == 300)
+        assert np.array_equal(ik[:, :, :1], iv)
+        for h in range(heads if l in (0, layers - 1) else 1):
+            oi, gap = oracle_mod.rvq_encode(x64[l, 0, h], cb[l, 0 if pooled else h])
+            assert compare_rvq(ik[h], oi, gap)[0] == 0, (l, h)
