@@ -341,7 +341,8 @@ int fkv_record_len(const fkv_ctx *ctx);
  * Only the kv half of each record is written.  Runs on the tensor cores
  * (tcgen05) with split-fp16 operands whose score error is below 5e-5 of the
  * residual's squared norm; ties closer than that may differ from a float64
- * search. */
+ * search, but not with the shape of the call: a vector gets the same indices
+ * in a bulk write, in any part of it and in an append. */
 int fkv_rvq_encode(fkv_ctx *ctx, int kv, const fkv_cache *x, int64_t t0, int64_t t1,
                    void *sym_dev, int64_t stream_stride, int64_t rec0, void *stream);
 

@@ -67,6 +67,7 @@ void destroy_cbset(fkv_cbset &s)
 {
     cudaFree(s.cb32);
     cudaFree(s.cb16);
+    cudaFree(s.cbsum);
     cudaFree(s.escale);
     cudaFree(s.escale_h);
     cudaFree(s.cbaug);
@@ -176,6 +177,10 @@ int upload_cbset(fkv_ctx *ctx, int kv, const float *host, int stages)
     CK(cudaMalloc(&s.escale, es.size() * sizeof(int)), "codebook alloc");
     CK(cudaMemcpy(s.cb32, host, ncode * D * sizeof(float), cudaMemcpyHostToDevice), "codebook copy");
     CK(cudaMemcpy(s.cb16, c16.data(), c16.size() * sizeof(__half), cudaMemcpyHostToDevice), "codebook copy");
+    if (D == 64) {
+        CK(cudaMalloc(&s.cbsum, ncode * D * sizeof(float)), "codebook alloc");
+        CK(launch_join_codewords(ctx, s, nullptr), "codebook launch");
+    }
     CK(cudaMemcpy(s.escale, es.data(), es.size() * sizeof(int), cudaMemcpyHostToDevice), "codebook copy");
     {
         // each head's copy of its codebook group's scales
@@ -443,7 +448,6 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
     ctx->d_pre = reinterpret_cast<double2 *>(base + o_pre);
     CK(cudaMemcpy(base, tab.data(), tab.size(), cudaMemcpyHostToDevice), "context copy");
     CK(launch_pre_table(ctx, nullptr), "point table launch");
-    CK(cudaStreamSynchronize(nullptr), "context init");   // before any other stream uses the tables
 
     if (cb) {
         // the allocation-free archive read's fixed scratch: its address is
@@ -472,6 +476,7 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
         if (rc != FKV_OK)
             return bail(rc);
     }
+    CK(cudaStreamSynchronize(nullptr), "context init");   // before any other stream uses the tables
     *out = ctx;
     return FKV_OK;
 }

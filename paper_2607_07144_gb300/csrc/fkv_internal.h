@@ -29,6 +29,9 @@ struct fkv_cbset {
     CUtensorMap tmap_aug;     // cbaug as [lines][64] fp16 (4 codewords a line), box {64, 32}, no swizzle
     // 64-dimensional heads only (rvq.cu k_rvq64): cb16 holds the hi/lo split of
     // -2 c 2^-e with max |c 2^-e| in [2^3, 2^9), and cbaug the norm operand.
+    // cbsum is that split's hi + lo as float32, the codeword that every residual
+    // update of 64-dimensional heads subtracts.
+    float *cbsum = nullptr;   // [G][S][K][64]
     __half *cbaug = nullptr;  // [G][S] blocks of K x 16 fp16 in core-matrix layout (32 B per codeword)
 };
 
@@ -164,6 +167,8 @@ cudaError_t launch_ac_encode(const fkv_ctx *c, const void *sym, int64_t n_stream
 cudaError_t launch_ac_decode(const fkv_ctx *c, const uint32_t *words, int64_t word_stride, const int64_t *nbits,
                              int64_t n_streams, int64_t n, int adaptive, void *sym, int64_t sym_stride, cudaStream_t st);
 // rvq.cu
+// Fill cb.cbsum from cb.cb16 (cb.stages stages of c's codebook groups).
+cudaError_t launch_join_codewords(const fkv_ctx *c, const fkv_cbset &cb, cudaStream_t st);
 cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int64_t t0, int64_t t1,
                               void *sym, int64_t stream_stride, int64_t rec0, cudaStream_t st);
 // Decoded archive symbols in one of two layouts: the token records of the

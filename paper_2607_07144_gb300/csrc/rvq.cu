@@ -31,6 +31,7 @@ struct RvqArgs {
     int64_t s_layer, s_batch, s_head, s_pos;
     int n_layers, n_heads, S;
     const float *cb32;
+    const float *cbsum;    // [G][S][KC][64] hi + lo of cb16's codewords (64-dim heads)
     const int *escale;
     const int *escale_h;   // [Ly*H][S] escale of each head's codebook group
     const __half *cbaug;
@@ -873,8 +874,10 @@ k_rvq64(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int pairs_per
 // have seen the first.  For acc_full that takes the two: a round of one unit
 // issues a slot's blocks back to back on the two accumulators, and the MMAs of
 // block u + 1 wait for no read of block u, those of u + 2 (by acc_free) do;
-// between stages a_ready does it.  The epilogue takes the chosen codeword
-// from its float32 row in L2, two rows per instruction.
+// between stages a_ready does it.  The epilogue takes the chosen codeword's
+// hi + lo from a float32 row in L2, two rows per instruction: the values that
+// k_rvq64 has in its stage buffer, since a vector's indices must not depend on
+// the shape of the call that archives it.
 //
 // GPT-2-shaped cache, 1,138,176 vectors of K (4 stages) and of V (2): 486 us
 // against 633 for k_rvq64, and with 1024-codeword codebooks 1,013 against
@@ -1384,9 +1387,9 @@ k_rvq64_pair(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ C
                     break;
                 idx |= static_cast<uint64_t>(bidx) << (8 * sizeof(Sym) * s);
                 if (s + 1 < S) {
-                    // t <- t - c 2^(-e-er), the chosen codeword from its float32 row
-                    const float f = -pow2f(-e - er);
-                    const float *cbs = a.cb32 + static_cast<int64_t>(cgroup(g) * S + s) * KC * 64;
+                    // t <- t - c' 2^-er = t + (hi + lo) 2^(-1-er), as k_rvq64 does
+                    const float f = pow2f(-1 - er);
+                    const float *cbs = a.cbsum + static_cast<int64_t>(cgroup(g) * S + s) * KC * 64;
                     if (e_next == e) {
                         // |t| stays below 2^12 + S 2^9 < 2^14: the row shift holds
                         if (__all_sync(0xFFFFFFFFu, er == 0))
@@ -2500,7 +2503,29 @@ __global__ void __launch_bounds__(96, 1) k_wait_check(unsigned *status, uint64_t
         out[5] = 1;
 }
 
+// cbsum of one codebook set: hi + lo of each element (exact in float32).
+__global__ void __launch_bounds__(256)
+k_join_codewords(const __half *__restrict__ cb16, int64_t n, int per_stage, float *__restrict__ out)
+{
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+    if (i < n) {
+        const __half *hi = cb16 + i + i / per_stage * per_stage;      // a stage's hi block, its lo block behind it
+        out[i] = __half2float(hi[0]) + __half2float(hi[per_stage]);
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_join_codewords(const fkv_ctx *c, const fkv_cbset &cb, cudaStream_t st)
+{
+    const int per_stage = c->KC * c->D;
+    const int64_t n = static_cast<int64_t>(c->Ly) * (c->pooled ? 1 : c->H) * cb.stages * per_stage;
+    const int64_t blocks = (n + 255) / 256;
+    if (blocks > 0x7FFFFFFF)
+        return cudaErrorInvalidConfiguration;
+    k_join_codewords<<<static_cast<unsigned>(blocks), 256, 0, st>>>(cb.cb16, n, per_stage, cb.cbsum);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_wait_check(unsigned *status, uint64_t limit_ns, int *out_dev, cudaStream_t st)
 {
@@ -2586,6 +2611,7 @@ cudaError_t launch_rvq_encode(const fkv_ctx *c, int kv, const fkv_cache *x, int6
     a.escale_h = cb.escale_h;
     a.cbaug = cb.cbaug;
     a.cb16 = cb.cb16;
+    a.cbsum = cb.cbsum;
     a.KC = c->KC;
     a.pooled = c->pooled ? 1 : 0;
     a.sym = sym;
