@@ -400,17 +400,16 @@ int fkv_cache_upload(fkv_ctx *ctx, const fkv_cache *src_host, const fkv_cache *d
  * decode only the spans of that record and write its K and V head vectors to
  * out_dev, laid out [n_req][2 (K, V)][n_heads][dim] in `dtype`.  Streams hold
  * n_rec records each, points as in fkv_decode_kv.  Out-of-range requests
- * write zeros and set FKV_ERANGE.  Up to 3,648 requests are taken as they
- * come (up to 456 with a block each); more are taken grouped by layer (a
- * counting sort of their indices on the device, so that one layer's codebooks
- * serve the requests in flight).  A batch of at least 512 requests
- * per layer is staged: its records' symbols are decoded into a buffer first,
- * then rebuilt from (codebook group, dimension slice) copies in shared memory
- * as in fkv_decode_kv; smaller batches rebuild each record from codeword rows
- * in L2.  All give the same values.  The context keeps the index (and symbol)
- * buffer of the grouped calls, allocating it on first use and whenever n_req
- * outgrows it (after a
- * synchronisation of `stream`). */
+ * write zeros and set FKV_ERANGE.  A batch of at least 512 requests per layer
+ * is staged: grouped by layer (a counting sort of the requests on the device),
+ * its records' symbols are decoded into a buffer, then rebuilt from (codebook
+ * group, dimension slice) copies in shared memory as in fkv_decode_kv.  A
+ * smaller batch rebuilds each record from codeword rows in L2: up to 24
+ * requests per SM as they come (with a block each while the device holds that
+ * many blocks), more grouped by layer, so that one layer's codebooks serve the
+ * requests in flight.  All give the same values.  The context keeps the index
+ * (and symbol) buffer of the grouped calls, allocating it on first use and
+ * whenever n_req outgrows it (after a synchronisation of `stream`). */
 int fkv_read_kv(fkv_ctx *ctx, const double *pts_dev, int64_t n_streams, int64_t n_rec,
                 int64_t pt_stride, const int64_t *req_dev, int64_t n_req, void *out_dev,
                 int dtype, void *stream);

@@ -717,19 +717,22 @@ __global__ void __launch_bounds__(256) k_order_scatter(const int64_t *__restrict
 // L2 one request per warp.
 constexpr int64_t kStagedPerLayer = 512;
 
-// Up to this many requests (a warp each, about what is resident at once: three
-// blocks of eight warps on each of 152 SMs) run together, so that grouping
-// them by layer changes nothing but costs four launches: 96 records 10.2 us
-// without them and with a block each, 23.7 before.
-constexpr int64_t kUnordered = 3648;
-
-// Up to this many requests (a block each, resident at once) a request gets a
-// block of its own.
-constexpr int64_t kBlockEach = 456;
+// Up to this many requests an SM are taken as they come: they are one to three
+// rounds of a warp each (three blocks of eight warps an SM with 256 codewords,
+// one with 1024), in which grouping them by layer gains less than its four
+// launches cost.  3,648 records of 12 layers, as they come and (at 3,649)
+// grouped: 16.5 / 33.2 us (64 dimensions, 256 codewords), 21.9 / 41.8 (32
+// layers, 128 dimensions), 24.7 / 40.3 (64 dimensions, 1024 codewords).
+constexpr int64_t kUnorderedPerSm = 24;
 
 static bool read_staged(const fkv_ctx *c, int64_t n_req)
 {
     return n_req >= kStagedPerLayer * c->Ly;
+}
+
+static bool read_unordered(const fkv_ctx *c, int64_t n_req)
+{
+    return n_req <= kUnorderedPerSm * c->sms;
 }
 
 // Ints before the staged reads' symbol buffer: the entries and the layer
@@ -746,7 +749,7 @@ int64_t read_order_ints(const fkv_ctx *c, int64_t n_req)
     if (n_req <= 0 || n_req > 0x7FFFFFFF || 2 * (c->Ly + 1) > 12 * 1024)
         return 0;
     if (!read_staged(c, n_req))
-        return n_req <= kUnordered ? 0 : 4 * n_req + c->Ly + 1;
+        return read_unordered(c, n_req) ? 0 : 4 * n_req + c->Ly + 1;
     const int64_t R = static_cast<int64_t>(c->H) * (c->cb[0].stages + c->cb[1].stages);
     const int64_t esz = c->KC == 256 ? 1 : 2;
     return read_scr_ints(c, n_req) + (n_req * R * esz + 3) / 4;
@@ -848,17 +851,25 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
         return cudaSuccess;
     const int esz = c->KC == 256 ? 1 : 2;
     const int smem = read_tables_bytes(a.N, a.L) + kReadWarps * kMaxRecord * esz;
-    const bool block = n_req <= kBlockEach;
-    const void *kern = esz == 1 ? (block ? reinterpret_cast<const void *>(k_read_kv<uint8_t, true>)
-                                         : reinterpret_cast<const void *>(k_read_kv<uint8_t, false>))
-                                : (block ? reinterpret_cast<const void *>(k_read_kv<uint16_t, true>)
-                                         : reinterpret_cast<const void *>(k_read_kv<uint16_t, false>));
-    // persistent: as many blocks as fit at once, or one per eight requests
+    // a block of its own for each request while all these are resident at once
+    // (96 GPT-2-shaped records 8.3 us, 22.1 grouped with a warp each; 456
+    // records of 1024 codewords, three to an SM that holds one block, 16.5 us
+    // against 14.5 with a warp each)
+    const void *kern = esz == 1 ? reinterpret_cast<const void *>(k_read_kv<uint8_t, true>)
+                                : reinterpret_cast<const void *>(k_read_kv<uint16_t, true>);
     int per_sm = 0;
     const int sms = c->sms;
     cudaError_t e = kernel_use(c, kern, kReadWarps * 32, smem, &per_sm);
     if (e != cudaSuccess)
         return e;
+    const bool block = n_req <= static_cast<int64_t>(sms) * per_sm;
+    if (!block) {
+        kern = esz == 1 ? reinterpret_cast<const void *>(k_read_kv<uint8_t, false>)
+                        : reinterpret_cast<const void *>(k_read_kv<uint16_t, false>);
+        e = kernel_use(c, kern, kReadWarps * 32, smem, &per_sm);
+        if (e != cudaSuccess)
+            return e;
+    }
     if (order && n_streams <= 0x7FFFFFFF && n_rec <= 0x7FFFFFFF) {
         // requests grouped by layer: n_req int4 entries, the layer counters after them
         int4 *ent = reinterpret_cast<int4 *>(order);
@@ -879,6 +890,7 @@ cudaError_t launch_read_kv(const fkv_ctx *c, const double *pts, int64_t n_stream
         if (read_staged(c, n_req))
             a.scr = order + read_scr_ints(c, n_req);
     }
+    // persistent: as many blocks as fit at once, or one per eight requests
     int64_t blocks = block ? n_req : (n_req + kReadWarps - 1) / kReadWarps;
     const int64_t resident = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
     if (blocks > resident)

@@ -244,3 +244,24 @@ def test_partial_rounds_on_pairs_of_sms(fkv, oracle_mod, dtype, pooled, layers, 
         for h in range(heads if l in (0, layers - 1) else 1):
             oi, gap = oracle_mod.rvq_encode(x64[l, 0, h], cb[l, 0 if pooled else h])
             assert compare_rvq(ik[h], oi, gap)[0] == 0, (l, h)
+
+
+@pytest.mark.parametrize("n_req", [1, 152, 153, 457, 3648, 3649])
+def test_record_reads_at_the_edges_of_each_path(fkv, n_req):
+    """With 1024 codewords one block of the record reads fits an SM: a block, a
+    warp and several rounds of a warp a request, and grouped by layer."""
+    cfg = synth.small_config(synth.CFG5, 517, n_layers=8, batch=2, seq=36 + 41)
+    K, V = synth.gpu_kv_cache(cfg, 0), synth.gpu_kv_cache(cfg, 1)
+    ctx = make_ctx(fkv, cfg)
+    pts = ctx.span_encode(encode(fkv, cfg, K, V, ctx))
+    P, ns = cfg.n_archived, cfg.batch * cfg.n_layers
+    Kr, Vr = torch.zeros_like(K), torch.zeros_like(V)
+    ctx.decode_kv(pts, P, Kr, Vr, t0=cfg.t0)
+    rng = np.random.default_rng(n_req)
+    req = np.stack([rng.integers(0, ns, n_req), rng.integers(0, P, n_req)], axis=1)
+    out = torch.full((n_req, 2, cfg.n_heads, cfg.dim), 9.0, dtype=K.dtype, device="cuda")
+    ctx.read_kv(pts, P, torch.from_numpy(req).cuda(), out)
+    assert ctx.sync_status() == 0
+    b, l, t = req[:, 0] // cfg.n_layers, req[:, 0] % cfg.n_layers, req[:, 1] + cfg.t0
+    h = out.cpu()
+    assert torch.equal(h[:, 0], Kr.cpu()[l, b, :, t]) and torch.equal(h[:, 1], Vr.cpu()[l, b, :, t])
