@@ -846,20 +846,33 @@ __device__ __forceinline__ auto span_writer(Sym *dst, int m)
     if constexpr (!WORDS) {
         return [=](int j, int c) { dst[m - 1 - j] = static_cast<Sym>(c); };
     } else {
+        const unsigned last = static_cast<unsigned>(reinterpret_cast<uintptr_t>(dst)) + m - 1;
         return [=, acc = 0u](int j, int c) mutable {
             acc = (acc << 8) | static_cast<unsigned>(c);
-            uint8_t *at = dst + (m - 1 - j);
-            const unsigned in_word = static_cast<unsigned>(reinterpret_cast<uintptr_t>(at)) & 3u;
-            if (in_word == 0u && j >= 3) {
-                *reinterpret_cast<unsigned *>(at) = acc;
-            } else if (in_word == 0u || j == m - 1) {
-                const int cnt = min(j + 1, 4 - static_cast<int>(in_word));
+            const unsigned in_word = (last - static_cast<unsigned>(j)) & 3u;
+            if (in_word == 0u) {
+                uint8_t *at = dst + (m - 1 - j);
+                if (j >= 3) {
+                    *reinterpret_cast<unsigned *>(at) = acc;
+                } else {
+                    for (int k = 0; k <= j; ++k)
+                        at[k] = static_cast<uint8_t>(acc >> (8 * k));
+                }
+            } else if (j == m - 1) {
+                const int cnt = min(m, 4 - static_cast<int>(in_word));
                 for (int k = 0; k < cnt; ++k)
-                    at[k] = static_cast<uint8_t>(acc >> (8 * k));
+                    dst[k] = static_cast<uint8_t>(acc >> (8 * k));
             }
         };
     }
 }
+
+// WORDS: bytes as words (span_writer) in batches of more than kWordSpans spans;
+// in smaller ones the stores are not what a warp waits for (8,097 spans of 44
+// symbols, N = 4: 12.6 us as bytes, 14.4 as words; 26,903 of 24, N = 8: 10.5 and
+// 12.6; 33,868 of 44, N = 4: 18.9 and 12.6).  A loop for each, for a branch
+// inside one costs up to 3 us.
+constexpr int64_t kWordSpans = 24576;
 
 template <typename Sym, fkvdec::Cell CELL, bool WORDS>
 __global__ void __launch_bounds__(dec_threads<Sym>())
@@ -872,20 +885,28 @@ k_span_decode_ragged(const double2 *__restrict__ pts, const int64_t *__restrict_
     __syncthreads();
     ragged_check(so, po, n_streams, L, status);
     const int64_t g0 = __ldg(&po[0]), g1 = __ldg(&po[n_streams]);
+    const bool many = g1 - g0 > kWordSpans;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t g = g0 + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < g1; g += stride) {
-        const int64_t i = ragged_stream(po, n_streams, g);
-        int64_t n;
-        if (!ragged_ok(so, po, i, L, &n))
-            continue;
-        const int64_t s = g - __ldg(&po[i]);
-        if (s < 0 || s * L >= n)
-            continue;
-        const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
-        Sym *dst = sym + __ldg(&so[i]) + s * L;
-        if (!fkvdec::decode_point<CELL>(t, pts[g], m, __ldg(&dc->alim[m]), [&] { return span_writer<WORDS>(dst, m); }))
-            atomicOr(status, FKV_ST_CORRUPT);
-    }
+    auto all = [&](auto words) {
+        for (int64_t g = g0 + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < g1; g += stride) {
+            const int64_t i = ragged_stream(po, n_streams, g);
+            int64_t n;
+            if (!ragged_ok(so, po, i, L, &n))
+                continue;
+            const int64_t s = g - __ldg(&po[i]);
+            if (s < 0 || s * L >= n)
+                continue;
+            const int m = static_cast<int>(min(static_cast<int64_t>(L), n - s * L));
+            Sym *dst = sym + __ldg(&so[i]) + s * L;
+            if (!fkvdec::decode_point<CELL>(t, pts[g], m, __ldg(&dc->alim[m]),
+                                            [&] { return span_writer<words.value>(dst, m); }))
+                atomicOr(status, FKV_ST_CORRUPT);
+        }
+    };
+    if (WORDS && many)
+        all(std::integral_constant<bool, WORDS>());
+    else
+        all(std::false_type());
 }
 
 // Random access into a ragged batch: request q = (stream, position), the
@@ -1706,11 +1727,12 @@ cudaError_t decode_ragged_t(const fkv_ctx *c, const double *pts, const int64_t *
 {
     auto kern = k_span_decode_ragged<Sym, fkvdec::kSectors, false>;
     if constexpr (sizeof(Sym) == 1) {
-        // words pay from longer spans on: 134 M symbols as words and as bytes,
-        // sectors: 0.385 / 0.349 ms at 12 symbols a span, 0.358 / 0.394 at 16,
-        // 0.354 / 0.546 at 22; scores: 0.658 / 0.630 at 24, 0.533 / 0.717 at 31
-        // (their walk, not the stores, bounds the shorter ones)
-        const bool words = c->L >= (c->N <= 8 && c->N != 4 ? 28 : 16);
+        // words pay from longer spans on (the walk bounds the shorter ones).  64
+        // streams of about 262,144 symbols as bytes and as words: sectors (N = 9)
+        // 55.1 / 57.2 us at 14 symbols a span, 58.4 / 46.1 at 16, 74.2 / 49.4 at 22;
+        // axes 37.1 / 43.4 at 16, 43.0 / 41.2 at 18, 83.9 / 33.0 at 44; scores 78.8 /
+        // 82.2 (N = 5) and 86.6 / 92.4 (N = 8) at 20, 77.3 / 69.8 and 83.8 / 85.5 at 24
+        const bool words = c->L >= (c->N == 4 ? 18 : c->N <= 8 ? 24 : 16);
         if (c->N == 4)
             kern = words ? k_span_decode_ragged<Sym, fkvdec::kAxes, true>
                          : k_span_decode_ragged<Sym, fkvdec::kAxes, false>;

@@ -129,3 +129,22 @@ def test_ragged_decode_writes_its_own_bytes_only(fkv, oracle_mod, N, L):
     req = torch.stack([torch.zeros(n, dtype=torch.int64), torch.arange(n)], 1).cuda()
     assert np.array_equal(ctx.read(p, n, req).cpu().numpy(), s)
     assert ctx.sync_status() == 0
+
+
+@pytest.mark.parametrize("N,L", [(3, 24), (4, 18), (4, 44), (5, 24), (8, 24), (9, 16), (16, 16)])
+def test_ragged_decode_of_many_spans_writes_its_own_bytes_only(fkv, N, L):
+    """More spans than the small batches whose bytes are stored one by one, so
+    that they go out as words: streams of every length and alignment, one long."""
+    ctx = fkv.Context(N, span_len=L)
+    rng = np.random.default_rng(100 * N + L)
+    ln = np.array(list(range(1, 2 * L + 3)) + [24700 * L + 1, 40 * L + 3], np.int64)
+    flat = rng.integers(0, N, size=int(ln.sum())).astype(np.uint8)
+    so, po = ctx.ragged_offsets(ln)
+    pts = ctx.span_encode_ragged(torch.from_numpy(flat).cuda(), so, po)
+    for shift in range(4):
+        out = torch.full((shift + flat.size + 9,), 0xEE, dtype=torch.uint8, device="cuda")
+        ctx.span_decode_ragged(pts, po, so, sym=out[shift:shift + flat.size])
+        h = out.cpu().numpy()
+        assert np.array_equal(h[shift:shift + flat.size], flat)
+        assert np.all(h[:shift] == 0xEE) and np.all(h[shift + flat.size:] == 0xEE)
+    assert ctx.sync_status() == 0
