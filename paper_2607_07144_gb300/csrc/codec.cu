@@ -14,6 +14,8 @@
 // decode_core.cuh).
 #include <string.h>
 
+#include <type_traits>
+
 #include "decode_core.cuh"
 
 namespace {
@@ -238,6 +240,17 @@ struct EncTable {
     }
 };
 
+// The vertices as they are (encode_few).
+template <typename Sym>
+struct PlainTable {
+    double2 v[vtab_len<Sym>()];
+    __device__ __forceinline__ void load(const EncArgs &a)
+    {
+        for (int i = threadIdx.x; i < a.N; i += blockDim.x)
+            v[i] = a.V[i];
+    }
+};
+
 // One span from the anchor: its first pre_k symbols from the table, the rest
 // walked, the product on the integer pipe.  With r = 1/2 (HALF) the product
 // is exact, and the walk keeps S = 2^j p (scaling by powers of two commutes
@@ -304,6 +317,47 @@ __device__ __forceinline__ double2 encode_anchored(const Sym *s, int m, const En
     return bad ? make_double2(nan, nan) : make_double2(x, y);
 }
 
+// The same by the plain walk after the table's symbols, for few spans: with up
+// to four warps on an SM its FP64 pipe keeps up, and a binary64 operation's
+// latency is less than that of its integer form.
+template <typename Sym>
+__device__ __forceinline__ double2 encode_few(const Sym *s, int m, const double2 *V, const EncArgs &a)
+{
+    const unsigned N = static_cast<unsigned>(a.N);
+    double x = 0.0, y = 0.0;
+    bool bad = false;
+    int k = 0;
+    if (a.pre_k > 2 && m >= a.pre_k) {         // one or two symbols: no slower walked than looked up
+        unsigned at = 0;
+        for (; k < a.pre_k; ++k) {
+            const unsigned c = s[k];
+            bad |= c >= N;
+            at = at * N + c;
+        }
+        if (!bad) {
+            const double2 p = __ldg(&a.pre[at]);
+            x = p.x;
+            y = p.y;
+        }
+    }
+    for (; k < m; ++k) {
+        unsigned c = s[k];
+        bad |= c >= N;
+        c = min(c, N - 1);
+        const double2 v = V[c];
+        x = __dadd_rn(v.x, __dmul_rn(a.r, __dsub_rn(x, v.x)));
+        y = __dadd_rn(v.y, __dmul_rn(a.r, __dsub_rn(y, v.y)));
+    }
+    const double nan = __longlong_as_double(-1ll);
+    return bad ? make_double2(nan, nan) : make_double2(x, y);
+}
+
+// Spans a block (and so an SM) up to which encode_few is used.  Streams of 40
+// spans, one alone, us by it and by the integer product (and by the whole walk
+// in binary64, as it once was): N = 7 8.5 / 12.5 (8.6), N = 16 6.4 / 8.4 (6.4), N = 256
+// 4.4 / 5.2 (4.4); 192 and 256 spans in one block: N = 9 10.5 / 10.6, 12.5 / 10.6.
+constexpr int kFewSpans = 128;
+
 // The table of points after k symbols from the anchor: entry i's symbols are
 // i's k digits to the base N, the first one most significant.
 __global__ void __launch_bounds__(kThreads) k_pre_table(const double2 *__restrict__ V, int N, double r, int k,
@@ -358,25 +412,33 @@ k_span_encode(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, int64_
 
 // The same for many short streams (a decode step's append): the threads count
 // through all streams' spans, so that a block, its table load and its warps
-// serve as many spans as it has threads, and read their symbols in place.
-// 2,048 streams of 48 symbols: 4.8 us, 8.4 with a block (and its table load) a
-// stream; from half a block's spans on, a block a stream loses little.
-template <bool HALF, typename Sym>
+// serve up to as many spans as it has threads, and read their symbols in
+// place; few spans spread over the SMs (per_block of a block's threads take
+// one).  2,048 streams of 48 symbols: 4.6 us; 6.3 with 256 spans to every block,
+// 10.5 with a block (and its table load) a stream.  From half a block's spans
+// on, many streams lose little by a block a stream; few are shared out all the
+// same (one of 1,000 spans, N = 16: 6.5 us, 8.5 by its own four blocks).
+template <bool HALF, bool FEW, typename Sym>
 __global__ void __launch_bounds__(kThreads)
 k_span_encode_flat(const Sym *__restrict__ sym, int64_t n, int64_t sym_stride, unsigned spans, unsigned total,
-                   fkvd::FastDiv div_spans, double2 *__restrict__ pts, int64_t pt_stride, const EncArgs a,
-                   unsigned *status)
+                   unsigned per_block, fkvd::FastDiv div_spans, double2 *__restrict__ pts, int64_t pt_stride,
+                   const EncArgs a, unsigned *status)
 {
-    __shared__ EncTable<HALF, Sym> tab;
+    __shared__ typename std::conditional<FEW, PlainTable<Sym>, EncTable<HALF, Sym>>::type tab;
     tab.load(a);
     __syncthreads();
-    const unsigned t = blockIdx.x * kThreads + threadIdx.x;
-    if (t >= total)
+    const unsigned t = blockIdx.x * per_block + threadIdx.x;
+    if (threadIdx.x >= per_block || t >= total)
         return;
     const unsigned stream = div_spans.div(t), s = t - stream * spans;
     const int64_t b = static_cast<int64_t>(s) * a.L;
     const int m = static_cast<int>(min(static_cast<int64_t>(a.L), n - b));
-    const double2 p = encode_anchored<HALF>(sym + stream * sym_stride + b, m, tab, a, RatioMul(a.r));
+    const Sym *my = sym + stream * sym_stride + b;
+    double2 p;
+    if constexpr (FEW)
+        p = encode_few(my, m, tab.v, a);
+    else
+        p = encode_anchored<HALF>(my, m, tab, a, RatioMul(a.r));
     if (__double2hiint(p.x) == -1)   // NaN: a symbol >= N
         atomicOr(status, FKV_ST_CORRUPT);
     pts[stream * pt_stride + s] = p;
@@ -809,10 +871,33 @@ __device__ __forceinline__ void ragged_check(const int64_t *__restrict__ so, con
     }
 }
 
+// At most kFewSpans slots of a ragged batch, one a thread of one block.  A call,
+// for inlined it costs the bulk loop registers (1 us of 11 for 1,000 spans).
+template <typename Sym>
+static __device__ __noinline__ void encode_ragged_few(const Sym *__restrict__ sym, const int64_t *__restrict__ so,
+                                                      int64_t n_streams, double2 *__restrict__ pts,
+                                                      const int64_t *__restrict__ po, const EncArgs &a, int64_t g,
+                                                      unsigned *status)
+{
+    const int64_t i = ragged_stream(po, n_streams, g);
+    int64_t n;
+    if (!ragged_ok(so, po, i, a.L, &n))
+        return;
+    const int64_t s = g - __ldg(&po[i]);
+    if (s < 0 || s * a.L >= n)
+        return;
+    const int m = static_cast<int>(min(static_cast<int64_t>(a.L), n - s * a.L));
+    const double2 p = encode_few(sym + __ldg(&so[i]) + s * a.L, m, a.V, a);
+    if (__double2hiint(p.x) == -1)
+        atomicOr(status, FKV_ST_CORRUPT);
+    pts[g] = p;
+}
+
 template <bool HALF, typename Sym>
 __global__ void __launch_bounds__(kThreads)
 k_span_encode_ragged(const Sym *__restrict__ sym, const int64_t *__restrict__ so, int64_t n_streams,
-                     double2 *__restrict__ pts, const int64_t *__restrict__ po, const EncArgs a, unsigned *status)
+                     double2 *__restrict__ pts, const int64_t *__restrict__ po, const __grid_constant__ EncArgs a,
+                     unsigned *status)
 {
     __shared__ EncTable<HALF, Sym> tab;
     const int L = a.L;
@@ -821,6 +906,11 @@ k_span_encode_ragged(const Sym *__restrict__ sym, const int64_t *__restrict__ so
     __syncthreads();
     ragged_check(so, po, n_streams, L, status);
     const int64_t g0 = __ldg(&po[0]), g1 = __ldg(&po[n_streams]);
+    if (!HALF && g1 - g0 <= kFewSpans) {
+        if (blockIdx.x == 0 && threadIdx.x < g1 - g0)
+            encode_ragged_few(sym, so, n_streams, pts, po, a, g0 + threadIdx.x, status);
+        return;
+    }
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
     for (int64_t g = g0 + static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; g < g1; g += stride) {
         const int64_t i = ragged_stream(po, n_streams, g);
@@ -1358,13 +1448,19 @@ cudaError_t span_encode_t(const fkv_ctx *c, const Sym *sym, int64_t n_streams, i
         return cudaSuccess;
     if (blocks > 0x7FFFFFFF)
         return cudaErrorInvalidConfiguration;
-    // streams of at most half a block's spans share blocks
-    if (spans <= kThreads / 2 && n_streams * spans <= 0x7FFFFFFF) {
-        const auto flat = c->r == 0.5 ? k_span_encode_flat<true, Sym> : k_span_encode_flat<false, Sym>;
+    // streams of at most half a block's spans share blocks, and so do all while
+    // they are few
+    if (n_streams * spans <= (spans <= kThreads / 2 ? 0x7FFFFFFF : kFewSpans * c->sms)) {
         const unsigned total = static_cast<unsigned>(n_streams * spans);
-        flat<<<(total + kThreads - 1) / kThreads, kThreads, 0, st>>>(
-            sym, n, sym_stride, static_cast<unsigned>(spans), total, fkvd::FastDiv::make(static_cast<unsigned>(spans)),
-            reinterpret_cast<double2 *>(pts), pt_stride, enc_args(c), c->d_status);
+        // an SM's share of the spans in whole warps, a block's threads at most
+        const unsigned share = (total / c->sms + 32) & ~31u, per = share < kThreads ? share : kThreads;
+        const auto flat = c->r == 0.5 ? k_span_encode_flat<true, false, Sym>
+                          : per <= kFewSpans ? k_span_encode_flat<false, true, Sym>
+                                             : k_span_encode_flat<false, false, Sym>;
+        flat<<<(total + per - 1) / per, kThreads, 0, st>>>(
+            sym, n, sym_stride, static_cast<unsigned>(spans), total, per,
+            fkvd::FastDiv::make(static_cast<unsigned>(spans)), reinterpret_cast<double2 *>(pts), pt_stride,
+            enc_args(c), c->d_status);
         return cudaGetLastError();
     }
     const auto kern = c->r == 0.5 ? k_span_encode<true, Sym> : k_span_encode<false, Sym>;

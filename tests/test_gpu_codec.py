@@ -255,3 +255,27 @@ def test_many_short_streams_encode_bit_exact(fkv, oracle_mod, N, spans):
     got = pts.cpu().numpy()
     assert np.array_equal(got[:, :spans].view(np.uint64), want.view(np.uint64))
     assert np.all(got[:, spans:] == 7.0) and ctx.sync_status() == 0
+
+
+@pytest.mark.parametrize("N", [4, 5, 16, 256, 1024])
+@pytest.mark.parametrize("ns,spans", [(1, 128), (1, 129), (64, 8), (4, 1300), (1, 19456), (1, 19457), (152, 129)])
+def test_few_spans_encode_bit_exact(fkv, oracle_mod, N, ns, spans):
+    """Few spans spread over the SMs and walked in binary64, around the numbers
+    where a block's share, or the stream's own blocks, take over; the same as a
+    ragged batch, whose line is 128 slots; a symbol that is none."""
+    ctx = _ctx(fkv, N)
+    n = spans * ctx.L - (ctx.L - 1)
+    sym = np.random.default_rng(spans + N).integers(0, N, size=(ns, n)).astype(np.uint8 if N <= 256 else np.uint16)
+    d = torch.from_numpy(sym if N <= 256 else sym.view(np.int16)).cuda()
+    want = _oracle_points(oracle_mod, sym, N, ctx.r, ctx.L)
+    assert np.array_equal(ctx.span_encode(d).cpu().numpy().view(np.uint64), want.view(np.uint64))
+    so, po = ctx.ragged_offsets(np.full(ns, n))
+    got = ctx.span_encode_ragged(d.reshape(-1), so, po)
+    assert np.array_equal(got.cpu().numpy().view(np.uint64).reshape(want.shape), want.view(np.uint64))
+    assert ctx.sync_status() == 0
+    if N != 256:
+        d[0, n - 1] = N
+        p = ctx.span_encode(d)
+        assert ctx.sync_status() == -5 and torch.isnan(p[0, -1]).all() and not torch.isnan(p[0, :-1]).any()
+        p = ctx.span_encode_ragged(d.reshape(-1), so, po).reshape(ns, spans, 2)
+        assert ctx.sync_status() == -5 and torch.isnan(p[0, -1]).all() and not torch.isnan(p[0, :-1]).any()
