@@ -343,9 +343,11 @@ __device__ __forceinline__ void load_add_chunk(const uint8_t *ahi, const uint8_t
 // row (f is passed as uniform, UF, when every row's is the same); cbk points
 // at the K block's first element of codeword 0 of the stage codebook.  Same
 // arithmetic as load_add_chunk and store_chunk: hi + lo exact, one rounding
-// in the multiply-add.  Software-pipelined over batches of 8 rows: the next
-// batch's codeword loads are in flight while one batch is updated.
-template <bool UF, int D = 128>
+// in the multiply-add.  Software-pipelined over batches of 8 rows: the loads of
+// the next AHEAD batches' codewords are in flight while one batch is updated
+// (two are what the pair kernels' registers hold; k_rvq128, whose epilogue
+// needs more, spills with two and took up to 6 % longer, with one stage too).
+template <bool UF, int D = 128, int AHEAD = 2>
 __device__ __forceinline__ void update_rows_t(uint8_t *ahi, uint8_t *alo, int quad, const float *cbk, int bidx,
                                               float f)
 {
@@ -354,18 +356,19 @@ __device__ __forceinline__ void update_rows_t(uint8_t *ahi, uint8_t *alo, int qu
     const uint32_t cw = static_cast<uint32_t>(li >> 1), wo = static_cast<uint32_t>((li & 1) << 3);
     const float4 *cl = reinterpret_cast<const float4 *>(cbk) + li;
     uint8_t *qhi = ahi + quad * 32 * 128, *qlo = alo + quad * 32 * 128;
-    float4 cv[3][4];
+    float4 cv[AHEAD + 1][4];
     auto fetch = [&](int b) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            cv[b % 3][j] = __ldg(cl + __shfl_sync(0xFFFFFFFFu, bidx, 8 * b + 2 * j + hs) * (D / 4));
+            cv[b % (AHEAD + 1)][j] = __ldg(cl + __shfl_sync(0xFFFFFFFFu, bidx, 8 * b + 2 * j + hs) * (D / 4));
     };
-    fetch(0);
-    fetch(1);
+#pragma unroll
+    for (int b = 0; b < AHEAD; ++b)
+        fetch(b);
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-        if (b < 2)
-            fetch(b + 2);
+        if (b + AHEAD < 4)
+            fetch(b + AHEAD);
         uint2 hv[4], lv[4];
         uint32_t off[4];
 #pragma unroll
@@ -377,7 +380,7 @@ __device__ __forceinline__ void update_rows_t(uint8_t *ahi, uint8_t *alo, int qu
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float4 c = cv[b % 3][j];
+            const float4 c = cv[b % (AHEAD + 1)][j];
             const float fj = UF ? f : __shfl_sync(0xFFFFFFFFu, f, 8 * b + 2 * j + hs);
             float v0, v1, v2, v3;
             join_half2(hv[j].x, lv[j].x, v0, v1);
@@ -1683,9 +1686,9 @@ k_rvq128(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int n_pairs)
                     const float4 *gc = reinterpret_cast<const float4 *>(cbs + bidx * D) + 16;
                     if (e_next == e) {
                         if (__all_sync(0xFFFFFFFFu, er == 0))
-                            update_rows_t<true>(ahi, alo, quad, cbs + 64, bidx, f);
+                            update_rows_t<true, 128, 1>(ahi, alo, quad, cbs + 64, bidx, f);
                         else
-                            update_rows_t<false>(ahi, alo, quad, cbs + 64, bidx, f);
+                            update_rows_t<false, 128, 1>(ahi, alo, quad, cbs + 64, bidx, f);
                     } else {
                         float mx = 0.0f;
 #pragma unroll 4
@@ -1860,9 +1863,9 @@ k_rvq128(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int n_pairs)
                     const float4 *gc = reinterpret_cast<const float4 *>(cbs + bidx * D);
                     if (e_next == e) {
                         if (__all_sync(0xFFFFFFFFu, er == 0))
-                            update_rows_t<true>(ahi, alo, quad, cbs, bidx, f);
+                            update_rows_t<true, 128, 1>(ahi, alo, quad, cbs, bidx, f);
                         else
-                            update_rows_t<false>(ahi, alo, quad, cbs, bidx, f);
+                            update_rows_t<false, 128, 1>(ahi, alo, quad, cbs, bidx, f);
                     } else {
                         float mx = 0.0f;
 #pragma unroll 4
