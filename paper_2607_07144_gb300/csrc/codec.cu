@@ -648,22 +648,20 @@ struct SuffixQuery {
 };
 
 // Whether the last symbols of the span stored as p are the query: step j of
-// the walk recovers the query's symbol len - 1 - j.  A call: few points are
-// candidates, and inlined the walks' registers halve the scan's warps.
-static __device__ __noinline__ bool ends_in(const fkvdec::Tables &t, double2 p, const SuffixQuery &qy)
+// the walk recovers the query's symbol len - 1 - j.  One cell test is inlined
+// (64 to 128 registers); with all three behind a call, the scan's own registers
+// spilled, and next to the tables of N = 1024 the spills missed L1: 10 M points
+// 56 us, 72 by the call.
+template <fkvdec::Cell CELL>
+__device__ __forceinline__ bool ends_in(const fkvdec::Tables &t, double2 p, const SuffixQuery &qy)
 {
     long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
     bool eq = true;
-    auto same = [&](int j, int c) { eq = eq && c == qy.sym[qy.len - 1 - j]; };
-    if (t.N > 8)
-        fkvdec::walk<fkvdec::kSectors>(t, X, Y, qy.len, same);
-    else if (t.N == 4)
-        fkvdec::walk<fkvdec::kAxes>(t, X, Y, qy.len, same);
-    else
-        fkvdec::walk<fkvdec::kScores>(t, X, Y, qy.len, same);
+    fkvdec::walk<CELL, true>(t, X, Y, qy.len, [&](int j, int c) { eq = eq && c == qy.sym[qy.len - 1 - j]; });
     return eq;
 }
 
+template <fkvdec::Cell CELL>
 __global__ void __launch_bounds__(kThreads)
 k_suffix_search(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, int64_t pt_stride, int64_t spans,
                 const __grid_constant__ SuffixQuery qy, double thr, double thr2, const double2 *__restrict__ V, double r,
@@ -729,7 +727,7 @@ k_suffix_search(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, i
                 const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
                 if (d2 <= thr2) {
                     atomicAdd(&counts[1], 1ull);
-                    if (ends_in(t, p, qy)) {
+                    if (ends_in<CELL>(t, p, qy)) {
                         const unsigned long long slot = atomicAdd(&counts[0], 1ull);
                         if (static_cast<long long>(slot) < cap) {
                             out[2 * slot] = su[i];
@@ -1591,14 +1589,16 @@ cudaError_t launch_suffix_search(const fkv_ctx *c, const double *pts, int64_t n_
     const double thr2 = t * t;
     const int smem = tables_bytes(c->N, c->L);
     unsigned grid = 0;
-    e = decode_grid(c, reinterpret_cast<const void *>(k_suffix_search), smem, cdiv(n_streams * spans, kThreads),
-                    &grid);
+    const auto kern = c->N > 8    ? k_suffix_search<fkvdec::kSectors>
+                      : c->N == 4 ? k_suffix_search<fkvdec::kAxes>
+                                  : k_suffix_search<fkvdec::kScores>;
+    e = decode_grid(c, reinterpret_cast<const void *>(kern), smem, cdiv(n_streams * spans, kThreads), &grid);
     if (e != cudaSuccess)
         return e;
-    k_suffix_search<<<grid, kThreads, smem, st>>>(reinterpret_cast<const double2 *>(pts), n_streams, n, pt_stride,
-                                                  spans, qy, t, thr2, c->d_V, c->r, c->d_dec, c->d_T, c->N, c->L,
-                                                  reinterpret_cast<long long *>(out), cap,
-                                                  reinterpret_cast<unsigned long long *>(counts));
+    kern<<<grid, kThreads, smem, st>>>(reinterpret_cast<const double2 *>(pts), n_streams, n, pt_stride, spans, qy, t,
+                                       thr2, c->d_V, c->r, c->d_dec, c->d_T, c->N, c->L,
+                                       reinterpret_cast<long long *>(out), cap,
+                                       reinterpret_cast<unsigned long long *>(counts));
     return cudaGetLastError();
 }
 
