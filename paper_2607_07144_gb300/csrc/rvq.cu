@@ -2552,25 +2552,29 @@ cudaError_t launch_rvq64(const fkv_ctx *c, const CUtensorMap &tmap, const RvqArg
 // pairs a round, two slots an SM; k_rvq64_pair three units a cluster, so its
 // round is half as long again, and k_rvq128_pair two, so its rounds are the
 // same but only within groups (k_rvq128 pairs the tiles of all groups, an odd
-// group's last one too).  Measured, pair / single SM (16-bit input):
-//   64 dimensions, 1 stage: 0.74 .. 1.01 but for 2 units a cluster (1.11 for
-//   144 groups of 1 tile); more stages: 1.01 .. 1.30 up to 2 units (few units
-//   gain nothing and wait for their partner), 0.75 .. 0.96 at 3 (two rounds
-//   against one), 1.10 .. 1.22 at 4, 0.85 .. 1.08 from 5 to 12, 0.91 .. 0.98
-//   beyond (0.71 .. 0.77 on 4,464 units); a tile a group 1.08 .. 1.56; float32
-//   input at 1 unit 0.92 .. 1.05, and 19.3 / 22.9 us for the two launches of a
-//   layer of 12 heads and 988 positions (rows come whole lines at a time).
-//   1024 codewords: 0.67 .. 1.00 but for 2 units a cluster (up to 1.13).
-//   128 dimensions: 1.05 .. 1.33 when the pairs need a round more; else 0.71 ..
-//   0.97 from 2 stages on; 1 stage 0.80 .. 0.94 at an odd number of units a
-//   cluster, 0.99 .. 1.16 at an even one.
+// group's last one too).  Measured on 2,100 shapes, pair / single SM (launches
+// one after another take whole steps of 2 us, so that calls of 8 to 30 us
+// scatter by a step):
+//   64 dimensions, 1 stage: 0.65 .. 1.01 but for 2 units a cluster (0.84 ..
+//   1.25); more stages: up to 2 units 0.87 .. 1.40 (few units gain nothing and
+//   wait for their partner) but for float32 input at 1 unit, 0.84 .. 1.06
+//   (load_rows64 takes its rows whole lines at a time; up to 1.15 where the
+//   second of two tiles is half empty); 0.72 .. 0.96 at 3 units (two rounds
+//   against one), 0.85 .. 1.27 at 4, 0.80 .. 1.16 from 5 to 12, 0.81 .. 1.00
+//   beyond.  A tile a group leaves the unit's other tile empty: 1.00 .. 1.57.
+//   1024 codewords: 0.63 .. 1.00 but for 2 units a cluster (0.86 .. 1.30).
+//   128 dimensions: 0.90 .. 1.66 when the pairs need a round more; else 0.67 ..
+//   1.11 from 2 stages on (above 1.01 at 2 units of one tile); 1 stage 0.72 ..
+//   1.00 at an odd number of units a cluster, 0.84 .. 1.16 at an even one.
 bool pair_tiles(const fkv_ctx *c, int64_t tiles, int64_t groups, const RvqArgs &a)
 {
     const int64_t units = groups * ((tiles + 1) / 2), clusters = c->sms / 2;
     const int64_t per = (units + clusters - 1) / clusters;
     if (c->D == 64) {
-        if (c->KC == 1024 || a.S == 1)
+        if (c->KC == 1024)
             return per != 2;
+        if (a.S == 1)
+            return tiles > 1 && per != 2;
         return tiles > 1 && (per == 3 || per > 12 || (per == 1 && a.dtype == FKV_F32));
     }
     const int64_t pairs = (groups * tiles + 1) / 2;
