@@ -428,24 +428,26 @@ int fkv_create(int N, double r, int span_len, const fkv_codebooks *cb, fkv_ctx *
         dec.bound[i] = make_int2(static_cast<int>(lrint(ldexp(cos(th), 30))), static_cast<int>(-lrint(ldexp(sin(th), 30))));
     }
     dec.sect_sh = static_cast<int>(floor(65536.0 * log2(1.0 / r)));
-    // one allocation: the host-made tables in one copy, then the status word
-    // and the encoders' point table, filled on the device
+    // the host-made tables in one allocation and one copy, the status word behind
+    // them; the encoders' point table, filled on the device, by itself: of its
+    // 1 MB at most two fit a 2 MB page, whose mapping takes 80 us, and with the
+    // others behind it none would share one
     int pre_count = 0;
     ctx->pre_k = pre_table_symbols(N, span_len, &pre_count);
     auto up16 = [](size_t n) { return (n + 15) & ~size_t(15); };
     const size_t o_T = up16(N * sizeof(double2)), o_dec = o_T + up16(T.size() * sizeof(longlong2)),
-                 o_status = o_dec + up16(sizeof(dec)), o_pre = o_status + 16;
-    std::vector<uint8_t> tab(o_pre, 0);
+                 o_status = o_dec + up16(sizeof(dec));
+    std::vector<uint8_t> tab(o_status + 16, 0);
     memcpy(tab.data(), V.data(), N * sizeof(double2));
     memcpy(tab.data() + o_T, T.data(), T.size() * sizeof(longlong2));
     memcpy(tab.data() + o_dec, &dec, sizeof(dec));
     uint8_t *base = nullptr;
-    CK(cudaMalloc(&base, o_pre + pre_count * sizeof(double2)), "context alloc");
+    CK(cudaMalloc(&base, tab.size()), "context alloc");
     ctx->d_V = reinterpret_cast<double2 *>(base);
+    CK(cudaMalloc(&ctx->d_pre, pre_count * sizeof(double2)), "context alloc");
     ctx->d_T = reinterpret_cast<longlong2 *>(base + o_T);
     ctx->d_dec = reinterpret_cast<fkv_decconst *>(base + o_dec);
     ctx->d_status = reinterpret_cast<unsigned *>(base + o_status);
-    ctx->d_pre = reinterpret_cast<double2 *>(base + o_pre);
     CK(cudaMemcpy(base, tab.data(), tab.size(), cudaMemcpyHostToDevice), "context copy");
     CK(launch_pre_table(ctx, nullptr), "point table launch");
 
@@ -486,7 +488,8 @@ int fkv_destroy(fkv_ctx *ctx)
     if (!ctx)
         return FKV_OK;
     cudaDeviceSynchronize();
-    cudaFree(ctx->d_V);            // and every table of fkv_create behind it
+    cudaFree(ctx->d_V);            // and the tables of fkv_create behind it
+    cudaFree(ctx->d_pre);
     cudaFree(ctx->d_scratch);
     cudaFree(ctx->d_read_order);
     destroy_cbset(ctx->cb[0]);

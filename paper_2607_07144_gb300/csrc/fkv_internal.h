@@ -65,7 +65,7 @@ struct fkv_ctx {
     // kernels this context has launched (calls on one context are serialised)
     mutable fkv_kernel_use uses[32];
     mutable int n_uses = 0;
-    double2 *d_V = nullptr;        // [N] vertices; first of one allocation with d_T, d_dec, d_status and d_pre
+    double2 *d_V = nullptr;        // [N] vertices; first of one allocation with d_T, d_dec and d_status
     fkv_decconst *d_dec = nullptr; // decoder constants (device copy)
     longlong2 *d_T = nullptr;      // [L][N] (1-r) r^j V(c) in Q1.62
     double2 *d_pre = nullptr;      // [N^pre_k] points after pre_k symbols from the anchor (codec.cu)
