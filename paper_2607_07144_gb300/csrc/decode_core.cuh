@@ -246,13 +246,14 @@ template <bool ROLLED, int NC, class Classify, class Emit>
 __device__ __forceinline__ void walk_by(const Tables &t, long long &X, long long &Y, int steps, Classify classify,
                                         Emit emit)
 {
-    const int n = NC > 0 ? NC : t.N;
+    const longlong2 *T = t.T;
     auto step = [&](int j) {
         const int c = classify(X, Y);
         emit(j, c);
-        const longlong2 w = t.T[j * n + c];
+        const longlong2 w = T[c];
         X = static_cast<long long>(static_cast<unsigned long long>(X) - static_cast<unsigned long long>(w.x));
         Y = static_cast<long long>(static_cast<unsigned long long>(Y) - static_cast<unsigned long long>(w.y));
+        T += NC > 0 ? NC : t.N;
     };
     if constexpr (ROLLED) {
 #pragma unroll 1
