@@ -1180,10 +1180,13 @@ static __device__ __noinline__ double div_fp64(double a, double b) { return __dd
 
 // a / r rounded to nearest even, as __ddiv_rn(a, r), on the integer pipe: the
 // mantissa of a (at the top of 64 bits) times inv is the quotient's upper 64
-// bits, low by less than one unit, and rounds at its 53rd bit.  A quotient of
-// two 53-bit numbers is no midpoint (r not a power of two), so the rounding is
-// settled unless the dropped bits sit one unit below one half; those (1 in
-// 1024) and far-out exponents take the IEEE division.
+// bits, low by less than two units (inv is rounded down, and the product's
+// upper word again), and rounds at its 53rd bit.  A quotient of two 53-bit
+// numbers is no midpoint (r not a power of two).  So with the dropped bits of h
+// at one half or above the quotient rounds up, at one half less two units or
+// below it rounds down, and one unit below one half it may be on either side:
+// those (1 in 1024), far-out exponents and r a power of two take the IEEE
+// division.
 __device__ __forceinline__ double div_ratio(const LossyWalk &q, double a)
 {
     const unsigned hi = static_cast<unsigned>(__double2hiint(a)), lo = static_cast<unsigned>(__double2loint(a));

@@ -332,9 +332,9 @@ __device__ __forceinline__ void walk_sectors(const Tables &t, long long &X, long
 // the anchor (|Q_0| <= lim), the symbols then being those of the general walk.
 // The decoders and random reads are compiled for each cell test.  With all of
 // them in one kernel, chosen at each symbol, 134 M symbols took 0.402 ms for
-// N = 3 (0.326 by itself), 0.224 for N = 4 (0.170), 0.672 for N = 8 (0.549),
-// 0.416 for N = 256 (0.413); 4.2 M random reads 0.648 / 0.297 / 0.459 / 0.111
-// (0.432 / 0.218 / 0.402 / 0.110).
+// N = 3 (0.318 now), 0.224 for N = 4 (0.170), 0.672 for N = 8 (0.517), 0.416 for
+// N = 256 (0.412); 4.2 M random reads 0.648 / 0.297 / 0.459 / 0.111 (0.418 /
+// 0.219 / 0.377 / 0.100).
 template <Cell CELL, class Start>
 __device__ __forceinline__ bool decode_point(const Tables &t, double2 p, int m, long long lim, Start start)
 {

@@ -882,9 +882,9 @@ k_rvq64(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int pairs_per
 // k_rvq64 has in its stage buffer, since a vector's indices must not depend on
 // the shape of the call that archives it.
 //
-// GPT-2-shaped cache, 1,138,176 vectors of K (4 stages) and of V (2): 486 us
-// against 633 for k_rvq64, and with 1024-codeword codebooks 1,013 against
-// 1,192 (1,960 cycles a block, of which its 13 MMAs take 1,664).  At four stages a
+// GPT-2-shaped cache, 1,138,176 vectors of K (4 stages) and of V (2): 488 us
+// against 637 for k_rvq64, and with 1024-codeword codebooks 1,036 against
+// 1,205 (1,960 cycles a block, of which its 13 MMAs take 1,664).  At four stages a
 // slot's round is 1,560 cycles of input, 3,200 waiting for its MMAs, 1,270 of
 // argmin and 2/3 x 2,600 of update: instruction issue and L2 latency of the
 // epilogue, not the tensor pipe, still bound it.  On the way: 689 us with
@@ -940,7 +940,9 @@ __device__ __forceinline__ uint32_t map_cta(uint32_t addr, uint32_t rank)
 // shared or tensor memory, made visible to the tensor core by the proxy and
 // tcgen05 fences before it; only the lo stamp, a word in the leader, needs the
 // cluster-scope release, whose memory barrier costs every arrival some 500
-// cycles (16 % of all stalls).
+// cycles (16 % of all stalls).  The PTX model orders the rest across the CTAs
+// only at that scope; without it, it is the hardware that is relied on, as by
+// any remote arrival of default scope.
 template <bool STAMP = false>
 __device__ __forceinline__ void arrive_cluster(uint32_t bar)
 {
@@ -1943,8 +1945,8 @@ k_rvq128(const __grid_constant__ CUtensorMap tmap, const RvqArgs a, int n_pairs)
 // for each.  The input rows are taken whole lines at a time, eight loads in
 // flight, the first K block by the slot's warps and the second by the helpers.
 //
-// Llama-shaped cache, 4.19 M vectors of K (4 stages) and of V (2): 3.65 ms
-// against 3.98 for k_rvq128; 64 groups of 7 tiles in float32, 56 us against
+// Llama-shaped cache, 4.19 M vectors of K (4 stages) and of V (2): 3.69 ms
+// against 4.04 for k_rvq128; 64 groups of 7 tiles in float32, 56 us against
 // 71.  A slot's stage is 6,300 cycles waiting for its MMAs (its own take
 // 3,300, the other slot's come between), 1,000 of argmin, 2,530 of update and
 // 1,900 of input; reading all 16 codeword rows of an update ahead spills and
