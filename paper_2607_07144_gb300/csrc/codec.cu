@@ -657,7 +657,7 @@ __device__ __forceinline__ bool ends_in(const fkvdec::Tables &t, double2 p, cons
 {
     long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
     bool eq = true;
-    fkvdec::walk<CELL, true>(t, X, Y, qy.len, [&](int j, int c) { eq = eq && c == qy.sym[qy.len - 1 - j]; });
+    fkvdec::walk<CELL, 1>(t, X, Y, qy.len, [&](int j, int c) { eq = eq && c == qy.sym[qy.len - 1 - j]; });
     return eq;
 }
 
@@ -777,7 +777,7 @@ k_read(const double2 *__restrict__ pts, int64_t n_streams, int64_t n, int64_t pt
             const double2 p = pts[st * pt_stride + u];
             long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
             int sym = 0;
-            fkvdec::walk<CELL, true>(t, X, Y, m - o, [&](int j, int c) { sym = c; });
+            fkvdec::walk_read<CELL>(t, X, Y, m - o, [&](int j, int c) { sym = c; });
             out[q] = static_cast<Sym>(sym);
         }
         q = qn;
@@ -1023,7 +1023,7 @@ k_read_ragged(const double2 *__restrict__ pts, const int64_t *__restrict__ po, c
         const double2 p = pts[__ldg(&po[st]) + u];
         long long X = fkvdec::to_q62(p.x), Y = fkvdec::to_q62(p.y);
         int c = 0;
-        fkvdec::walk<CELL, true>(t, X, Y, m - o, [&](int, int cc) { c = cc; });
+        fkvdec::walk_read<CELL>(t, X, Y, m - o, [&](int, int cc) { c = cc; });
         out[q] = static_cast<Sym>(c);
     }
 }

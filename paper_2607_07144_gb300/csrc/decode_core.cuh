@@ -238,11 +238,12 @@ __device__ __forceinline__ long long to_q62(double v)
 // Decode `steps` symbols backward from Q (the span's stored point in Q1.62):
 // step j = 0 .. steps-1 emits the symbol at offset m-1-j of the span.
 // `emit(j, c)` receives each symbol.  Any Q, of any size: random reads,
-// retrieval, and spans that are no code point.  ROLLED for random reads, whose
-// lanes take different numbers of steps: in an unrolled loop they part ways in
-// the remainder.  4.2 M reads of N = 4, spans of 8: 62 us rolled, 88 unrolled;
-// of 44: 217 and 214.  NC: the alphabet's size where it is known, 0 else.
-template <bool ROLLED, int NC, class Classify, class Emit>
+// retrieval, and spans that are no code point.  UNROLL steps of the loop (0: the
+// compiler's choice): random reads of N <= 8 take few, since their lanes walk
+// different numbers of steps and part ways in the remainder of an unrolled loop.
+// 4.2 M reads of N = 4, spans of 8: 64 us by two steps, 88 as the compiler
+// unrolls it; of 44: 209 and 214.  NC: the alphabet's size where it is known, 0 else.
+template <int UNROLL, int NC, class Classify, class Emit>
 __device__ __forceinline__ void walk_by(const Tables &t, long long &X, long long &Y, int steps, Classify classify,
                                         Emit emit)
 {
@@ -255,8 +256,8 @@ __device__ __forceinline__ void walk_by(const Tables &t, long long &X, long long
         Y = static_cast<long long>(static_cast<unsigned long long>(Y) - static_cast<unsigned long long>(w.y));
         T += NC > 0 ? NC : t.N;
     };
-    if constexpr (ROLLED) {
-#pragma unroll 1
+    if constexpr (UNROLL > 0) {
+#pragma unroll UNROLL
         for (int j = 0; j < steps; ++j)
             step(j);
     } else {
@@ -268,16 +269,16 @@ __device__ __forceinline__ void walk_by(const Tables &t, long long &X, long long
 // The cell test of an alphabet: sectors (N > 8), the axes (N = 4), scores.
 enum Cell { kSectors, kAxes, kScores };
 
-template <Cell CELL, bool ROLLED = false, class Emit>
+template <Cell CELL, int UNROLL = 0, class Emit>
 __device__ __forceinline__ void walk(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
 {
     if (CELL == kSectors) {
-        walk_by<ROLLED, 0>(t, X, Y, steps, [&](long long x, long long y) { return classify_angle(t, x, y); }, emit);
+        walk_by<UNROLL, 0>(t, X, Y, steps, [&](long long x, long long y) { return classify_angle(t, x, y); }, emit);
     } else if (CELL == kAxes) {
-        walk_by<ROLLED, 4>(t, X, Y, steps, [](long long x, long long y) { return classify_axes(x, y); }, emit);
+        walk_by<UNROLL, 4>(t, X, Y, steps, [](long long x, long long y) { return classify_axes(x, y); }, emit);
     } else {
         auto scores = [&](auto n) {
-            walk_by<ROLLED, n.value>(
+            walk_by<UNROLL, n.value>(
                 t, X, Y, steps, [&](long long x, long long y) { return classify_scores<n.value>(t, x, y); }, emit);
         };
         switch (t.N) {
@@ -288,6 +289,16 @@ __device__ __forceinline__ void walk(const Tables &t, long long &X, long long &Y
         default: scores(std::integral_constant<int, 8>()); break;
         }
     }
+}
+
+// The walk of a random read, by the steps that its cell test's loop unrolls best
+// (sectors: 1 M reads of N = 64 29 us, 31 rolled; of N = 1024 in a ragged batch of
+// 20,000 streams 39.4, 51.3 rolled; scores: 4.2 M reads of N = 8, spans of 2, 66 us
+// rolled, 80 by two steps).
+template <Cell CELL, class Emit>
+__device__ __forceinline__ void walk_read(const Tables &t, long long &X, long long &Y, int steps, Emit emit)
+{
+    walk<CELL, CELL == kSectors ? 0 : CELL == kAxes ? 2 : 1>(t, X, Y, steps, emit);
 }
 
 template <class Emit>
