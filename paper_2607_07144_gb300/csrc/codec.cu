@@ -874,7 +874,7 @@ __device__ __forceinline__ void ragged_check(const int64_t *__restrict__ so, con
 template <typename Sym>
 static __device__ __noinline__ void encode_ragged_few(const Sym *__restrict__ sym, const int64_t *__restrict__ so,
                                                       int64_t n_streams, double2 *__restrict__ pts,
-                                                      const int64_t *__restrict__ po, const EncArgs &a, int64_t g,
+                                                      const int64_t *__restrict__ po, const EncArgs a, int64_t g,
                                                       unsigned *status)
 {
     const int64_t i = ragged_stream(po, n_streams, g);
@@ -894,8 +894,7 @@ static __device__ __noinline__ void encode_ragged_few(const Sym *__restrict__ sy
 template <bool HALF, typename Sym>
 __global__ void __launch_bounds__(kThreads)
 k_span_encode_ragged(const Sym *__restrict__ sym, const int64_t *__restrict__ so, int64_t n_streams,
-                     double2 *__restrict__ pts, const int64_t *__restrict__ po, const __grid_constant__ EncArgs a,
-                     unsigned *status)
+                     double2 *__restrict__ pts, const int64_t *__restrict__ po, const EncArgs a, unsigned *status)
 {
     __shared__ EncTable<HALF, Sym> tab;
     const int L = a.L;
